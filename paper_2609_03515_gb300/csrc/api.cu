@@ -99,6 +99,7 @@ PagedView view_of(const ikv_shape *s, const ikv_cache *c) {
     v.max_pages = c->max_pages;
     v.kv_heads = s->kv_heads;
     v.head_dim = s->head_dim;
+    v.page_shift = (c->page_size & (c->page_size - 1)) == 0 ? __builtin_ctz((unsigned)c->page_size) : -1;
     return v;
 }
 
@@ -197,27 +198,42 @@ T *at(void *ws, size_t off) {
     return reinterpret_cast<T *>(reinterpret_cast<unsigned char *>(ws) + off);
 }
 
-// split-K partition for lengths up to max_len: enough CTAs to fill the GPU
-// (ctas_per_sm x SMs), splits a multiple of `granule` tokens and at most
-// `max_split` tokens long, at most kMaxSplits per (sequence, layer, kv head)
-void choose_splits(const ikv_shape *s, int n_layers, int32_t max_len, int granule, int max_split,
-                   int32_t *split_tokens, int32_t *n_splits, int sms) {
+// split-K partition of the kernels of attend.cu for lengths up to max_len: at most kMaxSplits
+// splits per (sequence, layer, kv head) unit.
+void choose_splits(const ikv_shape *s, int n_layers, int32_t max_len, int32_t *split_tokens, int32_t *n_splits,
+                   int sms) {
     const int64_t units = (int64_t)s->batch * n_layers * s->kv_heads;
-    const int64_t want = (int64_t)sms * 4;
-    int64_t splits = (want + units - 1) / units;
-    const int64_t by_len = (max_len + kMinSplitTokens - 1) / kMinSplitTokens;
-    if (splits > by_len) splits = by_len;
-    const int64_t need = (max_len + max_split - 1) / max_split;
-    if (splits < need) splits = need;
-    if (splits > kMaxSplits) splits = kMaxSplits;
-    if (splits < 1) splits = 1;
-    int64_t st = (max_len + splits - 1) / splits;
-    st = (st + granule - 1) / granule * granule;
-    if (st < granule) st = granule;
+    int64_t best = 1;
+    if (s->dtype == IKV_F32) {
+        // The count that finishes first when the CTAs run in whole waves over the resident
+        // slots: waves x tokens of a split, plus what each CTA costs besides (as tokens of
+        // its stream) and what a merge does.  Measured, us a step for 1 / 2 / 3 / 4 / 5 / 7 /
+        // 9 / 12 splits: 128 units of 2049 tokens (d = 128, G = 4) 108 / 83 / 85 / 80 / 83 /
+        // 77 / 82 / 83 (7 taken: 2.95 waves), 256 units 129 / 135 / 135 / 135 / - / 135 (1 taken).
+        const int64_t slots = (int64_t)sms * kF32CtasPerSm;
+        int64_t best_cost = INT64_MAX;
+        for (int64_t n = 1; n <= kMaxSplits && (n == 1 || (n - 1) * kTileTokens < max_len); ++n) {
+            const int64_t st = ((max_len + n - 1) / n + kTileTokens - 1) / kTileTokens * kTileTokens;
+            const int64_t cost = (units * n + slots - 1) / slots * slots * st + units * n * kSplitCtaTokens +
+                                 (n > 1 ? slots * kSplitMergeTokens : 0);
+            if (cost < best_cost) {
+                best_cost = cost;
+                best = n;
+            }
+        }
+    } else {
+        const int64_t want = (int64_t)sms * 4;
+        best = (want + units - 1) / units;
+        const int64_t by_len = (max_len + kMinSplitTokens - 1) / kMinSplitTokens;
+        if (best > by_len) best = by_len;
+        if (best > kMaxSplits) best = kMaxSplits;
+        if (best < 1) best = 1;
+    }
+    int64_t st = ((max_len + best - 1) / best + kTileTokens - 1) / kTileTokens * kTileTokens;
+    if (st < kTileTokens) st = kTileTokens;
     *split_tokens = (int32_t)st;
-    int64_t ns = (max_len + st - 1) / st;
-    if (ns < 1) ns = 1;
-    *n_splits = (int32_t)ns;
+    const int64_t ns = (max_len + st - 1) / st;
+    *n_splits = (int32_t)(ns < 1 ? 1 : ns);
 }
 
 // attention (+ combine) over layers [layer0, layer0 + n_layers)
@@ -266,7 +282,7 @@ ikv_status run_attend(const ikv_shape *s, const ikv_cache *c, int32_t layer0, in
         // one chunk per unit: the kernel can hand the score pass normalised group sums
         a.gsum = gsum && logits && nc == 1 && use_tc(s, c, s->layers, max_len) ? 1 : 0;
     } else
-        choose_splits(s, n_layers, max_len, kTileTokens, 1 << 30, &a.split_tokens, &a.n_splits, sm_count());
+        choose_splits(s, n_layers, max_len, &a.split_tokens, &a.n_splits, sm_count());
     a.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)s->head_dim));
     a.logits = logits ? at<float>(ws, w.logits) : nullptr;
     if (gsum) *gsum = false;
@@ -293,18 +309,25 @@ ikv_status run_attend(const ikv_shape *s, const ikv_cache *c, int32_t layer0, in
     } else if (append) {
         IKV_TRY_CUDA(launch_append_rows(*append, st), "append rows launch");
     }
+    // the tensor-core and fp32 kernels merge their splits themselves: the last CTA of each
+    // unit writes out and lse2
+    const bool merges = tc || s->dtype == IKV_F32;
+    int32_t *arr = at<int32_t>(ws, w.arrivals);
+    if (merges && a.n_splits > 1 && !counters_zeroed)
+        IKV_TRY_CUDA(cudaMemsetAsync(arr, 0, sizeof(int32_t) * (size_t)s->batch * n_layers * s->kv_heads, st),
+                     "cudaMemsetAsync");
+    a.out = out;
+    a.lse2 = at<float>(ws, w.lse2);
+    a.arrivals = arr;
     if (tc) {
-        // fused combine: the last split of each unit writes out and lse2
-        int32_t *arr = at<int32_t>(ws, w.arrivals);
-        if (!counters_zeroed)
-            IKV_TRY_CUDA(cudaMemsetAsync(arr, 0, sizeof(int32_t) * (size_t)s->batch * n_layers * s->kv_heads, st),
-                         "cudaMemsetAsync");
         TcOutputs o{out, at<float>(ws, w.lse2), arr};
         if (max_len > 0) IKV_TRY_CUDA(launch_attend_tc(a, o, group, sm_count(), st), "tensor-core attend launch");
         if (tm && tm->attend_end) IKV_TRY_CUDA(cudaEventRecord(tm->attend_end, st), "cudaEventRecord");
     } else {
-        if (max_len > 0) IKV_TRY_CUDA(launch_attend(a, s->dtype, s->head_dim, group, st), "attend launch");
+        if (max_len > 0 || merges) IKV_TRY_CUDA(launch_attend(a, s->dtype, s->head_dim, group, st), "attend launch");
         if (tm && tm->attend_end) IKV_TRY_CUDA(cudaEventRecord(tm->attend_end, st), "cudaEventRecord");
+    }
+    if (!merges) {
         CombineArgs cb{};
         cb.len = c->len;
         cb.batch = s->batch;
@@ -475,7 +498,7 @@ ikv_status ikv_attend_plan(const ikv_shape *shape, const ikv_cache *cache, int32
         gs = nc == 1 && use_tc(shape, cache, shape->layers, max_len) ? 1 : 0;
         np = tc_passes(units, nc, sms, gs != 0);
     } else {
-        choose_splits(shape, n_layers, max_len, kTileTokens, 1 << 30, &ct, &nc, sms);
+        choose_splits(shape, n_layers, max_len, &ct, &nc, sms);
     }
     if (path) *path = tc ? IKV_PATH_TENSOR_CORE : IKV_PATH_CUDA_CORE;
     if (chunk_tokens) *chunk_tokens = ct;

@@ -13,6 +13,8 @@ constexpr int kTileTokens = 64;    // K/V rows staged per attention tile
 constexpr int kAttendThreads = 128;
 constexpr int kMaxSplits = 128;    // split-K partitions per (seq, layer, kv head)
 constexpr int kMinSplitTokens = 256;
+constexpr int kSplitCtaTokens = 32;       // a split CTA's fixed cost, as tokens of its stream
+constexpr int kSplitMergeTokens = 64;     // the merge of a unit's splits, likewise
 constexpr int kMaxLayersPerScorePass = 32;
 constexpr int kFusedSelectMaxLen = 16384;  // longest row bound for which the score pass also selects
 constexpr int kScoreLayersPerGroup = 8;   // eligible layers one score CTA folds (one warp each)
@@ -76,10 +78,12 @@ struct PagedView {
     const int32_t *block_table;
     const int32_t *start;       // [batch] or null (all zero)
     int32_t num_pages, page_size, max_pages, kv_heads, head_dim;
+    int32_t page_shift;         // log2(page_size), or -1 if it is no power of two
     __device__ __forceinline__ int32_t start_of(int32_t b) const { return start ? start[b] : 0; }
     __device__ __forceinline__ int64_t row_phys(int32_t b, int32_t l, int32_t g, int32_t phys) const {
-        const int32_t page = block_table[(int64_t)b * max_pages + phys / page_size];
-        return (((int64_t)l * num_pages + page) * kv_heads + g) * page_size + phys % page_size;
+        const int32_t lp = page_shift >= 0 ? phys >> page_shift : phys / page_size;
+        const int32_t page = block_table[(int64_t)b * max_pages + lp];
+        return (((int64_t)l * num_pages + page) * kv_heads + g) * page_size + (phys - lp * page_size);
     }
 };
 
@@ -111,6 +115,10 @@ struct AttendArgs {
     // of its query group's normalised probabilities ([batch][sc_layers][kv_heads][lstride])
     // instead of per-head logits
     int32_t gsum;
+    // fp32 kernel: results of units of one split, and of the last CTA to arrive at the others
+    void *out;                  // [n_layers][batch][H][D] fp32
+    float *lse2;                // [batch][sc_layers][H]
+    int32_t *arrivals;          // [batch][n_layers][kv_heads], zero on entry, left zero
     // tensor-core kernel: the launch may set up and start its K/V stream before the
     // programmatic-dependency wait (see TcArgs::early)
     int32_t early;
@@ -188,6 +196,8 @@ int tc_passes(int64_t units, int n_chunks, int sms, bool gsum);
 cudaError_t launch_attend_tc(const AttendArgs &a, const TcOutputs &o, int group, int sms, cudaStream_t st);
 
 // launchers (return cudaError_t of the launch)
+// CTAs of the fp32 kernel an SM holds (shared memory)
+constexpr int kF32CtasPerSm = 2;
 cudaError_t launch_attend(const AttendArgs &a, int dtype, int head_dim, int group, cudaStream_t st);
 cudaError_t launch_combine(const CombineArgs &a, int dtype, cudaStream_t st);
 cudaError_t launch_score_ema(const ScoreArgs &a, int32_t max_len, int sms, cudaStream_t st);
