@@ -86,7 +86,7 @@ def rank_seed(base_seed: int, rank: int) -> int:
 
 
 # revision of each attention kernel; a committed ncu summary counts only for its own revision
-ATTEND_KERNEL_REV = {"attend_tc_kernel": "attend_tc_v13", "attend_split_kernel": "attend_split_v2"}
+ATTEND_KERNEL_REV = {"attend_tc_kernel": "attend_tc_v13", "attend_bf16_kernel": "attend_bf16_v1", "attend_f32_kernel": "attend_f32_v1"}
 
 
 def schedule_name(w) -> str:
@@ -899,7 +899,7 @@ def run_ours(args):
     traj_ms = run_trajectory(traj_w, c, u_dev, qs_dev, kn_dev, vn_dev, ws, compact_mode, mh, dist)
     L = [min(x + 1, B + 1) for x, B in zip(w.prefill, w.budgets())]  # length seen by the timed steps
     att_kernel = ("attend_tc_kernel" if ikv.ikv_attend_path(c.shape(), c.cache(max(L))) == ikv.IKV_PATH_TENSOR_CORE
-                  else "attend_split_kernel")
+                  else "attend_f32_kernel" if w.dtype == gen.F32 else "attend_bf16_kernel")
 
     head_sched = schedule_name(w)
     modes = {}

@@ -204,30 +204,25 @@ void choose_splits(const ikv_shape *s, int n_layers, int32_t max_len, int32_t *s
                    int sms) {
     const int64_t units = (int64_t)s->batch * n_layers * s->kv_heads;
     int64_t best = 1;
-    if (s->dtype == IKV_F32) {
-        // The count that finishes first when the CTAs run in whole waves over the resident
-        // slots: waves x tokens of a split, plus what each CTA costs besides (as tokens of
-        // its stream) and what a merge does.  Measured, us a step for 1 / 2 / 3 / 4 / 5 / 7 /
-        // 9 / 12 splits: 128 units of 2049 tokens (d = 128, G = 4) 108 / 83 / 85 / 80 / 83 /
-        // 77 / 82 / 83 (7 taken: 2.95 waves), 256 units 129 / 135 / 135 / 135 / - / 135 (1 taken).
-        const int64_t slots = (int64_t)sms * kF32CtasPerSm;
-        int64_t best_cost = INT64_MAX;
-        for (int64_t n = 1; n <= kMaxSplits && (n == 1 || (n - 1) * kTileTokens < max_len); ++n) {
-            const int64_t st = ((max_len + n - 1) / n + kTileTokens - 1) / kTileTokens * kTileTokens;
-            const int64_t cost = (units * n + slots - 1) / slots * slots * st + units * n * kSplitCtaTokens +
-                                 (n > 1 ? slots * kSplitMergeTokens : 0);
-            if (cost < best_cost) {
-                best_cost = cost;
-                best = n;
-            }
+    // The count that finishes first when the CTAs run in whole waves over the resident
+    // slots: waves x tokens of a split, plus what each CTA costs besides (its ramp, as tokens
+    // of its stream: 112 KB of an SM's stream shared by the CTAs on it) and what a merge does.
+    // Measured, us a step for 1 / 2 / 3 / 4 / 5 / 7 splits of 2049 tokens.  fp32, d = 128,
+    // G = 4: 128 units 108 / 83 / 85 / 80 / 83 / 77 (7 taken: 2.95 waves), 256 units
+    // 129 / 135 / 135 / 135 / - / 135 (1 taken).  bf16, d = 64: 256 units 58 / 52 / 57 / 53 /
+    // - / 54 (2 taken), 1024 units 130 / 139 / 135 / 138 / 142 / 152 (1 taken).
+    const int ctas = s->dtype == IKV_F32 ? kF32CtasPerSm : s->head_dim == 64 ? kBf16D64CtasPerSm : kBf16D128CtasPerSm;
+    const int64_t slots = (int64_t)sms * ctas;
+    const int64_t cta_tokens = (112 << 10) / (ctas * 2 * s->head_dim * elem_bytes(s));
+    int64_t best_cost = INT64_MAX;
+    for (int64_t n = 1; n <= kMaxSplits && (n == 1 || (n - 1) * kTileTokens < max_len); ++n) {
+        const int64_t st = ((max_len + n - 1) / n + kTileTokens - 1) / kTileTokens * kTileTokens;
+        const int64_t cost = (units * n + slots - 1) / slots * slots * st + units * n * cta_tokens +
+                             (n > 1 ? slots * kSplitMergeTokens : 0);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = n;
         }
-    } else {
-        const int64_t want = (int64_t)sms * 4;
-        best = (want + units - 1) / units;
-        const int64_t by_len = (max_len + kMinSplitTokens - 1) / kMinSplitTokens;
-        if (best > by_len) best = by_len;
-        if (best > kMaxSplits) best = kMaxSplits;
-        if (best < 1) best = 1;
     }
     int64_t st = ((max_len + best - 1) / best + kTileTokens - 1) / kTileTokens * kTileTokens;
     if (st < kTileTokens) st = kTileTokens;
@@ -236,7 +231,7 @@ void choose_splits(const ikv_shape *s, int n_layers, int32_t max_len, int32_t *s
     *n_splits = (int32_t)(ns < 1 ? 1 : ns);
 }
 
-// attention (+ combine) over layers [layer0, layer0 + n_layers)
+// attention over layers [layer0, layer0 + n_layers)
 // The tensor-core kernel serves bf16, d = 128, groups {1,2,4,7,8}, page sizes that tile
 // 128 rows, and pools whose rows a 32-bit TMA coordinate reaches; the split-K CUDA-core
 // kernel serves the rest.
@@ -309,11 +304,9 @@ ikv_status run_attend(const ikv_shape *s, const ikv_cache *c, int32_t layer0, in
     } else if (append) {
         IKV_TRY_CUDA(launch_append_rows(*append, st), "append rows launch");
     }
-    // the tensor-core and fp32 kernels merge their splits themselves: the last CTA of each
-    // unit writes out and lse2
-    const bool merges = tc || s->dtype == IKV_F32;
+    // the last CTA of each unit of several splits merges them into out and lse2
     int32_t *arr = at<int32_t>(ws, w.arrivals);
-    if (merges && a.n_splits > 1 && !counters_zeroed)
+    if (a.n_splits > 1 && !counters_zeroed)
         IKV_TRY_CUDA(cudaMemsetAsync(arr, 0, sizeof(int32_t) * (size_t)s->batch * n_layers * s->kv_heads, st),
                      "cudaMemsetAsync");
     a.out = out;
@@ -324,25 +317,8 @@ ikv_status run_attend(const ikv_shape *s, const ikv_cache *c, int32_t layer0, in
         if (max_len > 0) IKV_TRY_CUDA(launch_attend_tc(a, o, group, sm_count(), st), "tensor-core attend launch");
         if (tm && tm->attend_end) IKV_TRY_CUDA(cudaEventRecord(tm->attend_end, st), "cudaEventRecord");
     } else {
-        if (max_len > 0 || merges) IKV_TRY_CUDA(launch_attend(a, s->dtype, s->head_dim, group, st), "attend launch");
+        IKV_TRY_CUDA(launch_attend(a, s->dtype, s->head_dim, group, st), "attend launch");
         if (tm && tm->attend_end) IKV_TRY_CUDA(cudaEventRecord(tm->attend_end, st), "cudaEventRecord");
-    }
-    if (!merges) {
-        CombineArgs cb{};
-        cb.len = c->len;
-        cb.batch = s->batch;
-        cb.q_heads = s->q_heads;
-        cb.n_layers = n_layers;
-        cb.split_tokens = a.split_tokens;
-        cb.n_splits = a.n_splits;
-        cb.head_dim = s->head_dim;
-        cb.part_ml = a.part_ml;
-        cb.part_o = a.part_o;
-        cb.out = out;
-        cb.lse2 = at<float>(ws, w.lse2);
-        cb.sc_layers = a.sc_layers;
-        cb.sc_layer0 = a.sc_layer0;
-        IKV_TRY_CUDA(launch_combine(cb, s->dtype, st), "combine launch");
     }
     if (split_out) *split_out = a.split_tokens;
     if (nsplit_out) *nsplit_out = a.n_splits;

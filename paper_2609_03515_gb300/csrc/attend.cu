@@ -1,71 +1,31 @@
-// Split-K grouped-query decode attention that also emits per-token logits.
+// Split-K grouped-query decode attention that also emits per-token logits, for the shapes
+// the TMA / tcgen05 kernel of attend_tc.cu does not take: fp32 caches, 64-dim heads, page
+// sizes that do not tile 128 rows, pools past its 32-bit row coordinates.
 //
-// One CTA handles (split s, kv head g, sequence b, layer l): the G query heads
-// of KV head g against cache slots [s*split, min((s+1)*split, len[b])).
-// K/V rows stream through shared memory in 64-token tiles (cp.async, 16-byte
-// chunks, XOR-swizzled by row so both the token-major QK reads and the
-// dim-major PV reads are bank-conflict free).  QK: each warp owns a quarter of
-// the head dimension and two tokens per lane; partial dot products meet in
-// shared memory.  Softmax is online per head in the log2 domain (the query is
-// pre-scaled by log2(e)/sqrt(d)); each tile's logits are written out for the
-// Eq. 1 score pass.  PV: each thread owns one 16-byte column chunk of V for all
-// G heads over a strided subset of the tile's tokens.  The split's running
-// (max, sum) and unnormalised output go to the workspace; combine_kernel merges
-// splits, writes the output and the per-head log-sum-exp.
+// One CTA of four warps handles (split s, kv head g, sequence b, layer l): the G query heads
+// of KV head g against cache slots [s*split, min((s+1)*split, len[b])).  Each warp streams its
+// own share of the tokens through a private cp.async ring and keeps its own online softmax
+// in the log2 domain; the logits are written out for the Eq. 1 score pass.  The warps'
+// results meet in shared memory once, at the end; a unit of several splits is merged by its
+// last CTA to arrive.
 #include "ikv_internal.cuh"
 
 namespace ikv {
 namespace {
 
-__device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
-    const uint32_t s = static_cast<uint32_t>(__cvta_generic_to_shared(smem));
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem) : "memory");
+// 16 bytes to shared memory, the first n of them (0 or 16) from gmem and the rest zeros
+__device__ __forceinline__ void cp_async16_n(uint32_t smem, const void *gmem, uint32_t n) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(smem), "l"(gmem), "r"(n) : "memory");
 }
-// the same, or 16 zero bytes (nothing read) when !in
 __device__ __forceinline__ void cp_async16_zfill(void *smem, const void *gmem, bool in) {
-    const uint32_t s = static_cast<uint32_t>(__cvta_generic_to_shared(smem));
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(s), "l"(gmem), "r"(in ? 16 : 0) : "memory");
+    cp_async16_n(static_cast<uint32_t>(__cvta_generic_to_shared(smem)), gmem, in ? 16u : 0u);
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
-template <typename T>
-struct Chunk;
-template <>
-struct Chunk<__nv_bfloat16> {
-    static constexpr int kElems = 8;
-    __device__ __forceinline__ static void load(const uint4 &c, float *x) {
-        const uint32_t w[4] = {c.x, c.y, c.z, c.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            x[2 * i] = __uint_as_float(w[i] << 16);
-            x[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
-        }
-    }
-    __device__ __forceinline__ static void store(void *p, int64_t idx, float v) {
-        reinterpret_cast<__nv_bfloat16 *>(p)[idx] = __float2bfloat16_rn(v);
-    }
-    __device__ __forceinline__ static float read(const void *p, int64_t idx) {
-        return __bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(p)[idx]);
-    }
-};
-template <>
-struct Chunk<float> {
-    static constexpr int kElems = 4;
-    __device__ __forceinline__ static void load(const uint4 &c, float *x) {
-        x[0] = __uint_as_float(c.x);
-        x[1] = __uint_as_float(c.y);
-        x[2] = __uint_as_float(c.z);
-        x[3] = __uint_as_float(c.w);
-    }
-    __device__ __forceinline__ static void store(void *p, int64_t idx, float v) {
-        reinterpret_cast<float *>(p)[idx] = v;
-    }
-    __device__ __forceinline__ static float read(const void *p, int64_t idx) {
-        return reinterpret_cast<const float *>(p)[idx];
-    }
-};
+__device__ __forceinline__ void store_as(__nv_bfloat16 *p, float v) { *p = __float2bfloat16_rn(v); }
+__device__ __forceinline__ void store_as(float *p, float v) { *p = v; }
 
 __device__ __forceinline__ float warp_max(float v) {
 #pragma unroll
@@ -76,243 +36,6 @@ __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
-}
-
-template <typename T, int D, int G>
-struct AttendCfg {
-    static constexpr int TT = kTileTokens;
-    static constexpr int kRowBytes = D * (int)sizeof(T);
-    static constexpr int CPR = kRowBytes / 16;             // 16-byte chunks per row
-    static constexpr int EPC = Chunk<T>::kElems;          // elements per chunk
-    static constexpr int QCH = CPR / 4;                   // chunks per warp in QK
-    static constexpr int NTG = kAttendThreads / CPR;      // token groups in PV
-    static constexpr int kTileBytes = TT * kRowBytes;
-    static constexpr int kStageBytes = 2 * kTileBytes;    // K + V
-    static constexpr int NSTAGE = kStageBytes <= 32768 ? 3 : 2;
-    static constexpr int GP = (G + 3) / 4 * 4;
-    static constexpr int kStageArea = NSTAGE * kStageBytes;
-    static constexpr int kObufBytes = NTG * G * D * 4;
-    static_assert(kObufBytes <= kStageArea, "output reduction must fit in the stage area");
-    static_assert(CPR >= 8 && CPR % 4 == 0, "row must be >= 8 chunks");
-    // float regions after the stage area
-    static constexpr int kQ = 0;                          // G*D
-    static constexpr int kRed = kQ + G * D;               // 4*G*TT
-    static constexpr int kZ = kRed + 4 * G * TT;          // G*TT
-    static constexpr int kP = kZ + G * TT;                // TT*GP
-    static constexpr int kM = kP + TT * GP;               // G
-    static constexpr int kL = kM + GP;                    // G
-    static constexpr int kC = kL + GP;                    // G
-    static constexpr int kFloats = kC + GP;
-    static constexpr int kSmemBytes = kStageArea + kFloats * 4;
-};
-
-template <typename T, int D, int G, bool LOGITS>
-__global__ void __launch_bounds__(kAttendThreads, 2) attend_split_kernel(const AttendArgs a) {
-    using C = AttendCfg<T, D, G>;
-    pdl_wait();
-    extern __shared__ __align__(128) unsigned char smem[];
-    float *fs = reinterpret_cast<float *>(smem + C::kStageArea);
-    float *q_s = fs + C::kQ;
-    float *red = fs + C::kRed;
-    float *zt = fs + C::kZ;
-    float *p_s = fs + C::kP;
-    float *m_run = fs + C::kM;
-    float *l_run = fs + C::kL;
-    float *corr_s = fs + C::kC;
-
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int s = blockIdx.x, g = blockIdx.y;
-    const int b = blockIdx.z % a.batch, li = blockIdx.z / a.batch;
-    const int l = a.layer0 + li;
-    const int L = a.len[b];
-    const int S0 = a.pv.start_of(b);
-    const int32_t *prow = a.pos ? a.pos + ((int64_t)b * a.rows_per_seq + (a.rows_per_seq == 1 ? 0 : g)) * a.cap : nullptr;
-    const int t0 = s * a.split_tokens;
-    if (t0 >= L) return;
-    const int t1 = min(t0 + a.split_tokens, L);
-    const int H = a.q_heads;
-    const int n_tiles = (t1 - t0 + C::TT - 1) / C::TT;
-
-    const unsigned char *kbase = reinterpret_cast<const unsigned char *>(a.k);
-    const unsigned char *vbase = reinterpret_cast<const unsigned char *>(a.v);
-
-    auto issue_tile = [&](int tile) {
-        unsigned char *st = smem + (tile % C::NSTAGE) * C::kStageBytes;
-        const int base = t0 + tile * C::TT;
-#pragma unroll
-        for (int it = 0; it < C::TT * C::CPR / kAttendThreads; ++it) {
-            const int idx = it * kAttendThreads + tid;
-            const int j = idx / C::CPR, c = idx % C::CPR;
-            const int tok = base + j;
-            if (tok < t1) {
-                const int64_t row = a.pv.row_phys(b, l, g, S0 + tok);
-                const int off = j * C::kRowBytes + ((c ^ (j & 7)) << 4);
-                cp_async16(st + off, kbase + row * C::kRowBytes + c * 16);
-                cp_async16(st + C::kTileBytes + off, vbase + row * C::kRowBytes + c * 16);
-            }
-        }
-    };
-
-    // prologue: start the first tiles before touching anything else
-#pragma unroll
-    for (int i = 0; i < C::NSTAGE - 1; ++i) {
-        if (i < n_tiles) issue_tile(i);
-        cp_async_commit();
-    }
-
-    // query of the G heads, pre-scaled into the log2 domain
-    const int64_t qoff = (((int64_t)li * a.batch + b) * H + (int64_t)g * G) * D;
-    for (int i = tid; i < G * D; i += kAttendThreads) q_s[i] = Chunk<T>::read(a.q, qoff + i) * a.scale_log2;
-    if (tid < G) {
-        m_run[tid] = -INFINITY;
-        l_run[tid] = 0.f;
-    }
-
-    float o[G][C::EPC];
-#pragma unroll
-    for (int h = 0; h < G; ++h)
-#pragma unroll
-        for (int e = 0; e < C::EPC; ++e) o[h][e] = 0.f;
-
-    const int pc = tid % C::CPR;   // PV column chunk
-    const int tg = tid / C::CPR;   // PV token group
-
-    for (int tile = 0; tile < n_tiles; ++tile) {
-        __syncthreads();  // previous tile's PV done with its stage and with p_s
-        if (tile + C::NSTAGE - 1 < n_tiles) issue_tile(tile + C::NSTAGE - 1);
-        cp_async_commit();
-        cp_async_wait<C::NSTAGE - 1>();
-        __syncthreads();
-
-        const unsigned char *Ks = smem + (tile % C::NSTAGE) * C::kStageBytes;
-        const unsigned char *Vs = Ks + C::kTileBytes;
-        const int tbase = t0 + tile * C::TT;
-        const int nv = min(C::TT, t1 - tbase);
-
-        // ---- QK: warp owns chunks [warp*QCH, (warp+1)*QCH), lane owns tokens lane, lane+32
-        {
-            float acc0[G], acc1[G];
-#pragma unroll
-            for (int h = 0; h < G; ++h) acc0[h] = acc1[h] = 0.f;
-            const int j0 = lane, j1 = lane + 32;
-#pragma unroll
-            for (int qc = 0; qc < C::QCH; ++qc) {
-                const int c = warp * C::QCH + qc;
-                float x0[C::EPC], x1[C::EPC];
-                Chunk<T>::load(*reinterpret_cast<const uint4 *>(Ks + j0 * C::kRowBytes + ((c ^ (j0 & 7)) << 4)), x0);
-                Chunk<T>::load(*reinterpret_cast<const uint4 *>(Ks + j1 * C::kRowBytes + ((c ^ (j1 & 7)) << 4)), x1);
-#pragma unroll
-                for (int h = 0; h < G; ++h) {
-                    const float4 *qp = reinterpret_cast<const float4 *>(q_s + h * D + c * C::EPC);
-#pragma unroll
-                    for (int e4 = 0; e4 < C::EPC / 4; ++e4) {
-                        const float4 qv = qp[e4];
-                        acc0[h] = fmaf(qv.x, x0[4 * e4 + 0], acc0[h]);
-                        acc0[h] = fmaf(qv.y, x0[4 * e4 + 1], acc0[h]);
-                        acc0[h] = fmaf(qv.z, x0[4 * e4 + 2], acc0[h]);
-                        acc0[h] = fmaf(qv.w, x0[4 * e4 + 3], acc0[h]);
-                        acc1[h] = fmaf(qv.x, x1[4 * e4 + 0], acc1[h]);
-                        acc1[h] = fmaf(qv.y, x1[4 * e4 + 1], acc1[h]);
-                        acc1[h] = fmaf(qv.z, x1[4 * e4 + 2], acc1[h]);
-                        acc1[h] = fmaf(qv.w, x1[4 * e4 + 3], acc1[h]);
-                    }
-                }
-            }
-#pragma unroll
-            for (int h = 0; h < G; ++h) {
-                red[(warp * G + h) * C::TT + j0] = acc0[h];
-                red[(warp * G + h) * C::TT + j1] = acc1[h];
-            }
-        }
-        __syncthreads();
-
-        // ---- logits of this tile (log2 domain), masked tail and dead slots (-inf)
-        for (int idx = tid; idx < G * C::TT; idx += kAttendThreads) {
-            const int h = idx / C::TT, j = idx % C::TT;
-            float z = red[(0 * G + h) * C::TT + j] + red[(1 * G + h) * C::TT + j] + red[(2 * G + h) * C::TT + j] +
-                      red[(3 * G + h) * C::TT + j];
-            if (j < nv) {
-                if (prow && prow[tbase + j] < 0) z = -INFINITY;
-                if (LOGITS)
-                    a.logits[((((int64_t)b * a.sc_layers + a.sc_layer0 + li) * H) + g * G + h) * (int64_t)a.lstride +
-                             tbase + j] = z;
-            } else {
-                z = -INFINITY;
-            }
-            zt[h * C::TT + j] = z;
-        }
-        __syncthreads();
-
-        // ---- online softmax per head
-        for (int h = warp; h < G; h += kAttendThreads / 32) {
-            const float za = zt[h * C::TT + lane], zb = zt[h * C::TT + lane + 32];
-            const float mx = warp_max(fmaxf(za, zb));
-            const float m_old = m_run[h];
-            const float m_new = fmaxf(m_old, mx);
-            const float m_ref = m_new == -INFINITY ? 0.f : m_new;  // every slot so far dead: nothing to scale
-            const float corr = exp2f(m_old - m_ref);
-            const float pa = exp2f(za - m_ref), pb = exp2f(zb - m_ref);
-            const float sum = warp_sum(pa + pb);
-            p_s[lane * C::GP + h] = pa;
-            p_s[(lane + 32) * C::GP + h] = pb;
-            __syncwarp();
-            if (lane == 0) {
-                l_run[h] = l_run[h] * corr + sum;
-                m_run[h] = m_new;
-                corr_s[h] = corr;
-            }
-        }
-        __syncthreads();
-
-        // ---- PV
-        {
-#pragma unroll
-            for (int h = 0; h < G; ++h) {
-                const float cr = corr_s[h];
-#pragma unroll
-                for (int e = 0; e < C::EPC; ++e) o[h][e] *= cr;
-            }
-            for (int j = tg; j < nv; j += C::NTG) {
-                float xv[C::EPC];
-                Chunk<T>::load(*reinterpret_cast<const uint4 *>(Vs + j * C::kRowBytes + ((pc ^ (j & 7)) << 4)), xv);
-                float p[C::GP];
-#pragma unroll
-                for (int h4 = 0; h4 < C::GP / 4; ++h4) {
-                    const float4 pv = reinterpret_cast<const float4 *>(p_s + j * C::GP)[h4];
-                    p[4 * h4] = pv.x;
-                    p[4 * h4 + 1] = pv.y;
-                    p[4 * h4 + 2] = pv.z;
-                    p[4 * h4 + 3] = pv.w;
-                }
-#pragma unroll
-                for (int h = 0; h < G; ++h)
-#pragma unroll
-                    for (int e = 0; e < C::EPC; ++e) o[h][e] = fmaf(p[h], xv[e], o[h][e]);
-            }
-        }
-    }
-
-    // ---- reduce the PV token groups, write the split partial
-    cp_async_wait<0>();
-    __syncthreads();
-    float *obuf = reinterpret_cast<float *>(smem);
-#pragma unroll
-    for (int h = 0; h < G; ++h)
-#pragma unroll
-        for (int e = 0; e < C::EPC; ++e) obuf[(tg * G + h) * D + pc * C::EPC + e] = o[h][e];
-    __syncthreads();
-    const int64_t pbase = (((int64_t)b * a.n_layers + li) * H + (int64_t)g * G) * a.n_splits;
-    for (int idx = tid; idx < G * D; idx += kAttendThreads) {
-        const int h = idx / D, e = idx % D;
-        float acc = 0.f;
-#pragma unroll
-        for (int t = 0; t < C::NTG; ++t) acc += obuf[(t * G + h) * D + e];
-        a.part_o[((pbase + (int64_t)h * a.n_splits) + s) * D + e] = acc;
-    }
-    if (tid < G) {
-        a.part_ml[((pbase + (int64_t)tid * a.n_splits) + s) * 2 + 0] = m_run[tid];
-        a.part_ml[((pbase + (int64_t)tid * a.n_splits) + s) * 2 + 1] = l_run[tid];
-    }
 }
 
 // What the CTAs of a (sequence, layer, kv head) unit do once a CTA has its split's result:
@@ -343,7 +66,7 @@ __device__ __forceinline__ void finish_split(const AttendArgs &a, float *obuf, f
             acc += obuf[(w * G + h) * D + e] * f;
         }
         if (ns_active == 1) {
-            Chunk<T>::store(a.out, (hrow + h) * D + e, sum > 0.f ? acc / sum : 0.f);
+            store_as(static_cast<T *>(a.out) + (hrow + h) * D + e, sum > 0.f ? acc / sum : 0.f);
             if (e == 0) a.lse2[lrow + h] = sum > 0.f ? M + log2f(sum) : -INFINITY;
         } else {
             const int64_t at = pbase + (int64_t)h * a.n_splits + s;
@@ -407,7 +130,7 @@ __device__ __forceinline__ void finish_split(const AttendArgs &a, float *obuf, f
         }
 #pragma unroll
         for (int e = 0; e < E; ++e)
-            Chunk<T>::store(a.out, (hrow + h) * D + lane * E + e, W > 0.f ? acc[e] / W : 0.f);
+            store_as(static_cast<T *>(a.out) + (hrow + h) * D + lane * E + e, W > 0.f ? acc[e] / W : 0.f);
         if (lane == 0) a.lse2[lrow + h] = W > 0.f ? M + log2f(W) : -INFINITY;
         __syncwarp();
     }
@@ -417,7 +140,7 @@ __device__ __forceinline__ void finish_split(const AttendArgs &a, float *obuf, f
 template <typename T>
 __device__ __forceinline__ void store_empty(const AttendArgs &a, int G, int D, int b, int li, int g) {
     const int64_t hrow = ((int64_t)li * a.batch + b) * a.q_heads + (int64_t)g * G;
-    for (int i = threadIdx.x; i < G * D; i += kAttendThreads) Chunk<T>::store(a.out, hrow * D + i, 0.f);
+    for (int i = threadIdx.x; i < G * D; i += kAttendThreads) store_as(static_cast<T *>(a.out) + hrow * D + i, 0.f);
     if ((int)threadIdx.x < G)
         a.lse2[((int64_t)b * a.sc_layers + a.sc_layer0 + li) * a.q_heads + (int64_t)g * G + threadIdx.x] = -INFINITY;
 }
@@ -641,49 +364,251 @@ __global__ void __launch_bounds__(kAttendThreads, 2) attend_f32_kernel(const Att
     finish_split<float, D, GP, C::P>(a, obuf, mlbuf, G, s, ns_active, b, li, g);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(128) combine_kernel(const CombineArgs a) {
-    pdl_wait();
-    const int h = blockIdx.x;
-    const int b = blockIdx.y % a.batch, li = blockIdx.y / a.batch;
-    const int D = a.head_dim;
-    const int L = a.len[b];
-    const int ns = min((L + a.split_tokens - 1) / a.split_tokens, a.n_splits);
-    const int64_t pbase = (((int64_t)b * a.n_layers + li) * a.q_heads + h) * a.n_splits;
-    const float *ml = a.part_ml + pbase * 2;
-    float M = -INFINITY;
-    for (int s = 0; s < ns; ++s) M = fmaxf(M, ml[2 * s]);
-    const float Mref = M == -INFINITY ? 0.f : M;  // splits whose slots are all dead carry -inf
-    float wsum = 0.f;
-    for (int s = 0; s < ns; ++s) wsum += ml[2 * s + 1] * exp2f(ml[2 * s] - Mref);
-    const float inv = wsum > 0.f ? 1.f / wsum : 0.f;
-    const int64_t obase = (((int64_t)li * a.batch + b) * a.q_heads + h) * D;
-    for (int e = threadIdx.x; e < D; e += blockDim.x) {
-        float acc = 0.f;
-        for (int s = 0; s < ns; ++s) acc += a.part_o[(pbase + s) * D + e] * exp2f(ml[2 * s] - Mref);
-        Chunk<T>::store(a.out, obase + e, acc * inv);
-    }
-    if (a.lse2 && threadIdx.x == 0)
-        a.lse2[((int64_t)b * a.sc_layers + a.sc_layer0 + li) * a.q_heads + h] = wsum > 0.f ? M + log2f(wsum) : -INFINITY;
+// bf16 K/V (head_dim 64, and the 128-dim shapes the TMA kernel of attend_tc.cu does not
+// take).  HBM bound; mma.sync keeps the arithmetic (32 m16n8k16 per 16 tokens of 64 dims)
+// under half of the stream's time.  As in the fp32 kernel every warp runs alone: its own
+// ring of 16-token stages, its own online softmax over every fourth group of the split, no
+// block barrier.  The heads are the M rows: S = Q K^T leaves each lane four logits of one
+// head, which are the A operand of O += P V as they stand.  Rows 8-15 of that operand would
+// be padding (a group has at most 8 heads); they carry the second of three bf16 terms whose
+// sum is the fp32 probability bit for bit (8 + 8 + 8 mantissa bits), and one more product
+// adds the third, so P loses nothing to the tensor cores' operand type. Measured, a whole step of
+// b = 8, 16 layers, 32 / 8 heads of 64, 2048 tokens (539 MB, 79.5 us at the copy rate):
+// 222.4 -> 128.5 us against the CUDA-core kernel with its block barriers; 128 dims in
+// 48-token pages 271 -> 208 us when 32 tokens, not 16, came to share the row look-ups and
+// the registers left room for 16 warps an SM.  What is left: the ramp of each CTA (length,
+// table, rows: three dependent loads) and 1.7 waves of CTAs.
+__device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t (&r)[4]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr)
+                 : "memory");
+}
+__device__ __forceinline__ void ldsm_x4_trans(uint32_t addr, uint32_t (&r)[4]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr)
+                 : "memory");
+}
+__device__ __forceinline__ void mma_16x8x16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
+                                            uint32_t b0, uint32_t b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, "
+        "%2, %3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+// x and y to bf16 (packed), and what that leaves of them
+__device__ __forceinline__ uint32_t take_bf16(float &x, float &y) {
+    const __nv_bfloat162 t = __floats2bfloat162_rn(x, y);
+    x -= __low2float(t);
+    y -= __high2float(t);
+    return *reinterpret_cast<const uint32_t *>(&t);
 }
 
-template <typename T, int D, int G>
-cudaError_t launch_attend_t(const AttendArgs &a, cudaStream_t st) {
-    using C = AttendCfg<T, D, G>;
-    dim3 grid(a.n_splits, a.pv.kv_heads, a.batch * a.n_layers);
-    if (a.logits) {
-        auto k = attend_split_kernel<T, D, G, true>;
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
-        if (e != cudaSuccess) return e;
-        { cudaError_t le = launch_k(k, grid, dim3(kAttendThreads), C::kSmemBytes, st, a); if (le != cudaSuccess) return le; }
-    } else {
-        auto k = attend_split_kernel<T, D, G, false>;
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
-        if (e != cudaSuccess) return e;
-        { cudaError_t le = launch_k(k, grid, dim3(kAttendThreads), C::kSmemBytes, st, a); if (le != cudaSuccess) return le; }
+template <int D>
+struct Bf16Cfg {
+    static constexpr int GP = 8;                 // heads of the M rows 0-7
+    static constexpr int TW = 16;                // tokens of a stage; a warp's block is two stages
+    static constexpr int kRowB = D * 2;
+    static constexpr int RL = kRowB / 16;        // lanes of a row (16 bytes each)
+    static constexpr int RPI = 32 / RL;          // rows a warp copies at once
+    static constexpr int kStageB = 2 * TW * kRowB;
+    static constexpr int NST = 3;
+    static constexpr int kWarps = kAttendThreads / 32;
+    static constexpr int kRing = kWarps * NST * kStageB;
+    static constexpr int kSmemBytes = kRing + 2 * kWarps * GP * 4;
+    static constexpr int kCtasPerSm = D == 64 ? kBf16D64CtasPerSm : kBf16D128CtasPerSm;
+    static_assert(kWarps * GP * D * 4 <= kRing && kWarps * kMaxSplits * 4 <= kRing, "the merge reuses the ring");
+    static_assert(kCtasPerSm * (kSmemBytes + 1024) <= 227 * 1024, "resident CTAs");
+};
+
+template <int D>
+__global__ void __launch_bounds__(kAttendThreads, Bf16Cfg<D>::kCtasPerSm) attend_bf16_kernel(const AttendArgs a) {
+    using C = Bf16Cfg<D>;
+    constexpr int TW = C::TW, NST = C::NST;
+    pdl_wait();
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int s = blockIdx.x, g = blockIdx.y;
+    const int b = blockIdx.z % a.batch, li = blockIdx.z / a.batch;
+    const int l = a.layer0 + li;
+    const int G = a.q_heads / a.pv.kv_heads;
+    const int L = a.len[b];
+    const int S0 = a.pv.start_of(b);
+    const int t0 = s * a.split_tokens;
+    if (t0 >= L) {
+        if (s == 0) store_empty<__nv_bfloat16>(a, G, D, b, li, g);
+        return;
     }
-    note_launch();
-    return cudaGetLastError();
+    const int t1 = min(t0 + a.split_tokens, L);
+    const int ns_active = min((L + a.split_tokens - 1) / a.split_tokens, a.n_splits);
+    const int32_t *prow = a.pos ? a.pos + ((int64_t)b * a.rows_per_seq + (a.rows_per_seq == 1 ? 0 : g)) * a.cap : nullptr;
+    const uint32_t ring = static_cast<uint32_t>(__cvta_generic_to_shared(smem)) + warp * NST * C::kStageB;
+    float *mlbuf = reinterpret_cast<float *>(smem + C::kRing);
+
+    // The warp takes every fourth 32-token block of the split, from tok0 on.  Lane i looks up
+    // the pool row of the block's token i (a row index fits 32 bits: rows are 128 bytes at
+    // least; ~0 past the split) and its liveness, two blocks and one block ahead of their use.
+    int tok0 = t0 + warp * 32;
+    constexpr int kStride = C::kWarps * 32;
+    const int64_t page0 = (int64_t)l * a.pv.num_pages;
+    const int32_t *table = a.pv.block_table + (int64_t)b * a.pv.max_pages;
+    auto lookup = [&](int base) -> uint32_t {
+        const int tok = base + lane;
+        if (tok >= t1) return ~0u;
+        const int phys = S0 + tok;
+        const int lp = a.pv.page_shift >= 0 ? phys >> a.pv.page_shift : phys / a.pv.page_size;
+        return (uint32_t)(((page0 + table[lp]) * a.pv.kv_heads + g) * a.pv.page_size + (phys - lp * a.pv.page_size));
+    };
+    auto alive = [&](int base) -> bool { return base + lane < t1 && (!prow || __ldg(prow + base + lane) >= 0); };
+    // 16-byte chunk c of a row lies at c ^ (row % 8): the eight rows an ldmatrix reads at one
+    // chunk fall into different banks
+    const int cr = lane / C::RL, cc = lane % C::RL;
+    const unsigned char *kb = reinterpret_cast<const unsigned char *>(a.k) + cc * 16;
+    const unsigned char *vb = reinterpret_cast<const unsigned char *>(a.v) + cc * 16;
+    auto issue = [&](int stage, int half, uint32_t rows) {
+        const uint32_t st = ring + stage * C::kStageB + cr * C::kRowB;
+#pragma unroll
+        for (int t = 0; t < TW; t += C::RPI) {
+            const uint32_t r = __shfl_sync(0xffffffffu, rows, half * TW + t + cr);
+            const uint32_t n = r == ~0u ? 0u : 16u;
+            const uint64_t at = (uint64_t)(r == ~0u ? 0u : r) * C::kRowB;
+            const uint32_t dst = st + t * C::kRowB + ((cc ^ ((t + cr) & 7)) << 4);
+            cp_async16_n(dst, kb + at, n);
+            cp_async16_n(dst + TW * C::kRowB, vb + at, n);
+        }
+        cp_async_commit();
+    };
+    {
+        const uint32_t rows = lookup(tok0);
+        issue(0, 0, rows);
+        issue(1, 1, rows);
+    }
+    uint32_t rows_next = lookup(tok0 + kStride);
+    uint32_t live = __ballot_sync(0xffffffffu, alive(tok0));
+
+    // the lane's head (M row) and its tokens tq, tq + 1, tq + 8, tq + 9 of a stage
+    const int h = lane >> 2, tq = (lane & 3) * 2;
+    uint32_t qa[D / 16][2];
+    {
+        const __nv_bfloat16 *qg = reinterpret_cast<const __nv_bfloat16 *>(a.q) +
+                                  (((int64_t)li * a.batch + b) * a.q_heads + (int64_t)g * G + h) * D + tq;
+#pragma unroll
+        for (int k = 0; k < D / 16; ++k) {
+            qa[k][0] = h < G ? *reinterpret_cast<const uint32_t *>(qg + k * 16) : 0u;
+            qa[k][1] = h < G ? *reinterpret_cast<const uint32_t *>(qg + k * 16 + 8) : 0u;
+        }
+    }
+    float *lg = a.logits && h < G
+                    ? a.logits + ((((int64_t)b * a.sc_layers + a.sc_layer0 + li) * a.q_heads) + (int64_t)g * G + h) *
+                                     (int64_t)a.lstride + tq
+                    : nullptr;
+    // ldmatrix row addresses: K as B (tokens x dims), V transposed (dims x tokens)
+    const int mat = lane >> 3, mr = lane & 7;
+    const uint32_t k_row = (uint32_t)(((mat >> 1) * 8 + mr) * C::kRowB), k_c = mat & 1;
+    const uint32_t v_row = (uint32_t)((TW + (mat & 1) * 8 + mr) * C::kRowB), v_c = mat >> 1;
+
+    float o[D / 8][4];
+#pragma unroll
+    for (int n = 0; n < D / 8; ++n)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) o[n][e] = 0.f;
+    float m_run = -INFINITY, l_run = 0.f;
+    int stage = 0;  // ring stage of the next 16 tokens
+
+    for (; tok0 < t1; tok0 += kStride) {
+        const uint32_t rows = rows_next;
+        rows_next = lookup(tok0 + 2 * kStride);
+        const bool alive_next = alive(tok0 + kStride);
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            __syncwarp();  // the stage about to be refilled was read in the previous round
+            issue(stage == 0 ? NST - 1 : stage - 1, half, rows);
+            cp_async_wait<NST - 1>();
+            __syncwarp();  // every lane's copies of this stage have landed
+            const uint32_t st = ring + stage * C::kStageB;
+            stage = stage == NST - 1 ? 0 : stage + 1;
+            float sc[2][4];
+#pragma unroll
+            for (int n = 0; n < 2; ++n)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) sc[n][e] = 0.f;
+#pragma unroll
+            for (int k = 0; k < D / 16; ++k) {
+                uint32_t kf[4];
+                ldsm_x4(st + k_row + (((2 * k + k_c) ^ mr) << 4), kf);
+                mma_16x8x16(sc[0], qa[k][0], 0u, qa[k][1], 0u, kf[0], kf[1]);
+                mma_16x8x16(sc[1], qa[k][0], 0u, qa[k][1], 0u, kf[2], kf[3]);
+            }
+            const uint32_t lv = h < G ? live >> (half * TW + tq) : 0u;  // bits 0, 1, 8, 9: the lane's tokens
+            float z[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                z[j] = (lv >> ((j >> 1) * 8 + (j & 1))) & 1u ? sc[j >> 1][j & 1] * a.scale_log2 : -INFINITY;
+            if (lg) {
+                const int x = tok0 + half * TW;
+#pragma unroll
+                for (int n = 0; n < 2; ++n) {
+                    if (x + n * 8 + tq + 1 < t1)
+                        *reinterpret_cast<float2 *>(lg + x + n * 8) = make_float2(z[2 * n], z[2 * n + 1]);
+                    else if (x + n * 8 + tq < t1)
+                        lg[x + n * 8] = z[2 * n];
+                }
+            }
+            float mx = fmaxf(fmaxf(z[0], z[1]), fmaxf(z[2], z[3]));
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+            const float m_new = fmaxf(m_run, mx);
+            const float ref = m_new == -INFINITY ? 0.f : m_new;  // every token so far dead: nothing to scale
+            if (__any_sync(0xffffffffu, m_new != m_run)) {
+                const float corr = exp2f(m_run - ref);
+                l_run *= corr;
+#pragma unroll
+                for (int n = 0; n < D / 8; ++n)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) o[n][e] *= corr;
+            }
+            m_run = m_new;
+            float p[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) p[j] = exp2f(z[j] - ref);
+            l_run += (p[0] + p[1]) + (p[2] + p[3]);
+            const uint32_t h0 = take_bf16(p[0], p[1]), h1 = take_bf16(p[2], p[3]);
+            const uint32_t m0 = take_bf16(p[0], p[1]), m1 = take_bf16(p[2], p[3]);
+            const uint32_t l0 = take_bf16(p[0], p[1]), l1 = take_bf16(p[2], p[3]);
+#pragma unroll
+            for (int n = 0; n < D / 16; ++n) {
+                uint32_t vf[4];
+                ldsm_x4_trans(st + v_row + (((2 * n + v_c) ^ mr) << 4), vf);
+                mma_16x8x16(o[2 * n], h0, m0, h1, m1, vf[0], vf[1]);
+                mma_16x8x16(o[2 * n + 1], h0, m0, h1, m1, vf[2], vf[3]);
+                mma_16x8x16(o[2 * n], 0u, l0, 0u, l1, vf[0], vf[1]);
+                mma_16x8x16(o[2 * n + 1], 0u, l0, 0u, l1, vf[2], vf[3]);
+            }
+        }
+        live = __ballot_sync(0xffffffffu, alive_next);
+    }
+    l_run += __shfl_xor_sync(0xffffffffu, l_run, 1);
+    l_run += __shfl_xor_sync(0xffffffffu, l_run, 2);
+    cp_async_wait<0>();
+    __syncthreads();  // every warp is done with its ring: the outputs go there
+    float *obuf = reinterpret_cast<float *>(smem);
+    if ((lane & 3) == 0) {
+        mlbuf[(warp * C::GP + h) * 2] = m_run;
+        mlbuf[(warp * C::GP + h) * 2 + 1] = l_run;
+    }
+    if (h < G) {
+#pragma unroll
+        for (int n = 0; n < D / 8; ++n) {
+            // an infinite V makes the first term's sum infinite and the others' NaN (0 x inf)
+            const float x = isfinite(o[n][0]) ? o[n][0] + o[n][2] : o[n][0];
+            const float y = isfinite(o[n][1]) ? o[n][1] + o[n][3] : o[n][1];
+            *reinterpret_cast<float2 *>(obuf + (warp * G + h) * D + n * 8 + tq) = make_float2(x, y);
+        }
+    }
+    __syncthreads();
+    finish_split<__nv_bfloat16, D, C::GP, C::kWarps>(a, obuf, mlbuf, G, s, ns_active, b, li, g);
 }
 
 template <int D, int G>
@@ -708,39 +633,28 @@ cudaError_t launch_attend_f32(const AttendArgs &a, int group, cudaStream_t st) {
     }
 }
 
-template <typename T, int D>
-cudaError_t launch_attend_d(const AttendArgs &a, int group, cudaStream_t st) {
-    switch (group) {
-        case 1: return launch_attend_t<T, D, 1>(a, st);
-        case 2: return launch_attend_t<T, D, 2>(a, st);
-        case 4: return launch_attend_t<T, D, 4>(a, st);
-        case 7: return launch_attend_t<T, D, 7>(a, st);
-        case 8: return launch_attend_t<T, D, 8>(a, st);
-        default: return cudaErrorInvalidValue;
-    }
+template <int D>
+cudaError_t launch_attend_bf16(const AttendArgs &a, cudaStream_t st) {
+    constexpr int smem = Bf16Cfg<D>::kSmemBytes;
+    cudaError_t e = cudaFuncSetAttribute(attend_bf16_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    e = launch_k(attend_bf16_kernel<D>, dim3(a.n_splits, a.pv.kv_heads, a.batch * a.n_layers), dim3(kAttendThreads), smem,
+                 st, a);
+    note_launch();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace
 
 cudaError_t launch_attend(const AttendArgs &a, int dtype, int head_dim, int group, cudaStream_t st) {
     if (dtype == IKV_BF16) {
-        if (head_dim == 128) return launch_attend_d<__nv_bfloat16, 128>(a, group, st);
-        if (head_dim == 64) return launch_attend_d<__nv_bfloat16, 64>(a, group, st);
+        if (head_dim == 128) return launch_attend_bf16<128>(a, st);
+        if (head_dim == 64) return launch_attend_bf16<64>(a, st);
     } else {
         if (head_dim == 128) return launch_attend_f32<128>(a, group, st);
         if (head_dim == 64) return launch_attend_f32<64>(a, group, st);
     }
     return cudaErrorInvalidValue;
-}
-
-cudaError_t launch_combine(const CombineArgs &a, int dtype, cudaStream_t st) {
-    dim3 grid(a.q_heads, a.batch * a.n_layers);
-    if (dtype == IKV_BF16)
-        { cudaError_t le = launch_k(combine_kernel<__nv_bfloat16>, grid, dim3(128), 0, st, a); if (le != cudaSuccess) return le; }
-    else
-        { cudaError_t le = launch_k(combine_kernel<float>, grid, dim3(128), 0, st, a); if (le != cudaSuccess) return le; }
-    note_launch();
-    return cudaGetLastError();
 }
 
 }  // namespace ikv

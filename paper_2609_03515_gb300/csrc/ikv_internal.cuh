@@ -9,12 +9,10 @@
 
 namespace ikv {
 
-constexpr int kTileTokens = 64;    // K/V rows staged per attention tile
+constexpr int kTileTokens = 64;    // splits of attend.cu are multiples of a tile
 constexpr int kAttendThreads = 128;
 constexpr int kMaxSplits = 128;    // split-K partitions per (seq, layer, kv head)
-constexpr int kMinSplitTokens = 256;
-constexpr int kSplitCtaTokens = 32;       // a split CTA's fixed cost, as tokens of its stream
-constexpr int kSplitMergeTokens = 64;     // the merge of a unit's splits, likewise
+constexpr int kSplitMergeTokens = 64;  // cost of merging a unit's splits, as tokens of its stream
 constexpr int kMaxLayersPerScorePass = 32;
 constexpr int kFusedSelectMaxLen = 16384;  // longest row bound for which the score pass also selects
 constexpr int kScoreLayersPerGroup = 8;   // eligible layers one score CTA folds (one warp each)
@@ -115,22 +113,13 @@ struct AttendArgs {
     // of its query group's normalised probabilities ([batch][sc_layers][kv_heads][lstride])
     // instead of per-head logits
     int32_t gsum;
-    // fp32 kernel: results of units of one split, and of the last CTA to arrive at the others
-    void *out;                  // [n_layers][batch][H][D] fp32
+    // kernels of attend.cu: results of units of one split, and of the last CTA to arrive at the others
+    void *out;                  // [n_layers][batch][H][D] (dtype)
     float *lse2;                // [batch][sc_layers][H]
     int32_t *arrivals;          // [batch][n_layers][kv_heads], zero on entry, left zero
     // tensor-core kernel: the launch may set up and start its K/V stream before the
     // programmatic-dependency wait (see TcArgs::early)
     int32_t early;
-};
-
-struct CombineArgs {
-    const int32_t *len;
-    int32_t batch, q_heads, n_layers, split_tokens, n_splits, head_dim;
-    const float *part_ml, *part_o;
-    void *out;                  // [n_layers][batch][H][D] (dtype)
-    float *lse2;                // [batch][sc_layers][H] log2-sum-exp, or null
-    int32_t sc_layers, sc_layer0;
 };
 
 // Deferred compaction inside selection: when a row has exactly one slot too many and
@@ -196,10 +185,9 @@ int tc_passes(int64_t units, int n_chunks, int sms, bool gsum);
 cudaError_t launch_attend_tc(const AttendArgs &a, const TcOutputs &o, int group, int sms, cudaStream_t st);
 
 // launchers (return cudaError_t of the launch)
-// CTAs of the fp32 kernel an SM holds (shared memory)
-constexpr int kF32CtasPerSm = 2;
+// CTAs of its kernels an SM holds (shared memory)
+constexpr int kF32CtasPerSm = 2, kBf16D64CtasPerSm = 4, kBf16D128CtasPerSm = 2;
 cudaError_t launch_attend(const AttendArgs &a, int dtype, int head_dim, int group, cudaStream_t st);
-cudaError_t launch_combine(const CombineArgs &a, int dtype, cudaStream_t st);
 cudaError_t launch_score_ema(const ScoreArgs &a, int32_t max_len, int sms, cudaStream_t st);
 // token blocks (and tokens per lane V) the score pass uses for max_len
 int score_blocks(const ScoreArgs &a, int32_t max_len, int sms, int *V);

@@ -29,9 +29,9 @@ def _reference(c, layer, q, b, g, L, live):
 EDGES = [0, 1, 7, 8, 9, 15, 16, 17, 31, 32, 33, 63, 64, 65, 127, 129, 511, 513, 2049]
 
 
-@pytest.mark.parametrize("dtype", [ikv.IKV_F32])
-@pytest.mark.parametrize("d,G,ps", [(64, 1, 64), (64, 2, 7), (64, 4, 16), (64, 7, 1), (64, 8, 48), (128, 1, 16),
-                                    (128, 2, 64), (128, 4, 3), (128, 7, 48), (128, 8, 100)])
+@pytest.mark.parametrize("dtype", [ikv.IKV_F32, ikv.IKV_BF16])
+@pytest.mark.parametrize("d,G,ps", [(64, 1, 64), (64, 2, 7), (64, 4, 16), (64, 7, 1), (64, 8, 48), (128, 1, 12),
+                                    (128, 2, 80), (128, 4, 3), (128, 7, 48), (128, 8, 100)])
 def test_attention_edges(dtype, d, G, ps):
     dt = torch.bfloat16 if dtype == ikv.IKV_BF16 else torch.float32
     kvh = 2
