@@ -129,8 +129,8 @@ typedef struct {
 
 /* Optional per-kernel CUDA events recorded on the call's stream by ikv_step
  * (caller-created with cudaEventCreate; NULL members are skipped):
- * begin (before the append), append_end, attend_end (after the attention
- * kernel), combine_end (after the split combine), score_end (after the score
+ * begin (before the append), append_end, attend_end, combine_end
+ * (both after the attention kernel, which merges its splits itself), score_end (after the score
  * + EMA kernels), select_end, end (after compaction). */
 typedef struct {
     cudaEvent_t begin, append_end, attend_end, combine_end, score_end, select_end, end;
@@ -231,8 +231,8 @@ ikv_status ikv_test_stall_next_attention(void);
  * IKV_PATH_TENSOR_CORE -- TMA-staged K/V tiles, tcgen05 QK^T and PV with TMEM
  *   accumulators; bf16, head_dim 128, group size 1, 2, 4, 7 or 8, page_size a
  *   divisor of 128 (>= 8) or a multiple of 128;
- * IKV_PATH_CUDA_CORE -- split-K flash decoding on the CUDA cores plus a combine
- *   kernel; every other supported shape.
+ * IKV_PATH_CUDA_CORE -- split-K flash decoding without TMA and TMEM (cp.async rings; fp32
+ *   on the FMA units, bf16 on mma.sync); every other supported shape.
  * Host only; launches nothing.  *path receives the value. */
 enum { IKV_PATH_CUDA_CORE = 0, IKV_PATH_TENSOR_CORE = 1 };
 ikv_status ikv_attend_path(const ikv_shape *shape, const ikv_cache *cache, int32_t *path);

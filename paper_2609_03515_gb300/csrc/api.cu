@@ -233,8 +233,8 @@ void choose_splits(const ikv_shape *s, int n_layers, int32_t max_len, int32_t *s
 
 // attention over layers [layer0, layer0 + n_layers)
 // The tensor-core kernel serves bf16, d = 128, groups {1,2,4,7,8}, page sizes that tile
-// 128 rows, and pools whose rows a 32-bit TMA coordinate reaches; the split-K CUDA-core
-// kernel serves the rest.
+// 128 rows, and pools whose rows a 32-bit TMA coordinate reaches; the split-K kernels of
+// attend.cu serve the rest.
 static bool use_tc(const ikv_shape *s, const ikv_cache *c, int32_t layers_touched, int32_t max_len) {
     const int group = s->q_heads / s->kv_heads;
     const uint64_t pool_rows = (uint64_t)layers_touched * c->num_pages * s->kv_heads * c->page_size;
@@ -255,7 +255,7 @@ ikv_status run_attend(const ikv_shape *s, const ikv_cache *c, int32_t layer0, in
                       const void *q, void *out, void *ws, const AttendWs &w, bool logits, int32_t *split_out,
                       int32_t *nsplit_out, cudaStream_t st, const ikv_timing *tm = nullptr,
                       bool counters_zeroed = false, int32_t sc_layers = 0, int32_t sc_layer0 = 0,
-                      const AppendArgs *append = nullptr, bool *gsum = nullptr) {
+                      const AppendArgs *append = nullptr, bool *gsum = nullptr, AttendArgs *unmerged = nullptr) {
     AttendArgs a{};
     a.k = c->k;
     a.v = c->v;
@@ -305,13 +305,15 @@ ikv_status run_attend(const ikv_shape *s, const ikv_cache *c, int32_t layer0, in
         IKV_TRY_CUDA(launch_append_rows(*append, st), "append rows launch");
     }
     // the last CTA of each unit of several splits merges them into out and lse2
-    int32_t *arr = at<int32_t>(ws, w.arrivals);
-    if (a.n_splits > 1 && !counters_zeroed)
+    // (`unmerged`: the caller's next kernel does, from the arguments handed back in it)
+    int32_t *arr = unmerged ? nullptr : at<int32_t>(ws, w.arrivals);
+    if (arr && a.n_splits > 1 && !counters_zeroed)
         IKV_TRY_CUDA(cudaMemsetAsync(arr, 0, sizeof(int32_t) * (size_t)s->batch * n_layers * s->kv_heads, st),
                      "cudaMemsetAsync");
     a.out = out;
     a.lse2 = at<float>(ws, w.lse2);
     a.arrivals = arr;
+    if (unmerged) *unmerged = a;
     if (tc) {
         TcOutputs o{out, at<float>(ws, w.lse2), arr};
         if (max_len > 0) IKV_TRY_CUDA(launch_attend_tc(a, o, group, sm_count(), st), "tensor-core attend launch");
@@ -498,13 +500,42 @@ ikv_status ikv_decode_attend_score(const ikv_shape *shape, const ikv_cache *cach
     const bool want_score = score || ema;
     const AttendWs w = attend_ws(shape, cap_of(cache), 1, want_score);
     if (!ws || ws_bytes < w.end) return fail(IKV_ERR_WORKSPACE, "workspace needs %zu bytes", w.end);
-    if ((e = run_attend(shape, cache, layer, 1, cache->max_len, q, out, ws, w, want_score, nullptr, nullptr, stream)))
+    // the score pass's ramp (and this attention's, in a chain of layer calls) overlaps the
+    // kernel before it
+    PdlScope pdl;
+    AttendArgs at_args{};
+    bool gsum = false;
+    if ((e = run_attend(shape, cache, layer, 1, cache->max_len, q, out, ws, w, want_score, nullptr, nullptr, stream,
+                        nullptr, false, 0, 0, nullptr, &gsum, &at_args)))
         return e;
-    if (want_score) {
-        const int32_t elig0 = 0;
-        if ((e = run_score(shape, cache, 1, &elig0, 1, cache->max_len, ws, w, ema ? alpha : 0.f, ema, score, stream)))
-            return e;
-    }
+    const bool tc = use_tc(shape, cache, layer + 1, cache->max_len);
+    ScoreOneArgs sa{};
+    sa.len = cache->len;
+    sa.start = cache->start;
+    sa.batch = shape->batch;
+    sa.q_heads = shape->q_heads;
+    sa.kv_heads = shape->kv_heads;
+    sa.rows_per_seq = rows_per_seq(shape);
+    sa.cap = cap_of(cache);
+    sa.head_dim = shape->head_dim;
+    sa.bf16 = shape->dtype == IKV_BF16;
+    sa.logits = at_args.logits;
+    sa.lstride = at_args.lstride;
+    sa.gsum = gsum;
+    sa.lse2 = at_args.lse2;
+    sa.tile = tc ? kTcTile : 0;
+    sa.split_tokens = at_args.split_tokens;
+    sa.passes = tc ? tc_passes((int64_t)shape->batch * shape->kv_heads, at_args.n_splits, sm_count(), gsum) : 1;
+    sa.n_splits = at_args.n_splits;
+    sa.part_ml = at_args.part_ml;
+    sa.part_o = at_args.part_o;
+    sa.out = out;
+    sa.alpha = alpha;
+    sa.score = score;
+    sa.ema = ema;
+    // rows and both arrays on 16-byte boundaries (null counts)
+    sa.vec = sa.cap % 4 == 0 && aligned16(score) && aligned16(ema);
+    IKV_TRY_CUDA(launch_score_one(sa, cache->max_len, sm_count(), stream), "score launch");
     return IKV_OK;
 }
 

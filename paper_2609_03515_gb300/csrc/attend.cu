@@ -8,7 +8,7 @@
 // in the log2 domain; the logits are written out for the Eq. 1 score pass.  The warps'
 // results meet in shared memory once, at the end; a unit of several splits is merged by its
 // last CTA to arrive.
-#include "ikv_internal.cuh"
+#include "merge.cuh"
 
 namespace ikv {
 namespace {
@@ -24,20 +24,6 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
-__device__ __forceinline__ void store_as(__nv_bfloat16 *p, float v) { *p = __float2bfloat16_rn(v); }
-__device__ __forceinline__ void store_as(float *p, float v) { *p = v; }
-
-__device__ __forceinline__ float warp_max(float v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
 // What the CTAs of a (sequence, layer, kv head) unit do once a CTA has its split's result:
 // P partial softmaxes over disjoint tokens, obuf [P][G][D] unnormalised outputs and mlbuf
 // [P][GP][2] (max, sum) in shared memory, merged into the split's (max, sum, output).  A
@@ -47,7 +33,7 @@ __device__ __forceinline__ float warp_sum(float v) {
 template <typename T, int D, int GP, int P>
 __device__ __forceinline__ void finish_split(const AttendArgs &a, float *obuf, float *mlbuf, int G, int s,
                                              int ns_active, int b, int li, int g) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, warp = tid >> 5;
     const int H = a.q_heads;
     const int64_t hrow = ((int64_t)li * a.batch + b) * H + (int64_t)g * G;           // out rows
     const int64_t lrow = ((int64_t)b * a.sc_layers + a.sc_layer0 + li) * H + (int64_t)g * G;  // lse2
@@ -77,7 +63,7 @@ __device__ __forceinline__ void finish_split(const AttendArgs &a, float *obuf, f
             }
         }
     }
-    if (ns_active == 1) return;
+    if (ns_active == 1 || !a.arrivals) return;  // without counters the caller merges later
     __shared__ int last;
     const int64_t unit = ((int64_t)b * a.n_layers + li) * a.pv.kv_heads + g;
     __syncthreads();
@@ -85,55 +71,10 @@ __device__ __forceinline__ void finish_split(const AttendArgs &a, float *obuf, f
     __syncthreads();
     if (!last) return;
     if (tid == 0) a.arrivals[unit] = 0;
-    // warp w merges heads w, w + 4, ...: the (max, sum) pairs give each split's weight, then
-    // every lane sums D / 32 output dims over the splits, eight loads in flight
-    constexpr int E = D / 32;
-    float *wq = obuf + warp * kMaxSplits;
-    for (int h = warp; h < G; h += kAttendThreads / 32) {
-        const float2 *ml = reinterpret_cast<const float2 *>(a.part_ml) + pbase + (int64_t)h * a.n_splits;
-        const float *po = a.part_o + (pbase + (int64_t)h * a.n_splits) * D + lane * E;
-        float mv[kMaxSplits / 32], lv[kMaxSplits / 32], M = -INFINITY;
-#pragma unroll
-        for (int k = 0; k < kMaxSplits / 32; ++k) {
-            const int q = lane + 32 * k;
-            const float2 x = q < ns_active ? __ldcg(ml + q) : make_float2(-INFINITY, 0.f);
-            mv[k] = x.x;
-            lv[k] = x.y;
-            M = fmaxf(M, x.x);
-        }
-        M = warp_max(M);
-        const float ref = M == -INFINITY ? 0.f : M;
-        float W = 0.f;
-#pragma unroll
-        for (int k = 0; k < kMaxSplits / 32; ++k) {
-            const float f = exp2f(mv[k] - ref);
-            W += lv[k] * f;
-            wq[lane + 32 * k] = f;
-        }
-        W = warp_sum(W);
-        __syncwarp();
-        float acc[E];
-#pragma unroll
-        for (int e = 0; e < E; ++e) acc[e] = 0.f;
-        for (int q0 = 0; q0 < ns_active; q0 += 8) {
-            float ov[8][E];
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-#pragma unroll
-                for (int e = 0; e < E; ++e) ov[j][e] = q0 + j < ns_active ? __ldcg(po + (int64_t)(q0 + j) * D + e) : 0.f;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const float f = q0 + j < ns_active ? wq[q0 + j] : 0.f;
-#pragma unroll
-                for (int e = 0; e < E; ++e) acc[e] += f * ov[j][e];
-            }
-        }
-#pragma unroll
-        for (int e = 0; e < E; ++e)
-            store_as(static_cast<T *>(a.out) + (hrow + h) * D + lane * E + e, W > 0.f ? acc[e] / W : 0.f);
-        if (lane == 0) a.lse2[lrow + h] = W > 0.f ? M + log2f(W) : -INFINITY;
-        __syncwarp();
-    }
+    for (int h = warp; h < G; h += kAttendThreads / 32)
+        merge_head<D / 32>(reinterpret_cast<const float2 *>(a.part_ml) + pbase + (int64_t)h * a.n_splits,
+                           a.part_o + (pbase + (int64_t)h * a.n_splits) * D, ns_active, obuf + warp * kMaxSplits,
+                           static_cast<T *>(a.out) + (hrow + h) * D, a.lse2 + lrow + h);
 }
 
 // A sequence without slots: output 0, log-sum-exp -inf (written by its first split's CTA).

@@ -79,7 +79,8 @@ struct TcArgs {
     float *part_ml, *part_o;
     __nv_bfloat16 *out;         // [n_layers][batch][H][128]
     float *lse2;                // [batch][sc_layers][H]
-    int32_t *arrivals;          // [batch][n_layers][kv_heads], zero on entry, left zero
+    int32_t *arrivals;          // [batch][n_layers][kv_heads], zero on entry, left zero; or null: units of
+                                // several chunks leave their partials for the caller to merge
     const int32_t *pos;         // [rows][cap], -1 at dead slots; null: every slot below len is live
     int32_t rows_per_seq;
     int32_t sc_layers, sc_layer0;  // local layer li is layer sc_layer0 + li of logits / lse2
@@ -751,13 +752,16 @@ __global__ void __launch_bounds__(kThreads, 2)
             }
             // The last CTA of (sequence, layer, kv head) to finish merges every CTA's
             // partial into the output and the per-head log-sum-exp.  Arrival counter
-            // only: no CTA waits for another.
-            softmax_bar();
+            // only: no CTA waits for another.  (Without counters the caller's next kernel
+            // merges the partials.)
             int *last_flag = reinterpret_cast<int *>(sm + kOffMisc + 8);
             const int64_t unit = ((int64_t)b * a.n_layers + li) * a.kv_heads + g;
-            if (tid == 0) *last_flag = arrive_acq_rel(a.arrivals + unit) == nc_unit - 1 ? 1 : 0;
-            softmax_bar();
-            if (*last_flag && ok) {
+            if (a.arrivals) {
+                softmax_bar();
+                if (tid == 0) *last_flag = arrive_acq_rel(a.arrivals + unit) == nc_unit - 1 ? 1 : 0;
+                softmax_bar();
+            }
+            if (a.arrivals && *last_flag && ok) {
                 // partial weights [G][n_splits] in the P buffers (every MMA has completed)
                 float *wq = reinterpret_cast<float *>(sm + kOffP);
                 // warp w merges heads w, w + 4: (1) the partials' (max, sum) pairs give the

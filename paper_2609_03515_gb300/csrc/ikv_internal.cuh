@@ -116,7 +116,8 @@ struct AttendArgs {
     // kernels of attend.cu: results of units of one split, and of the last CTA to arrive at the others
     void *out;                  // [n_layers][batch][H][D] (dtype)
     float *lse2;                // [batch][sc_layers][H]
-    int32_t *arrivals;          // [batch][n_layers][kv_heads], zero on entry, left zero
+    int32_t *arrivals;          // [batch][n_layers][kv_heads], zero on entry, left zero; null: partials are
+                                // left for the caller to merge
     // tensor-core kernel: the launch may set up and start its K/V stream before the
     // programmatic-dependency wait (see TcArgs::early)
     int32_t early;
@@ -170,7 +171,27 @@ struct ScoreArgs {
     uint32_t *sel_cnt;             // [rows][nblk] each block's live slots
 };
 
+// One layer's score pass and split merge (the workspace entry point): score.cu
+struct ScoreOneArgs {
+    const int32_t *len, *start;     // [batch]; start may be null
+    int32_t batch, q_heads, kv_heads, rows_per_seq, cap, head_dim, bf16;
+    const float *logits;            // [batch][H][lstride], or group sums [batch][kv_heads][lstride]
+    int32_t lstride, gsum;
+    const float *lse2;              // [batch][H]: of sequences the attention covered with one chunk
+    // the attention's partition: tiles of `tile` slots from the one holding start (0: slots),
+    // split_tokens a chunk, `passes` chunks a partial; partials as in AttendArgs
+    int32_t tile, split_tokens, passes, n_splits;
+    const float *part_ml, *part_o;
+    void *out;                      // [batch][H][D] (dtype)
+    float alpha;
+    float *score, *ema;             // [rows][cap] or null
+    int32_t vec;                    // their rows lie on 16-byte boundaries
+    int32_t row_ctas, tok_ctas;     // CTAs of a row, of all rows; set by the launcher
+};
+cudaError_t launch_score_one(const ScoreOneArgs &a, int32_t max_len, int sms, cudaStream_t st);
+
 // tensor-core attention (bf16, head_dim 128): attend_tc.cu
+constexpr int kTcTile = 128;
 bool tc_supported(int dtype, int head_dim, int group, int page_size);
 int tc_max_split_tokens();
 // the tensor-core kernel also merges its splits (last CTA of each unit)

@@ -17,6 +17,7 @@
 // so its first pass only stores s_l and per-block partial entropies, and
 // entropy_fold_kernel applies the weights and folds.
 #include "ikv_internal.cuh"
+#include "merge.cuh"
 #include "select_row.cuh"
 
 namespace ikv {
@@ -61,11 +62,9 @@ __device__ __forceinline__ float ld_cluster_f32(const float *p, int rank) {
     return v;
 }
 
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
+// A head's log-sum-exp as the scores subtract it: -inf (no live slot) becomes +inf, so that
+// its -inf logits give probability 0 and not NaN.
+__device__ __forceinline__ float finite_lse(float x) { return x == -INFINITY ? INFINITY : x; }
 
 // The pass is latency bound: every head of a batch of 32 / V is loaded before any
 // is used, the per-head log-sum-exp travels by shuffle, and the utility is fetched
@@ -132,7 +131,7 @@ __global__ void __launch_bounds__(kScoreThreads, 4) score_kernel(const ScoreArgs
         if (a.gsum) zp = a.logits + (((int64_t)b * a.n_layers + li) * a.kv_heads + g0) * (int64_t)a.lstride + il;
         for (int hb = 0; hb < nrows; hb += kHB) {
             const int nb = min(kHB, nrows - hb);
-            const float lse_lane = !a.gsum && lane < nb ? ll[hb + lane] : 0.f;
+            const float lse_lane = !a.gsum && lane < nb ? finite_lse(ll[hb + lane]) : 0.f;
             VT z[kHB];
 #pragma unroll
             for (int j = 0; j < kHB; ++j) {
@@ -321,6 +320,184 @@ __global__ void __launch_bounds__(kScoreThreads, 4) score_kernel(const ScoreArgs
     } else {
         select_row<kScoreThreads>(r, a.cap, a.ema, a.len, a.rows_per_seq, a.budget, a.sel_pos, a.keep, a.keep_len,
                                   a.df);
+    }
+}
+
+// Eq. 1 score of a single layer and Eq. 4 on the utility (either may be absent), after the
+// attention of the workspace entry point; also the merge of that attention's split partials,
+// which costs the attention kernel a memset of its counters and a chain of arrival, reload and
+// store at its end, and here runs beside the scores.
+//
+// The first a.tok_ctas CTAs take a row's tokens, 32 V (8 / HS) at a time, the others eight
+// heads' merges.  HS = 8: the CTA's warps share the row's heads between them (head h to warp
+// h % 8), so a small launch spreads over every SM and a lane has a few loads; HS = 1: each
+// warp has its own tokens and walks all heads, and a CTA takes several blocks of its row.  A
+// head's log-sum-exp comes from the attention (one chunk) or from its chunks' (max, sum)
+// pairs.  A small launch is a chain of latencies, so everything whose address does not hang
+// on the row's length is loaded before the length arrives.  Measured against score_kernel,
+// whose CTA gives each of its eight warps a layer and had one to give: 128 rows of 7 heads x
+// 14k tokens (51 MB of logits, 22 MB of score and utility) 59 -> 21 us.  One layer of 32
+// heads x 3277 tokens with the attention before it, in a chain of 32 such calls:
+// 16.4 -> 11.7 us a layer, with the memset gone and the two launches overlapping (PDL).
+constexpr int kOneThreads = 256;
+constexpr int kOnePairs = 4;  // heads whose (max, sum) pairs a warp has in flight
+template <int V, int HS>
+__global__ void __launch_bounds__(kOneThreads, HS == 8 ? 4 : 3) score_one_kernel(const ScoreOneArgs a) {
+    using VT = typename VecF<V>::T;
+    pdl_wait();
+    constexpr int kWarps = kOneThreads / 32;
+    constexpr int kTok = 32 * V * (kWarps / HS);  // tokens per block
+    constexpr int kHB = HS == 8 ? 4 : 8;          // heads loaded before any is used
+    extern __shared__ float lse_s[];              // [heads of a row]
+    __shared__ float part[HS == 8 ? kWarps : 1][32 * V];
+    __shared__ float wq[kWarps][kMaxSplits];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // chunks that hold partials of sequence b (1: the attention finished the sequence itself)
+    auto chunks = [&](int L, int S) {
+        if (L <= 0) return 1;
+        const int n = a.tile > 0 ? (S + L + a.tile - 1) / a.tile - S / a.tile : L;  // tiles or tokens
+        const int per = a.tile > 0 ? a.split_tokens / a.tile : a.split_tokens;
+        return min(((n + per - 1) / per + a.passes - 1) / a.passes, a.n_splits);
+    };
+    if ((int)blockIdx.x >= a.tok_ctas) {
+        const int hh = ((int)blockIdx.x - a.tok_ctas) * kWarps + warp;
+        if (hh >= a.batch * a.q_heads) return;
+        const int b = hh / a.q_heads;
+        const int n = chunks(a.len[b], a.start ? a.start[b] : 0);
+        if (n <= 1) return;
+        const float2 *ml = reinterpret_cast<const float2 *>(a.part_ml) + (int64_t)hh * a.n_splits;
+        const float *po = a.part_o + (int64_t)hh * a.n_splits * a.head_dim;
+        if (a.bf16) {
+            __nv_bfloat16 *o = static_cast<__nv_bfloat16 *>(a.out) + (int64_t)hh * a.head_dim;
+            if (a.head_dim == 128) merge_head<4>(ml, po, n, wq[warp], o, (float *)nullptr);
+            else merge_head<2>(ml, po, n, wq[warp], o, (float *)nullptr);
+        } else {
+            float *o = static_cast<float *>(a.out) + (int64_t)hh * a.head_dim;
+            if (a.head_dim == 128) merge_head<4>(ml, po, n, wq[warp], o, (float *)nullptr);
+            else merge_head<2>(ml, po, n, wq[warp], o, (float *)nullptr);
+        }
+        return;
+    }
+    const int r = blockIdx.x / a.row_ctas;
+    int blk = blockIdx.x % a.row_ctas;  // the CTA takes blocks blk, blk + row_ctas, ...
+    const int b = r / a.rows_per_seq;
+    const int L = a.len[b];
+    const int S = a.start ? a.start[b] : 0;
+    int h0 = 0, nh = a.q_heads;  // the row's heads
+    if (a.rows_per_seq > 1) {
+        nh = a.q_heads / a.kv_heads;
+        h0 = (r % a.rows_per_seq) * nh;
+    }
+    const float inv = 1.f / (float)nh;
+    // with group sums a row per KV head holds its query group's summed probabilities
+    const int G = a.q_heads / a.kv_heads;
+    const int rows = a.gsum ? nh / G : nh;
+    const int hfirst = HS == 8 ? warp : 0;
+    const int lane_tok = HS == 8 ? lane * V : (warp * 32 + lane) * V;  // the lane's first token of a block
+    const float *zp = a.logits + ((int64_t)b * (a.gsum ? a.kv_heads : a.q_heads) + (a.gsum ? h0 / G : h0)) * (int64_t)a.lstride +
+                      lane_tok;
+    VT z[kHB];
+    auto load = [&](int i0, int j0) {  // logits rows are padded to lstride, a multiple of 128
+#pragma unroll
+        for (int j = 0; j < kHB; ++j) {
+            const int h = hfirst + (j0 + j) * HS;
+            if (i0 + lane_tok < a.lstride && h < rows) z[j] = __ldg(reinterpret_cast<const VT *>(zp + (int64_t)h * a.lstride + i0));
+        }
+    };
+    load(blk * kTok, 0);
+    float m0 = 0.f;  // HS = 8: the utility of the token this thread folds
+    if (HS == 8 && a.ema && threadIdx.x < 32 * V && blk * kTok + (int)threadIdx.x < a.cap)
+        m0 = a.ema[(int64_t)r * a.cap + blk * kTok + threadIdx.x];
+    if (!a.gsum) {
+        const int64_t base = (int64_t)b * a.q_heads + h0;
+        const float2 *pairs = reinterpret_cast<const float2 *>(a.part_ml) + base * a.n_splits;
+        if (a.n_splits <= 1) {
+            for (int h = threadIdx.x; h < nh; h += kOneThreads) lse_s[h] = finite_lse(a.lse2[base + h]);
+        } else {
+            for (int hb = warp; hb < nh; hb += kOnePairs * kWarps) {
+                float2 x[kOnePairs];
+                float one[kOnePairs];  // the log-sum-exp if the attention wrote it
+#pragma unroll
+                for (int j = 0; j < kOnePairs; ++j) {
+                    const int h = hb + j * kWarps;
+                    const bool in = h < nh && lane < a.n_splits;
+                    x[j] = in ? __ldcg(pairs + (int64_t)h * a.n_splits + lane) : make_float2(-INFINITY, 0.f);
+                    one[j] = h < nh ? __ldcg(a.lse2 + base + h) : 0.f;
+                }
+                const int n = chunks(L, S);
+#pragma unroll
+                for (int j = 0; j < kOnePairs; ++j) {
+                    const int h = hb + j * kWarps;  // (past nh: nothing loaded, nothing stored)
+                    float M = lane < n ? x[j].x : -INFINITY;
+                    for (int c = 32 + lane; h < nh && c < n; c += 32) M = fmaxf(M, __ldcg(&pairs[(int64_t)h * a.n_splits + c].x));
+                    M = warp_max(M);
+                    const float ref = M == -INFINITY ? 0.f : M;
+                    float W = lane < n ? x[j].y * exp2f(x[j].x - ref) : 0.f;
+                    for (int c = 32 + lane; h < nh && c < n; c += 32) {
+                        const float2 y = __ldcg(pairs + (int64_t)h * a.n_splits + c);
+                        W += y.y * exp2f(y.x - ref);
+                    }
+                    W = warp_sum(W);
+                    if (lane == 0 && h < nh) lse_s[h] = finite_lse(n <= 1 ? one[j] : W > 0.f ? M + log2f(W) : -INFINITY);
+                }
+            }
+        }
+        __syncthreads();
+    }
+    for (bool first = true; blk * kTok < L; blk += a.row_ctas, first = false) {
+        const int i0 = blk * kTok, il = i0 + lane_tok;
+        if (!first) load(i0, 0);
+        const int64_t at = (int64_t)r * a.cap + il;
+        VT m4{};
+        const bool whole = HS == 1 && V == 4 && a.vec && il + V <= L;
+        if (whole && a.ema) m4 = *reinterpret_cast<const VT *>(a.ema + at);
+        float acc[V];
+#pragma unroll
+        for (int v = 0; v < V; ++v) acc[v] = 0.f;
+        for (int j0 = 0; hfirst + j0 * HS < rows; j0 += kHB) {
+            if (j0) load(i0, j0);
+#pragma unroll
+            for (int j = 0; j < kHB; ++j) {
+                const int h = hfirst + (j0 + j) * HS;
+                if (il < L && h < rows) {
+                    const float lj = a.gsum ? 0.f : lse_s[h];
+#pragma unroll
+                    for (int v = 0; v < V; ++v) acc[v] += a.gsum ? vget(z[j], v) : exp2f(vget(z[j], v) - lj);
+                }
+            }
+        }
+        if (HS == 1) {
+            if (whole) {
+                VT s4, e4;
+#pragma unroll
+                for (int v = 0; v < V; ++v) {
+                    reinterpret_cast<float *>(&s4)[v] = acc[v] * inv;
+                    reinterpret_cast<float *>(&e4)[v] = a.alpha * vget(m4, v) + (1.f - a.alpha) * (acc[v] * inv);
+                }
+                if (a.score) *reinterpret_cast<VT *>(a.score + at) = s4;
+                if (a.ema) *reinterpret_cast<VT *>(a.ema + at) = e4;
+            } else {
+#pragma unroll
+                for (int v = 0; v < V; ++v)
+                    if (il + v < L) {
+                        if (a.score) a.score[at + v] = acc[v] * inv;
+                        if (a.ema) a.ema[at + v] = a.alpha * a.ema[at + v] + (1.f - a.alpha) * (acc[v] * inv);
+                    }
+            }
+        } else {  // one block a CTA
+#pragma unroll
+            for (int v = 0; v < V; ++v) part[HS == 8 ? warp : 0][lane * V + v] = acc[v];
+            __syncthreads();
+            const int t = threadIdx.x;
+            if (t < 32 * V && i0 + t < L) {
+                float s = 0.f;
+#pragma unroll
+                for (int w = 0; w < kWarps; ++w) s += part[HS == 8 ? w : 0][t];
+                s *= inv;
+                if (a.score) a.score[(int64_t)r * a.cap + i0 + t] = s;
+                if (a.ema) a.ema[(int64_t)r * a.cap + i0 + t] = a.alpha * m0 + (1.f - a.alpha) * s;
+            }
+        }
     }
 }
 
@@ -522,6 +699,35 @@ cudaError_t launch_score_ema(const ScoreArgs &a, int32_t max_len, int sms, cudaS
     if (e != cudaSuccess) return e;
     note_launch();
     return cudaGetLastError();
+}
+
+template <int V, int HS>
+static cudaError_t launch_one(ScoreOneArgs a, int32_t max_len, int64_t rows, int sms, cudaStream_t st) {
+    constexpr int tok = 32 * V * (kOneThreads / 32 / HS);
+    const int nblk = (max_len + tok - 1) / tok;
+    a.row_ctas = nblk;
+    if (HS == 1) {  // about one wave, the blocks of a row dealt evenly to its CTAs
+        const int64_t want = ((int64_t)sms * 3 + rows - 1) / (rows > 0 ? rows : 1);
+        const int per = (int)((nblk + want - 1) / want);
+        a.row_ctas = (nblk + per - 1) / per;
+    }
+    a.tok_ctas = (int)(rows * a.row_ctas);
+    const int merge = a.n_splits > 1 ? (a.batch * a.q_heads + 7) / 8 : 0;
+    const int nh = a.rows_per_seq > 1 ? a.q_heads / a.kv_heads : a.q_heads;
+    cudaError_t e = launch_k(score_one_kernel<V, HS>, dim3((unsigned)(a.tok_ctas + merge)), dim3(kOneThreads),
+                             sizeof(float) * nh, st, a);
+    note_launch();
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+cudaError_t launch_score_one(const ScoreOneArgs &a, int32_t max_len, int sms, cudaStream_t st) {
+    const int64_t rows = a.score || a.ema ? (int64_t)a.batch * a.rows_per_seq : 0;  // 0: the merge alone
+    if (max_len <= 0 || (rows == 0 && a.n_splits <= 1)) return cudaSuccess;
+    // the widest form that gives every SM two CTAs
+    auto ctas = [&](int tok) { return rows * ((max_len + tok - 1) / tok); };
+    if (ctas(1024) >= 2 * sms) return launch_one<4, 1>(a, max_len, rows, sms, st);
+    if (ctas(128) >= 2 * sms) return launch_one<4, 8>(a, max_len, rows, sms, st);
+    return launch_one<1, 8>(a, max_len, rows, sms, st);
 }
 
 cudaError_t launch_entropy_fold(const ScoreArgs &a, int32_t max_len, cudaStream_t st) {
