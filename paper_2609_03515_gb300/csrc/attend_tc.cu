@@ -182,15 +182,6 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
         : "memory");
 }
 
-__device__ __forceinline__ void bulk_prefetch_l2(const void *p, uint32_t bytes) {
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap *map, int x, int y) {
-    asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global [%0, {%1, %2}];" ::"l"(reinterpret_cast<uint64_t>(map)),
-                 "r"(x), "r"(y)
-                 : "memory");
-}
-
 // smem matrix descriptor, 128-byte swizzle (sm_100 family, version 1)
 __device__ __forceinline__ uint64_t sdesc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
     uint64_t d = (uint64_t)((saddr >> 4) & 0x3FFFu);
@@ -363,7 +354,10 @@ __global__ void __launch_bounds__(kThreads, 2)
     // Prologue.  The producer lane initialises the barriers and starts the K/V stream at
     // once (every load up to the ring's depth); the TMEM allocation and P zeroing below
     // overlap the loads' latency.  An early CTA does all of this before the dependency
-    // wait, so it overlaps the previous kernel's tail.
+    // wait, so it overlaps the previous kernel's tail.  (It asks for no more than the ring
+    // holds: L2 prefetches of its other tiles cost more than they saved.  Steps of 32 layers
+    // driven one by one, us with / without them: 8 units of 27 tiles a layer 265 / 249, 8 of
+    // 103 456 / 426, 16 of 103 in 16-token pages 966 / 800; 16 layers, 128 of 27 771 / 645.)
     if (warp == 4 && lane == 0) {
         for (int i = 0; i < kNst; ++i) {
             mbar_init(full(i), 1);
@@ -382,24 +376,6 @@ __global__ void __launch_bounds__(kThreads, 2)
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         while (ld_J < kNst && ld_p < np) issue_next();
-        // an early CTA also pulls the rest of its tiles, and its q rows, into L2 while it
-        // waits, so the loads it can only issue later find them there (a prefetch cannot
-        // return stale data: L2 is where writes land)
-        if (early) {
-            for (int p = ld_p, j = ld_j; p < np;) {
-                const CUtensorMap *tm = j < chunk_n(p) ? &tmK : &tmV;
-                for (int bx = 0; bx < boxes; ++bx) {
-                    const int row = box_row(p, j, bx);
-                    tma_prefetch_2d(tm, 0, row);
-                    tma_prefetch_2d(tm, 64, row);
-                }
-                if (++j == 2 * chunk_n(p)) {
-                    ++p;
-                    j = 0;
-                }
-            }
-            bulk_prefetch_l2(a.q + (((int64_t)li * a.batch + b) * a.q_heads + (int64_t)g * G) * kD, G * kD * 2);
-        }
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
