@@ -385,9 +385,9 @@ ikv_status run_score(const ikv_shape *s, const ikv_cache *c, int32_t n_layers, c
         sa.n_elig = n_elig - k0 < kMaxLayersPerScorePass ? n_elig - k0 : kMaxLayersPerScorePass;
         sa.k0 = k0;
         for (int k = 0; k < sa.n_elig; ++k) sa.elig[k] = elig[k0 + k];
-        // the last pass of an Eq. 1 / VNorm fold also selects, unless the rows may be long
-        // (step 1 after a long prefill): the general selection then runs in the 1024-thread
-        // select kernel rather than on the score pass's last 256-thread CTA per row
+        // the last pass of an Eq. 1 / VNorm fold also selects, unless the rows may be so long
+        // (step 1 after a long prefill) that their keys would cost the pass its four CTAs an SM:
+        // the selection then runs in its own kernel, a cluster of CTAs per row
         if (fuse && ema && !store_only && scorer != IKV_SCORE_ENTROPY && k0 + sa.n_elig == n_elig &&
             max_len <= kFusedSelectMaxLen) {
             sa.fuse_select = 1;
@@ -399,6 +399,7 @@ ikv_status run_score(const ikv_shape *s, const ikv_cache *c, int32_t n_layers, c
             sa.df = fuse->df;
             sa.sel_best = fuse->best;
             sa.sel_cnt = fuse->cnt;
+            sa.sel_keys = max_len;
             if (fused) *fused = true;
         }
         IKV_TRY_CUDA(launch_score_ema(sa, max_len, sm_count(), st), "score launch");
@@ -570,7 +571,7 @@ ikv_status ikv_select_budget(int32_t rows, int32_t cap, const float *util, const
         return fail(IKV_ERR_ARG, "util/len/budget/keep/keep_len is NULL");
     // max_holes 0: the kernel never writes pos here
     IKV_TRY_CUDA(launch_select(rows, cap, util, len, rows_per_seq_, budget, const_cast<int32_t *>(pos), keep,
-                               keep_len, DeferArgs{0, cap, nullptr}, stream),
+                               keep_len, DeferArgs{0, cap, nullptr}, sm_count(), stream),
                  "select launch");
     return IKV_OK;
 }
@@ -780,7 +781,7 @@ static ikv_status evict_impl(const ikv_shape *shape, const ikv_params *p, ikv_ca
     if (!selected)
         IKV_TRY_CUDA(launch_select(R, cap, ema, cache->len, rows_per_seq(shape), p->budget,
                                    cache->dead_slots ? cache->pos : nullptr, at<int32_t>(ws, w.keep),
-                                   at<int32_t>(ws, w.keep_len), DeferArgs{p->max_holes, cap, cache->start}, stream),
+                                   at<int32_t>(ws, w.keep_len), DeferArgs{p->max_holes, cap, cache->start}, sm_count(), stream),
                      "select launch");
     ikv_status e;
     if (tm && (e = record(tm->select_end, stream))) return e;
@@ -832,7 +833,7 @@ static ikv_status trace_before(const ikv_shape *shape, const ikv_params *p, cons
     const int32_t R = shape->batch * rows_per_seq(shape);
     IKV_TRY_CUDA(launch_select(R, cx.cap, at<float>(ws, cx.w.raw), cache->len, rows_per_seq(shape), p->budget,
                                cache->dead_slots ? cache->pos : nullptr, at<int32_t>(ws, cx.w.keep_raw),
-                               at<int32_t>(ws, cx.w.n_raw), DeferArgs{0, cx.cap, nullptr}, stream),
+                               at<int32_t>(ws, cx.w.n_raw), DeferArgs{0, cx.cap, nullptr}, sm_count(), stream),
                  "trace select launch");
     IKV_TRY_CUDA(launch_trace_gather(trace_args(shape, p, cache, ws, cx), cx.L1, stream), "trace gather launch");
     return IKV_OK;
@@ -888,7 +889,7 @@ static ikv_status layer_evict(const ikv_shape *shape, const ikv_params *p, ikv_c
     const int32_t K = shape->layers;
     IKV_TRY_CUDA(launch_select(shape->batch * K, cx.cap, at<float>(ws, cx.w.util), cache->len, K, p->budget, nullptr,
                                at<int32_t>(ws, cx.w.keep), at<int32_t>(ws, cx.w.keep_len), DeferArgs{0, cx.cap, nullptr},
-                               stream),
+                               sm_count(), stream),
                  "select launch");
     return compact_impl(shape, cache, at<int32_t>(ws, cx.w.keep), at<int32_t>(ws, cx.w.keep_len), nullptr,
                         p->compact_mode, at<int32_t>(ws, cx.w.moves), at<int32_t>(ws, cx.w.n_moves),

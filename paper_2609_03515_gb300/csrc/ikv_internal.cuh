@@ -14,7 +14,7 @@ constexpr int kAttendThreads = 128;
 constexpr int kMaxSplits = 128;    // split-K partitions per (seq, layer, kv head)
 constexpr int kSplitMergeTokens = 64;  // cost of merging a unit's splits, as tokens of its stream
 constexpr int kMaxLayersPerScorePass = 32;
-constexpr int kFusedSelectMaxLen = 16384;  // longest row bound for which the score pass also selects
+constexpr int kFusedSelectMaxLen = 12288;  // longest row bound for which the score pass also selects
 constexpr int kScoreLayersPerGroup = 8;   // eligible layers one score CTA folds (one warp each)
 constexpr int kMaxLayers = 512;
 
@@ -167,6 +167,7 @@ struct ScoreArgs {
     int32_t *sel_pos;           // pos when dead slots are in use, else null
     int32_t *keep, *keep_len;   // [rows][cap], [rows]
     DeferArgs df;
+    int32_t sel_keys;              // keys the selection keeps in shared memory
     unsigned long long *sel_best;  // [rows][nblk] each block's lowest (key, ~slot) among live slots
     uint32_t *sel_cnt;             // [rows][nblk] each block's live slots
 };
@@ -222,7 +223,7 @@ cudaError_t launch_ema_update(int32_t rows, int32_t cap, float *ema, const float
                               int32_t rows_per_seq, float alpha, int32_t max_len, cudaStream_t st);
 cudaError_t launch_select(int32_t rows, int32_t cap, const float *util, const int32_t *len, int32_t rows_per_seq,
                           const int32_t *budget, int32_t *pos, int32_t *keep, int32_t *keep_len, const DeferArgs &df,
-                          cudaStream_t st);
+                          int sms, cudaStream_t st);
 
 struct CompactArgs {
     void *k, *v;

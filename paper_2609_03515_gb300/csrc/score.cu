@@ -48,20 +48,6 @@ __device__ __forceinline__ float agg_factor(int n, int agg, float alpha) {
     return f;
 }
 
-// thread-block cluster: barrier over every thread of the cluster (release / acquire), and a
-// load from the shared memory of the cluster's CTA `rank` at the address of `p` in this one
-__device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ float ld_cluster_f32(const float *p, int rank) {
-    const uint32_t a = static_cast<uint32_t>(__cvta_generic_to_shared(p));
-    uint32_t ra;
-    float v;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(rank));
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(ra) : "memory");
-    return v;
-}
-
 // A head's log-sum-exp as the scores subtract it: -inf (no live slot) becomes +inf, so that
 // its -inf logits give probability 0 and not NaN.
 __device__ __forceinline__ float finite_lse(float x) { return x == -INFINITY ? INFINITY : x; }
@@ -77,7 +63,8 @@ __global__ void __launch_bounds__(kScoreThreads, 4) score_kernel(const ScoreArgs
     constexpr int kTok = 32 * V;   // tokens per CTA
     constexpr int kHB = 32 / V;    // heads per load batch (32 registers of loads)
     __shared__ __align__(16) float sl[kScoreWarps][kTok];
-    extern __shared__ float wsm[];  // VNorm: per warp, [row's kv heads][kTok] value-norm weights
+    // VNorm: per warp, [row's kv heads][kTok] value-norm weights; later the selection's keys
+    extern __shared__ float wsm[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int r = blockIdx.y;
     const int lg = blockIdx.z, n_lg = gridDim.z;  // this CTA's layer group, and how many there are
@@ -234,7 +221,7 @@ __global__ void __launch_bounds__(kScoreThreads, 4) score_kernel(const ScoreArgs
             constexpr int kMaxGroups = (kMaxLayersPerScorePass + kScoreWarps - 1) / kScoreWarps;
             float cq[kMaxGroups];
 #pragma unroll
-            for (int q = 1; q < kMaxGroups; ++q) cq[q] = q < n_lg ? ld_cluster_f32(&cpart[threadIdx.x], q) : 0.f;
+            for (int q = 1; q < kMaxGroups; ++q) cq[q] = q < n_lg ? ld_cluster(&cpart[threadIdx.x], q) : 0.f;
             cq[0] = c;
 #pragma unroll
             for (int q = 0; q < kMaxGroups; ++q)
@@ -318,8 +305,8 @@ __global__ void __launch_bounds__(kScoreThreads, 4) score_kernel(const ScoreArgs
             a.keep_len[r] = -1 - B;
         }
     } else {
-        select_row<kScoreThreads>(r, a.cap, a.ema, a.len, a.rows_per_seq, a.budget, a.sel_pos, a.keep, a.keep_len,
-                                  a.df);
+        select_row<kScoreThreads>(0, 1, r, a.cap, a.ema, a.len, a.rows_per_seq, a.budget, a.sel_pos, a.keep, a.keep_len,
+                                  a.df, reinterpret_cast<uint32_t *>(wsm), a.sel_keys);
     }
 }
 
@@ -650,6 +637,7 @@ template <int V, int SCORER>
 static cudaError_t launch_score_v(const ScoreArgs &a, dim3 grid, size_t reserve, cudaStream_t st) {
     size_t smem = SCORER == IKV_SCORE_VNORM ? vnorm_smem(a, V) : 0;
     if (smem < reserve) smem = reserve;
+    if (a.fuse_select && smem < sizeof(uint32_t) * (size_t)a.sel_keys) smem = sizeof(uint32_t) * (size_t)a.sel_keys;
     static bool limit_set = false;
     if (!limit_set) {
         cudaError_t e = cudaFuncSetAttribute(score_kernel<V, SCORER>, cudaFuncAttributeMaxDynamicSharedMemorySize,

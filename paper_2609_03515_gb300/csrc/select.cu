@@ -1,42 +1,89 @@
 // Budgeted selection: keep the B highest utilities of a row (Sec. 3: evict the
 // lowest m whenever the cache exceeds B).
 //
-// One 1024-thread CTA per utility row.  Utilities map to order-preserving
+// A row is shared by a cluster of up to eight 512-thread CTAs (a short one: one of 1024), which
+// load it once and keep its keys in shared memory.  Utilities map to order-preserving
 // 32-bit keys (sign-flipped IEEE bits; -0.0 folded onto +0.0; NaN -> 1, below
 // every number).  Dead slots (pos < 0, deferred compaction) get key 0: below
 // every live key, never kept, not counted against B.  General case: an
-// MSB-first radix select with 8-bit digits (four passes, warp-aggregated
-// shared-memory histograms) finds the exact B-th largest key theta and how
-// many theta-valued slots survive; one more pass writes the kept slots in
-// ascending order (two block scans per 1024-slot chunk), keeping the lowest
+// MSB-first radix select with 8-bit digits (four passes over the keys, shared-memory
+// histograms, summed across the cluster through distributed shared memory)
+// finds the exact B-th largest key theta; one more sweep writes the kept slots in
+// ascending order (per-warp ballots after one exchange of counts), keeping the lowest
 // slots among keys equal to theta.  Steady-state case, one live slot too many:
-// a single pass finds the slot to evict (lowest key, and among equal keys the
-// highest slot).  The result depends only on the fp32 values, so it is
+// the first sweep finds theta, the lowest key, itself (among equal keys the
+// highest slot goes).  The result depends only on the fp32 values, so it is
 // bit-exact against any correct sort.
+//
+// Bound by latency, not by the few hundred kilobytes it touches: a chain of barriers.  One
+// 1024-thread CTA a row, re-reading the row from L2 in every pass and scanning twice per 1024
+// slots, took 41 us for 32 rows of 16385 slots and 124 us for one of 32769; clusters of four and
+// eight take 18 and 17 us.  Rows below 6144 slots stay with one CTA: at 3.3k slots a cluster of
+// two took 8.5 us where one CTA took 6.4, its barriers costing more than its halves save.
 #include "select_row.cuh"
 
 namespace ikv {
 namespace {
 
-__global__ void __launch_bounds__(kSelThreads) select_kernel(int32_t cap, const float *__restrict__ util,
-                                                              const int32_t *__restrict__ len, int32_t rps,
-                                                              const int32_t *__restrict__ budget, int32_t *pos,
-                                                              int32_t *keep, int32_t *keep_len, DeferArgs df) {
+constexpr int kSelSlots = 3072;         // slots a CTA should have to be worth a cluster's barriers
+constexpr int kSelKeysMax = 48 * 1024;  // keys a CTA keeps in shared memory
+
+template <int NT>
+__global__ void __launch_bounds__(NT, NT == 1024 ? 1 : 2)
+    select_kernel(int32_t cap, const float *__restrict__ util, const int32_t *__restrict__ len, int32_t rps,
+                  const int32_t *__restrict__ budget, int32_t *pos, int32_t *keep, int32_t *keep_len, DeferArgs df,
+                  int32_t ctas, int32_t keys_cap) {
+    extern __shared__ uint32_t keys[];
     pdl_wait();
-    select_row(blockIdx.x, cap, util, len, rps, budget, pos, keep, keep_len, df);
+    select_row<NT>(blockIdx.x % ctas, ctas, blockIdx.x / ctas, cap, util, len, rps, budget, pos, keep, keep_len, df,
+                   keys, keys_cap);
 }
 
 }  // namespace
 
 cudaError_t launch_select(int32_t rows, int32_t cap, const float *util, const int32_t *len, int32_t rows_per_seq,
                           const int32_t *budget, int32_t *pos, int32_t *keep, int32_t *keep_len, const DeferArgs &df,
-                          cudaStream_t st) {
+                          int sms, cudaStream_t st) {
     if (rows <= 0) return cudaSuccess;
-    cudaError_t e = launch_k(select_kernel, dim3(rows), dim3(kSelThreads), 0, st, cap, util, len, rows_per_seq, budget,
-                             pos, keep, keep_len, df);
-    if (e != cudaSuccess) return e;
+    // the largest cluster that leaves every CTA some slots and the launch about a wave
+    int C = kSelMaxCtas;
+    while (C > 1 && ((int64_t)rows * C > 2 * sms || (int64_t)C * kSelSlots > cap)) C >>= 1;
+    const int seg = (cap + C - 1) / C;
+    const int32_t keys_cap = seg < kSelKeysMax ? seg : kSelKeysMax;
+    static bool limit_set = false;
+    if (!limit_set) {
+        const int bytes = kSelKeysMax * (int)sizeof(uint32_t);
+        cudaError_t e = cudaFuncSetAttribute(select_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(select_kernel<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        if (e != cudaSuccess) return e;
+        limit_set = true;
+    }
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)C * (unsigned)rows);
+    cfg.blockDim = dim3(C > 1 ? 512 : 1024);
+    cfg.dynamicSmemBytes = (size_t)keys_cap * sizeof(uint32_t);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    int n = 0;
+    if (C > 1) {
+        attr[n].id = cudaLaunchAttributeClusterDimension;
+        attr[n].val.clusterDim.x = C;
+        attr[n].val.clusterDim.y = 1;
+        attr[n].val.clusterDim.z = 1;
+        ++n;
+    }
+    if (pdl_enabled()) {
+        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n].val.programmaticStreamSerializationAllowed = 1;
+        ++n;
+    }
+    cfg.attrs = attr;
+    cfg.numAttrs = n;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, C > 1 ? select_kernel<512> : select_kernel<1024>, cap, util, len, rows_per_seq, budget, pos, keep, keep_len,
+                                       df, C, keys_cap);
     note_launch();
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace ikv

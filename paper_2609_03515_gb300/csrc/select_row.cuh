@@ -1,13 +1,11 @@
-// Budgeted selection of one utility row by one CTA; used by the select kernel and by
-// the score pass, whose last CTA of a row selects that row at once.  See select.cu.
+// Budgeted selection of one utility row, by a CTA or by a cluster of CTAs that share the row;
+// used by the select kernel and by the score pass, whose last CTA of a row selects that row
+// at once.  See select.cu.
 #pragma once
 #include "ikv_internal.cuh"
 
 namespace ikv {
 namespace {
-
-
-constexpr int kSelThreads = 1024;
 
 __device__ __forceinline__ uint32_t ord_key(float f) {
     uint32_t u = __float_as_uint(f);
@@ -17,207 +15,301 @@ __device__ __forceinline__ uint32_t ord_key(float f) {
 }
 constexpr uint32_t kDeadKey = 0u;  // dead slots: below every live key, never kept
 
-// exclusive scan of one value per thread across a block of NT threads; returns (exclusive, total)
-template <int NT>
-__device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t *warp_tot, uint32_t &total) {
-    constexpr int NW = NT / 32;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) warp_tot[warp] = x;
-    __syncthreads();
-    if (warp == 0) {
-        uint32_t t = lane < NW ? warp_tot[lane] : 0u;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, t, o);
-            if (lane >= o) t += y;
-        }
-        if (lane < NW) warp_tot[lane] = t;  // inclusive over warps
-    }
-    __syncthreads();
-    const uint32_t before = warp == 0 ? 0u : warp_tot[warp - 1];
-    total = warp_tot[NW - 1];
-    __syncthreads();
-    return before + x - v;
+// thread-block cluster: barrier over every thread of the cluster (release / acquire), and
+// loads from the shared memory of the cluster's CTA `rank` at the address of `p` in this one
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t cluster_addr(const void *p, int rank) {
+    uint32_t ra;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+                 : "=r"(ra)
+                 : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(p))), "r"(rank));
+    return ra;
+}
+__device__ __forceinline__ float ld_cluster(const float *p, int rank) {
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_addr(p, rank)) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint32_t ld_cluster(const uint32_t *p, int rank) {
+    uint32_t v;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(cluster_addr(p, rank)) : "memory");
+    return v;
+}
+__device__ __forceinline__ unsigned long long ld_cluster(const unsigned long long *p, int rank) {
+    unsigned long long v;
+    asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(cluster_addr(p, rank)) : "memory");
+    return v;
 }
 
-// The selection of utility row r by the calling CTA, which must have NT threads (256 or
-// 1024) and be entered by all of them.
-template <int NT = kSelThreads>
-__device__ __forceinline__ void select_row(int r, int32_t cap, const float *__restrict__ util,
+constexpr int kSelMaxCtas = 8;  // CTAs that share a row (portable cluster size)
+
+// The selection of utility row r by C CTAs of NT threads (C > 1: the cluster they form; this
+// one is its `rank`-th), entered by all of their threads.  CTA `rank` owns a contiguous C-th of
+// the row's slots and keeps their keys in keys[0, keys_cap) (shared memory) when they fit;
+// otherwise every sweep reads the row again, eight loads in flight a thread.
+template <int NT>
+__device__ __forceinline__ void select_row(int rank, int C, int r, int32_t cap, const float *__restrict__ util,
                                            const int32_t *__restrict__ len, int32_t rps,
                                            const int32_t *__restrict__ budget, int32_t *pos, int32_t *keep,
-                                           int32_t *keep_len, DeferArgs df) {
-    static_assert(NT == 256 || NT == 1024, "the digit scan needs 256 threads at least, whole warps");
+                                           int32_t *keep_len, DeferArgs df, uint32_t *keys, int keys_cap) {
+    static_assert(NT >= 256 && NT % 32 == 0, "the digit scan needs 256 threads at least, whole warps");
     constexpr int NW = NT / 32;
-    __shared__ uint32_t hist[256];
-    __shared__ uint32_t warp_tot[32];
-    __shared__ unsigned long long s_min[32];
-    __shared__ uint32_t s_digit, s_above, s_live;
+    constexpr int U = 8;  // keys a thread has in flight
+    __shared__ uint32_t hist[2][256];
+    __shared__ uint32_t warp_a[NW], warp_b[NW];
+    __shared__ unsigned long long warp_min[NW], s_min;
+    __shared__ uint32_t s_digit, s_above, s_live, s_gt, s_eq;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int L = len[r / rps];
-    int B = budget[r / rps];
-    if (B < 0) B = 0;
+    const int b = r / rps;
+    const int L = len[b];
+    const int B = max(budget[b], 0);
+    const int S = df.start ? df.start[b] : 0;
+    const int seg = (L + C - 1) / C;
+    const int lo = min(rank * seg, L), hi = min(lo + seg, L);
+    const bool cached = hi - lo <= keys_cap;
     const float *u = util + (int64_t)r * cap;
     int32_t *pr = pos ? pos + (int64_t)r * cap : nullptr;
     int32_t *kp = keep + (int64_t)r * cap;
-    auto live = [&](int i) { return !pr || pr[i] >= 0; };
-    auto key_at = [&](int i) { return live(i) ? ord_key(u[i]) : kDeadKey; };
-    // every slot i < L for which keep_if(i) holds, in ascending order (block scans)
-    auto write_kept = [&](auto keep_if) {
-        uint32_t run = 0u;
-        for (int base = 0; base < L; base += NT) {
-            const int i = base + tid;
-            const uint32_t kf = (i < L && keep_if(i)) ? 1u : 0u;
-            uint32_t tot;
-            const uint32_t at = block_excl_scan<NT>(kf, warp_tot, tot);
-            if (kf) kp[run + at] = i;
-            run += tot;
-        }
+    // (through L2: in the score pass other CTAs of the same launch wrote the utilities)
+    auto load_key = [&](int i) { return !pr || __ldcg(pr + i) >= 0 ? ord_key(__ldcg(u + i)) : kDeadKey; };
+    auto sync_all = [&]() {
+        if (C > 1) cluster_sync();
+        else __syncthreads();
     };
+    auto peer = [&](const auto *p, int c) { return C > 1 ? ld_cluster(p, c) : *p; };
 
-    // one pass: the live count and the lowest (key, highest slot) among the live slots,
+    // one sweep: the live count and the lowest (key, highest slot) among the live slots,
     // which is the victim whenever exactly one slot must go
-    if (tid == 0) s_live = 0u;
-    __syncthreads();
-    uint32_t c = 0u;
+    uint32_t cnt = 0u;
     unsigned long long best = ~0ull;
-    for (int i = tid; i < L; i += NT) {
-        if (!live(i)) continue;
-        ++c;
-        const unsigned long long v = ((unsigned long long)ord_key(u[i]) << 32) | (uint32_t)(~(uint32_t)i);
-        best = v < best ? v : best;
+    for (int i0 = lo + tid; i0 < hi; i0 += NT * U) {
+        float x[U];
+        int32_t p[U];
+#pragma unroll
+        for (int k = 0; k < U; ++k) {
+            const int i = i0 + k * NT;
+            x[k] = i < hi ? __ldcg(u + i) : 0.f;
+            p[k] = i < hi ? (pr ? __ldcg(pr + i) : 0) : -1;
+        }
+#pragma unroll
+        for (int k = 0; k < U; ++k) {
+            const int i = i0 + k * NT;
+            const uint32_t key = p[k] >= 0 ? ord_key(x[k]) : kDeadKey;
+            if (cached && i < hi) keys[i - lo] = key;
+            if (key == kDeadKey) continue;
+            ++cnt;
+            const unsigned long long v = ((unsigned long long)key << 32) | (uint32_t)(~(uint32_t)i);
+            best = v < best ? v : best;
+        }
     }
-    if (pr && c) atomicAdd(&s_live, c);
+    for (int i = tid; i < 512; i += NT) (&hist[0][0])[i] = 0u;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         const unsigned long long y = __shfl_xor_sync(0xffffffffu, best, o);
         best = y < best ? y : best;
+        cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
     }
-    if (lane == 0) s_min[warp] = best;
+    if (lane == 0) {
+        warp_min[warp] = best;
+        warp_a[warp] = cnt;
+    }
     __syncthreads();
     if (warp == 0) {
-        best = lane < NW ? s_min[lane] : ~0ull;
+        best = lane < NW ? warp_min[lane] : ~0ull;
+        cnt = lane < NW ? warp_a[lane] : 0u;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             const unsigned long long y = __shfl_xor_sync(0xffffffffu, best, o);
             best = y < best ? y : best;
+            cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
         }
-        if (lane == 0) s_min[0] = best;
+        if (lane == 0) {
+            s_min = best;
+            s_live = cnt;
+        }
     }
-    __syncthreads();
-    const int n_live = pr ? (int)s_live : L;
-
-    if (n_live <= B) {
-        if (n_live == L) {
-            for (int j = tid; j < L; j += NT) kp[j] = j;
-        } else {
-            write_kept([&](int i) { return live(i); });
-        }
-        if (tid == 0) keep_len[r] = n_live;
-        return;
-    }
-    if (B == 0) {
-        if (tid == 0) keep_len[r] = 0;
-        return;
-    }
-
-    if (n_live == B + 1) {
-        const int ev = (int)(~(uint32_t)(s_min[0] & 0xFFFFFFFFull));
-        const int b = r / rps;
-        if (pr && df.max_holes > 0 && L - B <= df.max_holes && (df.start ? df.start[b] : 0) + L < df.cap) {
-            // deferred compaction (the rule the compaction kernels apply): the victim is
-            // only marked dead, and keep_len < 0 tells compaction that nothing moves
-            if (tid == 0) {
-                pr[ev] = -1;
-                keep_len[r] = -1 - B;
-            }
-            return;
-        }
-        if (n_live == L) {
-            for (int j = tid; j < B; j += NT) kp[j] = j < ev ? j : j + 1;
-        } else {
-            write_kept([&](int i) { return i != ev && live(i); });
-        }
-        if (tid == 0) keep_len[r] = B;
-        return;
-    }
-
-    // general case: B < n_live - 1.  Dead slots carry the lowest key, and more than B
-    // live keys lie above it, so the B-th largest key theta is live and no dead slot
-    // is ever kept.
-    uint32_t prefix = 0u, mask = 0u, k = (uint32_t)B;
-    for (int pass = 0; pass < 4; ++pass) {
-        const int shift = 24 - 8 * pass;
-        for (int i = tid; i < 256; i += NT) hist[i] = 0u;
-        __syncthreads();
-        for (int base = 0; base < L; base += NT) {
-            const int i = base + tid;
-            uint32_t digit = 0xFFFFu;
-            if (i < L) {
-                const uint32_t key = key_at(i);
-                if ((key & mask) == prefix) digit = (key >> shift) & 0xFFu;
-            }
-            const uint32_t peers = __match_any_sync(0xffffffffu, digit);
-            if (digit != 0xFFFFu && lane == __ffs(peers) - 1) atomicAdd(&hist[digit], (uint32_t)__popc(peers));
-        }
-        __syncthreads();
-        // inclusive counts from the top digit down: thread t < 256 holds digit 255 - t
-        uint32_t v = 0u, x = 0u;
-        if (tid < 256) {
-            v = hist[255 - tid];
-            x = v;
+    sync_all();
+    // (remote loads are issued together, here and below: one round trip, not C)
+    int n_live = 0;
+    best = ~0ull;
+    {
+        uint32_t live[kSelMaxCtas];
+        unsigned long long low[kSelMaxCtas];
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-                if (lane >= o) x += y;
+        for (int c = 0; c < kSelMaxCtas; ++c) {
+            live[c] = c < C ? peer(&s_live, c) : 0u;
+            low[c] = c < C ? peer(&s_min, c) : ~0ull;
+        }
+#pragma unroll
+        for (int c = 0; c < kSelMaxCtas; ++c) {
+            n_live += (int)live[c];
+            best = low[c] < best ? low[c] : best;
+        }
+    }
+    const int kept = min(n_live, B);
+    if (n_live == B + 1 && B > 0 && pr && df.max_holes > 0 && L - B <= df.max_holes && S + L < df.cap) {
+        // deferred compaction (the rule the compaction kernels apply): the victim is
+        // only marked dead, and keep_len < 0 tells compaction that nothing moves
+        if (rank == 0 && tid == 0) {
+            pr[(int)(~(uint32_t)(best & 0xFFFFFFFFull))] = -1;
+            keep_len[r] = -1 - B;
+        }
+        if (C > 1) cluster_sync();  // a CTA may not leave while another reads its shared memory
+        return;
+    }
+    if (rank == 0 && tid == 0) keep_len[r] = kept;
+    if (n_live == L && kept >= L - 1) {  // no dead slot, at most one to go: no counting needed
+        const int ev = kept == L ? L : (int)(~(uint32_t)(best & 0xFFFFFFFFull));
+        if (kept > 0)
+            for (int i = lo + tid; i < hi; i += NT)
+                if (i != ev) kp[i < ev ? i : i - 1] = i;
+    } else if (kept > 0) {
+        // theta: the kept-th largest key.  Everything above it is kept, and of the slots equal
+        // to it the lowest ones.  All live slots kept: every live key is above the dead one.
+        // One slot too many: the lowest live key.
+        uint32_t theta = n_live <= B ? kDeadKey : (uint32_t)(best >> 32);
+        if (n_live > B + 1) {
+            // MSB-first radix select on the keys (dead slots carry the lowest one, and more than
+            // B live keys lie above it, so theta is live and no dead slot is ever kept).  The
+            // CTAs' histograms are summed by every CTA; two buffers, one barrier a digit.
+            uint32_t prefix = 0u, mask = 0u, k = (uint32_t)B;
+#pragma unroll 1
+            for (int pass = 0; pass < 4; ++pass) {
+                const int shift = 24 - 8 * pass;
+                uint32_t *h = hist[pass & 1];
+                for (int i0 = lo; i0 < hi; i0 += NT * U) {
+                    uint32_t d[U];
+#pragma unroll
+                    for (int q = 0; q < U; ++q) {
+                        const int i = i0 + q * NT + tid;
+                        const uint32_t key = i < hi ? (cached ? keys[i - lo] : load_key(i)) : 0u;
+                        d[q] = i < hi && (key & mask) == prefix ? (key >> shift) & 0xFFu : 0xFFFFu;
+                    }
+#pragma unroll
+                    for (int q = 0; q < U; ++q)
+                        if (d[q] != 0xFFFFu) atomicAdd(&h[d[q]], 1u);
+                }
+                sync_all();
+                // (every CTA is past its reads of the other buffer)
+                uint32_t v = 0u, x = 0u;
+                if (tid < 256) {
+                    hist[(pass & 1) ^ 1][tid] = 0u;
+                    // inclusive counts from the top digit down: thread t holds digit 255 - t
+                    uint32_t w[kSelMaxCtas];
+#pragma unroll
+                    for (int c = 0; c < kSelMaxCtas; ++c) w[c] = c < C ? peer(&h[255 - tid], c) : 0u;
+#pragma unroll
+                    for (int c = 0; c < kSelMaxCtas; ++c) v += w[c];
+                    x = v;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+                        if (lane >= o) x += y;
+                    }
+                    if (lane == 31) warp_a[warp] = x;
+                }
+                __syncthreads();
+                if (tid < 256) {
+                    uint32_t before = 0u;
+                    for (int w = 0; w < warp; ++w) before += warp_a[w];
+                    const uint32_t incl = before + x;
+                    if (incl - v < k && incl >= k) {  // exactly one digit satisfies this
+                        s_digit = 255u - (uint32_t)tid;
+                        s_above = incl - v;
+                    }
+                }
+                __syncthreads();
+                k -= s_above;
+                prefix |= s_digit << shift;
+                mask |= 0xFFu << shift;
             }
-            if (lane == 31) warp_tot[warp] = x;
+            theta = prefix;
+        }
+        // each warp owns a contiguous part of the segment: its counts above and at theta, the
+        // counts before it, then its kept slots in ascending order
+        const int part = (seg + NT - 1) / NT * 32;
+        const int wlo = min(lo + warp * part, hi), whi = min(wlo + part, hi);
+        uint32_t gt = 0u, eq = 0u;
+        for (int i0 = wlo + lane; i0 < whi; i0 += 32 * U) {
+            uint32_t key[U];
+#pragma unroll
+            for (int q = 0; q < U; ++q) {
+                const int i = i0 + 32 * q;
+                key[q] = i < whi ? (cached ? keys[i - lo] : load_key(i)) : kDeadKey;
+            }
+#pragma unroll
+            for (int q = 0; q < U; ++q) {
+                gt += key[q] > theta;
+                eq += key[q] == theta && key[q] != kDeadKey;
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            gt += __shfl_xor_sync(0xffffffffu, gt, o);
+            eq += __shfl_xor_sync(0xffffffffu, eq, o);
+        }
+        __syncthreads();  // warp_a is free
+        if (lane == 0) {
+            warp_a[warp] = gt;
+            warp_b[warp] = eq;
         }
         __syncthreads();
-        if (tid < 256) {
-            uint32_t before = 0u;
-            for (int w = 0; w < warp; ++w) before += warp_tot[w];
-            const uint32_t incl = before + x;
-            const uint32_t above = incl - v;
-            if (above < k && incl >= k) {  // exactly one digit satisfies this
-                s_digit = 255u - (uint32_t)tid;
-                s_above = above;
+        if (tid == 0) {
+            uint32_t g = 0u, e = 0u;
+            for (int w = 0; w < NW; ++w) {
+                const uint32_t wg = warp_a[w], we = warp_b[w];
+                warp_a[w] = g;
+                warp_b[w] = e;
+                g += wg;
+                e += we;
+            }
+            s_gt = g;
+            s_eq = e;
+        }
+        sync_all();
+        uint32_t gt_all = 0u, gt_run = warp_a[warp], eq_run = warp_b[warp];
+        {
+            uint32_t g[kSelMaxCtas], e[kSelMaxCtas];
+#pragma unroll
+            for (int c = 0; c < kSelMaxCtas; ++c) {
+                g[c] = c < C ? peer(&s_gt, c) : 0u;
+                e[c] = c < C ? peer(&s_eq, c) : 0u;
+            }
+#pragma unroll
+            for (int c = 0; c < kSelMaxCtas; ++c) {
+                gt_all += g[c];
+                if (c < rank) {
+                    gt_run += g[c];
+                    eq_run += e[c];
+                }
             }
         }
-        __syncthreads();
-        const uint32_t dsel = s_digit;
-        k -= s_above;
-        prefix |= dsel << shift;
-        mask |= 0xFFu << shift;
-        __syncthreads();
+        const uint32_t need_eq = (uint32_t)kept - gt_all;  // theta-valued slots that survive
+        const uint32_t below = (1u << lane) - 1u;
+        for (int i0 = wlo; i0 < whi; i0 += 32 * U) {
+            uint32_t key[U];
+#pragma unroll
+            for (int q = 0; q < U; ++q) {
+                const int i = i0 + 32 * q + lane;
+                key[q] = i < whi ? (cached ? keys[i - lo] : load_key(i)) : kDeadKey;
+            }
+#pragma unroll
+            for (int q = 0; q < U; ++q) {
+                if (i0 + 32 * q >= whi) break;
+                const bool is_gt = key[q] > theta, is_eq = key[q] == theta && key[q] != kDeadKey;
+                const uint32_t mg = __ballot_sync(0xffffffffu, is_gt), me = __ballot_sync(0xffffffffu, is_eq);
+                const uint32_t e = eq_run + __popc(me & below);
+                if (is_gt || (is_eq && e < need_eq))
+                    kp[gt_run + __popc(mg & below) + min(e, need_eq)] = i0 + 32 * q + lane;
+                gt_run += __popc(mg);
+                eq_run += __popc(me);
+            }
+        }
     }
-    const uint32_t theta = prefix;
-    const uint32_t need_eq = k;  // theta-valued slots that survive (lowest slots first)
-
-    uint32_t run_eq = 0u, run_keep = 0u;
-    for (int base = 0; base < L; base += NT) {
-        const int i = base + tid;
-        uint32_t key = 0u;
-        bool in = i < L;
-        if (in) key = key_at(i);
-        const uint32_t gt = (in && key > theta) ? 1u : 0u;
-        const uint32_t eq = (in && key == theta) ? 1u : 0u;
-        uint32_t eq_tot, kp_tot;
-        const uint32_t eq_rank = block_excl_scan<NT>(eq, warp_tot, eq_tot);
-        const uint32_t kf = (gt || (eq && run_eq + eq_rank < need_eq)) ? 1u : 0u;
-        const uint32_t at = block_excl_scan<NT>(kf, warp_tot, kp_tot);
-        if (kf) kp[run_keep + at] = i;
-        run_eq += eq_tot;
-        run_keep += kp_tot;
-    }
-    if (tid == 0) keep_len[r] = B;
+    if (C > 1) cluster_sync();  // a CTA may not leave while another reads its shared memory
 }
 
 }  // namespace

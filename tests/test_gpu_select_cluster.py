@@ -1,0 +1,78 @@
+"""Budgeted selection by clusters of CTAs: bit-exact against a stable sort at the sizes where
+the row's parts, the warps' parts and the keys in shared memory begin and end."""
+import pytest
+import torch
+
+from paper_2609_03515_gb300 import ikv
+
+pytestmark = pytest.mark.gpu
+
+
+def _want(util, pos, L, B):
+    """Slots kept, ascending: the B largest live utilities, lower slot first among equals."""
+    u = util[:L].clone()
+    u[u.isnan()] = -float("inf")
+    u = u + 0.0  # -0 == +0
+    live = torch.arange(L) if pos is None else torch.nonzero(pos[:L] >= 0).flatten()
+    nan = util[:L][live].isnan()
+    key = u[live]
+    # NaN below -inf: two stable sorts, least significant criterion first
+    order = torch.sort(key, descending=True, stable=True).indices
+    order = order[torch.sort(nan[order].int(), stable=True).indices]
+    return torch.sort(live[order[:min(B, live.numel())]]).values
+
+
+LENS = [0, 1, 2, 31, 33, 511, 512, 513, 1024, 1025, 4095, 4096, 4097, 8191, 8192, 8193, 16385]
+
+
+@pytest.mark.parametrize("rows,cap,lens", [
+    (17, 16448, LENS),             # clusters of eight, lengths that leave parts empty
+    (60, 3000, LENS[:10] + [3000]),  # clusters of two
+    (400, 1500, LENS[:10]),        # one CTA a row
+    (1, 70000, [70000]),           # one long row
+    (400, 70000, [60000, 33]),     # more keys than a CTA keeps in shared memory
+])
+@pytest.mark.parametrize("dead", [False, True])
+def test_select_cluster_bit_exact(rows, cap, lens, dead):
+    assert max(lens) <= cap
+    gen = torch.Generator().manual_seed(rows + cap)
+    ln = torch.tensor([lens[r % len(lens)] for r in range(rows)], dtype=torch.int32)
+    kinds = ["spread", "ties", "special", "low"]
+    util = torch.empty(rows, cap)
+    for r in range(min(rows, 40)):
+        kind = kinds[(r // len(lens) + r) % 4]
+        x = torch.randn(cap, generator=gen)
+        if kind == "spread":
+            x = torch.exp(4 * x - 9)
+        elif kind == "ties":
+            x = (x * 2).round() / 4
+        elif kind == "special":
+            x[torch.rand(cap, generator=gen) < 0.05] = float("nan")
+            x[torch.rand(cap, generator=gen) < 0.05] = float("inf")
+            x[torch.rand(cap, generator=gen) < 0.05] = -float("inf")
+            x[torch.rand(cap, generator=gen) < 0.2] = -0.0
+            x[torch.rand(cap, generator=gen) < 0.05] = torch.finfo(torch.float32).min
+        else:
+            x[:] = 0.0
+        util[r] = x
+    for r in range(40, rows):
+        util[r] = util[r % 40]
+    pos = torch.arange(cap, dtype=torch.int32).repeat(rows, 1)
+    if dead:
+        pos[torch.rand(pos.shape, generator=gen) < 0.1] = -1
+    live = [(int((pos[r, :int(ln[r])] >= 0).sum())) for r in range(rows)]
+    # none, one, a tenth, all but two, all but one, all, more than there are
+    pick = [lambda n: 0, lambda n: 1, lambda n: n // 10, lambda n: max(0, n - 2), lambda n: max(0, n - 1), lambda n: n,
+            lambda n: n + 5]
+    budget = torch.tensor([pick[(3 * r + r // len(lens)) % 7](live[r]) for r in range(rows)], dtype=torch.int32)
+    keep = torch.full((rows, cap), -9, dtype=torch.int32, device="cuda")
+    keep_len = torch.full((rows,), -9, dtype=torch.int32, device="cuda")
+    ikv.ikv_select_budget(rows, cap, util.cuda(), ln.cuda(), 1, budget.cuda(), pos.cuda() if dead else None, keep,
+                          keep_len)
+    torch.cuda.synchronize()
+    keep, keep_len = keep.cpu(), keep_len.cpu()
+    for r in list(range(min(rows, 120))) + [rows - 1]:
+        want = _want(util[r], pos[r] if dead else None, int(ln[r]), int(budget[r]))
+        assert int(keep_len[r]) == want.numel(), (r, int(ln[r]), int(budget[r]))
+        assert torch.equal(keep[r, :want.numel()].long(), want), (r, int(ln[r]), int(budget[r]))
+        assert torch.all(keep[r, want.numel():] == -9)
