@@ -31,6 +31,7 @@ constexpr int kCompThreads = 256;
 constexpr int kCompRows = 32;
 constexpr int kRelocateSlack = 128;  // slots a relocation to slot 0 must free
 constexpr int kCompStages = 4;
+constexpr int kCompRowSets = 8;      // tiles whose row numbers are kept: those in flight and the next
 
 __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
     const uint32_t s = static_cast<uint32_t>(__cvta_generic_to_shared(smem));
@@ -115,6 +116,7 @@ __device__ __forceinline__ void mark_dead_row(const CompactArgs &a, int r, int L
 // writes the new values, so no item sees them early.  Entered by every thread of the CTA.
 __device__ __forceinline__ void compact_stable_item(const CompactArgs &a, const int x, const int b,
                                                     unsigned char *cbuf, int *scratch) {
+    __shared__ uint32_t rows_s[kCompRowSets][2][kCompRows];
     const int tid = threadIdx.x;
     const int kvh = a.pv.kv_heads;
     const int nkv = a.layers * kvh;
@@ -176,40 +178,75 @@ __device__ __forceinline__ void compact_stable_item(const CompactArgs &a, const 
             unsigned char *vb = reinterpret_cast<unsigned char *>(a.v);
             // tile k covers rows [jb, jb + kCompRows) ascending (left) or descending (right)
             auto tile_base = [&](int tile) { return right ? j1 - (tile + 1) * kCompRows : j0 + tile * kCompRows; };
+            // Warp 0 finds each row's source and destination (pool rows; ~0 outside the tile's
+            // range) and leaves them in rows_s for the copies: the keep list two tiles and the
+            // block table one tile ahead of the tile being issued, so neither latency is waited
+            // for.  (Every thread finding its own rows, keep list then table then copy in turn:
+            // 237 us for the first compaction of 32 layers x 8 KV heads to 3277 of 32769 slots,
+            // 860 MB of reads and writes; this way 168 us, 0.75 of the copy rate.)
+            auto kept_slot = [&](int tile) {
+                const int j = tile_base(tile) + tid;
+                return tid < kCompRows && tile < n_tiles && j >= j0 && j < j1 ? kp[j] : -1;
+            };
+            auto find = [&](int tile, int slot, uint32_t &src, uint32_t &dst) {
+                src = slot < 0 ? ~0u : (uint32_t)a.pv.row_phys(b, l, g, S + slot);
+                dst = slot < 0 ? ~0u : (uint32_t)a.pv.row_phys(b, l, g, new_start + tile_base(tile) + tid);
+            };
+            auto put_rows = [&](int tile, uint32_t src, uint32_t dst) {
+                rows_s[tile % kCompRowSets][0][tid] = src;
+                rows_s[tile % kCompRowSets][1][tid] = dst;
+            };
+            constexpr int kAhead = kCompStages - 1;  // tiles whose copies are in flight
+            uint32_t src_next = ~0u, dst_next = ~0u;  // rows of tile `tile` + kAhead
+            int slot_next = -1;                       // kept slots of the one after it
+            if (tid < kCompRows) {
+                int slot[kAhead + 1];
+#pragma unroll
+                for (int i = 0; i <= kAhead; ++i) slot[i] = kept_slot(i);
+                slot_next = kept_slot(kAhead + 1);
+#pragma unroll
+                for (int i = 0; i <= kAhead; ++i) {
+                    find(i, slot[i], src_next, dst_next);
+                    if (i < kAhead) put_rows(i, src_next, dst_next);
+                }
+            }
+            __syncthreads();
             auto issue = [&](int tile) {
                 unsigned char *st = cbuf + (tile % kCompStages) * stageB;
-                const int jb = tile_base(tile);
                 for (int idx = tid; idx < kCompRows * CPR; idx += kCompThreads) {
                     const int jj = idx / CPR, c = idx % CPR;
-                    const int j = jb + jj;
-                    if (j >= j0 && j < j1) {
-                        const int64_t src = a.pv.row_phys(b, l, g, S + kp[j]);
-                        cp_async16(st + jj * rowB + c * 16, kb + src * rowB + c * 16);
-                        cp_async16(st + (kCompRows + jj) * rowB + c * 16, vb + src * rowB + c * 16);
+                    const uint32_t src = rows_s[tile % kCompRowSets][0][jj];
+                    if (src != ~0u) {
+                        const int64_t at = (int64_t)src * rowB + c * 16;
+                        cp_async16(st + jj * rowB + c * 16, kb + at);
+                        cp_async16(st + (kCompRows + jj) * rowB + c * 16, vb + at);
                     }
                 }
             };
 #pragma unroll
-            for (int i = 0; i < kCompStages - 1; ++i) {
+            for (int i = 0; i < kAhead; ++i) {
                 if (i < n_tiles) issue(i);
                 cp_async_commit();
             }
             for (int tile = 0; tile < n_tiles; ++tile) {
+                if (tid < kCompRows) put_rows(tile + kAhead, src_next, dst_next);
                 __syncthreads();  // the stage about to be refilled was written out last iteration
-                if (tile + kCompStages - 1 < n_tiles) issue(tile + kCompStages - 1);
+                if (tile + kAhead < n_tiles) issue(tile + kAhead);
                 cp_async_commit();
-                cp_async_wait<kCompStages - 1>();
+                if (tid < kCompRows) {
+                    find(tile + kAhead + 1, slot_next, src_next, dst_next);
+                    slot_next = kept_slot(tile + kAhead + 2);
+                }
+                cp_async_wait<kAhead>();
                 __syncthreads();  // every read of this tile has landed before any write
                 const unsigned char *st = cbuf + (tile % kCompStages) * stageB;
-                const int jb = tile_base(tile);
                 for (int idx = tid; idx < kCompRows * CPR; idx += kCompThreads) {
                     const int jj = idx / CPR, c = idx % CPR;
-                    const int j = jb + jj;
-                    if (j >= j0 && j < j1) {
-                        const int64_t dst = a.pv.row_phys(b, l, g, new_start + j);
-                        *reinterpret_cast<uint4 *>(kb + dst * rowB + c * 16) =
-                            *reinterpret_cast<const uint4 *>(st + jj * rowB + c * 16);
-                        *reinterpret_cast<uint4 *>(vb + dst * rowB + c * 16) =
+                    const uint32_t dst = rows_s[tile % kCompRowSets][1][jj];
+                    if (dst != ~0u) {
+                        const int64_t at = (int64_t)dst * rowB + c * 16;
+                        *reinterpret_cast<uint4 *>(kb + at) = *reinterpret_cast<const uint4 *>(st + jj * rowB + c * 16);
+                        *reinterpret_cast<uint4 *>(vb + at) =
                             *reinterpret_cast<const uint4 *>(st + (kCompRows + jj) * rowB + c * 16);
                     }
                 }
@@ -263,7 +300,7 @@ __device__ __forceinline__ void compact_stable_item(const CompactArgs &a, const 
 }
 
 // The stable compaction, one CTA per item: grid (items per sequence, sequences).
-__global__ void __launch_bounds__(kCompThreads) compact_stable_kernel(const CompactArgs a) {
+__global__ void __launch_bounds__(kCompThreads, 3) compact_stable_kernel(const CompactArgs a) {
     pdl_wait();
     extern __shared__ __align__(16) unsigned char cbuf[];
     __shared__ int scratch[32];
@@ -276,7 +313,7 @@ __global__ void __launch_bounds__(kCompThreads) compact_stable_kernel(const Comp
 // nothing moves) are skipped; their flags are read for 32 of the CTA's items at once, so a
 // step in which nothing moves costs one round of loads per CTA.  (One CTA per item: 16
 // sequences x 257 items of 64 KB shared memory took ~9 launch waves just to exit.)
-__global__ void __launch_bounds__(kCompThreads) compact_stable_strided_kernel(const CompactArgs a) {
+__global__ void __launch_bounds__(kCompThreads, 3) compact_stable_strided_kernel(const CompactArgs a) {
     pdl_wait();
     extern __shared__ __align__(16) unsigned char cbuf[];
     __shared__ int scratch[32];
