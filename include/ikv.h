@@ -129,8 +129,8 @@ typedef struct {
 
 /* Optional per-kernel CUDA events recorded on the call's stream by ikv_step
  * (caller-created with cudaEventCreate; NULL members are skipped):
- * begin (before the append), append_end, attend_end, combine_end
- * (both after the attention kernel, which merges its splits itself), score_end (after the score
+ * begin and append_end (before the attention kernel, which appends the new token),
+ * attend_end and combine_end (after it; it merges its splits itself), score_end (after the score
  * + EMA kernels), select_end, end (after compaction). */
 typedef struct {
     cudaEvent_t begin, append_end, attend_end, combine_end, score_end, select_end, end;

@@ -133,7 +133,7 @@ AttendWs attend_ws(const ikv_shape *s, int32_t cap, int n_layers, bool logits) {
 struct StepWs {
     AttendWs at;
     size_t keep, keep_len, done, cdone, sdone, moves, n_moves, sbuf, epart, vmean, slot, inv, util, live, raw, keep_raw,
-        n_raw, raw_pos, sel_best, sel_cnt, end;
+        n_raw, raw_pos, sel_best, sel_cnt, len1, end;
 };
 
 StepWs step_ws(const ikv_shape *s, int32_t cap, int32_t pos_cap) {
@@ -189,6 +189,8 @@ StepWs step_ws(const ikv_shape *s, int32_t cap, int32_t pos_cap) {
     off = align256(off + R * blk_max * sizeof(unsigned long long));
     w.sel_cnt = off;
     off = align256(off + R * blk_max * sizeof(uint32_t));
+    w.len1 = off;  // whole step: each sequence's length with the new token
+    off = align256(off + (size_t)s->batch * sizeof(int32_t));
     w.end = off;
     return w;
 }
@@ -255,7 +257,7 @@ ikv_status run_attend(const ikv_shape *s, const ikv_cache *c, int32_t layer0, in
                       const void *q, void *out, void *ws, const AttendWs &w, bool logits, int32_t *split_out,
                       int32_t *nsplit_out, cudaStream_t st, const ikv_timing *tm = nullptr,
                       bool counters_zeroed = false, int32_t sc_layers = 0, int32_t sc_layer0 = 0,
-                      const AppendArgs *append = nullptr, bool *gsum = nullptr, AttendArgs *unmerged = nullptr) {
+                      const NewRows *rows = nullptr, bool *gsum = nullptr, AttendArgs *unmerged = nullptr) {
     AttendArgs a{};
     a.k = c->k;
     a.v = c->v;
@@ -289,20 +291,17 @@ ikv_status run_attend(const ikv_shape *s, const ikv_cache *c, int32_t layer0, in
     a.rows_per_seq = rows_per_seq(s);
     a.sc_layers = sc_layers > 0 ? sc_layers : n_layers;
     a.sc_layer0 = sc_layer0;
-    // split step: the new token's rows of this layer are stored by the tensor-core kernel
-    // itself, or by a copy kernel ahead of the CUDA-core one
-    if (append && tc) {
-        a.k_new = append->k_new;
-        a.v_new = append->v_new;
-        a.slot = append->slot;
-        a.vnorm = append->vnorm;
+    if (rows) {  // the attention stores the new token's rows itself
+        a.k_new = rows->k;
+        a.v_new = rows->v;
+        a.slot = rows->slot;
+        a.vnorm = rows->vnorm;
+        a.book = rows->book;
         // a later layer call reads nothing before its dependency wait that the kernels
         // still draining ahead of it (the previous layer calls, or the caller's work
         // between them) write: the step's bookkeeping ran in ikv_step_begin, and this
         // layer's cached rows change only through the launch itself
-        a.early = layer0 > 0 ? 1 : 0;
-    } else if (append) {
-        IKV_TRY_CUDA(launch_append_rows(*append, st), "append rows launch");
+        a.early = tc && layer0 > 0 ? 1 : 0;
     }
     // the last CTA of each unit of several splits merges them into out and lse2
     // (`unmerged`: the caller's next kernel does, from the arguments handed back in it)
@@ -593,7 +592,8 @@ ikv_status ikv_compact_workspace_size(const ikv_shape *shape, const ikv_cache *c
 
 static ikv_status compact_impl(const ikv_shape *shape, ikv_cache *cache, const int32_t *keep, const int32_t *keep_len,
                                float *ema, int32_t mode, int32_t *moves, int32_t *n_moves, int32_t *done,
-                               cudaStream_t stream, int32_t max_holes = 0, bool by_layer = false) {
+                               cudaStream_t stream, int32_t max_holes = 0, bool by_layer = false,
+                               int32_t *len_out = nullptr) {
     CompactArgs a{};
     a.k = cache->k;
     a.v = cache->v;
@@ -605,6 +605,7 @@ static ikv_status compact_impl(const ikv_shape *shape, ikv_cache *cache, const i
     a.elem_bytes = elem_bytes(shape);
     a.mode = mode;
     a.len = cache->len;
+    a.len_out = len_out ? len_out : cache->len;
     a.pos = cache->pos;
     a.start = cache->start;
     a.done = done;
@@ -775,7 +776,8 @@ static ikv_status zero_control_words(const ikv_params *p, void *ws, const StepWs
 
 // Step 5: selection, then deferred or immediate compaction.
 static ikv_status evict_impl(const ikv_shape *shape, const ikv_params *p, ikv_cache *cache, float *ema, void *ws,
-                             const StepWs &w, cudaStream_t stream, const ikv_timing *tm, bool selected = false) {
+                             const StepWs &w, cudaStream_t stream, const ikv_timing *tm, bool selected = false,
+                             int32_t *len_out = nullptr) {
     const int32_t cap = cap_of(cache);
     const int32_t R = shape->batch * rows_per_seq(shape);
     if (!selected)
@@ -787,7 +789,7 @@ static ikv_status evict_impl(const ikv_shape *shape, const ikv_params *p, ikv_ca
     if (tm && (e = record(tm->select_end, stream))) return e;
     return compact_impl(shape, cache, at<int32_t>(ws, w.keep), at<int32_t>(ws, w.keep_len), ema, p->compact_mode,
                         at<int32_t>(ws, w.moves), at<int32_t>(ws, w.n_moves), at<int32_t>(ws, w.cdone), stream,
-                        p->max_holes);
+                        p->max_holes, false, len_out);
 }
 
 // The selection the score pass may run itself (not under the rank trace, whose raw
@@ -920,30 +922,18 @@ ikv_status ikv_step(const ikv_shape *shape, const ikv_params *p, ikv_cache *cach
     const StepWs &w = cx.w;
     const ikv_timing *tm = p->timing;
     if (cx.layerwise) {
-        // begin, every layer's new rows, one attention launch for all layers (each reads
-        // its own rows), then the per-layer evictions
+        // begin, one attention launch for all layers (each reads its own rows and stores the
+        // new token's), then the per-layer evictions
         if ((e = zero_control_words(p, ws, w, stream))) return e;
         LayerArgs la = layer_args(shape, p, cache, ema, ws, cx);
         IKV_TRY_CUDA(cudaMemsetAsync(la.live, 0, sizeof(uint32_t) * (size_t)shape->batch * la.live_words, stream),
                      "cudaMemsetAsync");
         IKV_TRY_CUDA(launch_layer_begin(la, cache->max_len, stream), "layer begin launch");
         PdlScope pdl;
-        AppendArgs ap{};
-        ap.k = cache->k;
-        ap.v = cache->v;
-        ap.pv = view_of(shape, cache);
-        ap.batch = shape->batch;
-        ap.layers = shape->layers;
-        ap.cap = cx.cap;
-        ap.elem_bytes = elem_bytes(shape);
-        ap.k_new = k_new;
-        ap.v_new = v_new;
-        ap.vnorm = cache->vnorm;
-        ap.slot = at<int32_t>(ws, w.slot);
-        IKV_TRY_CUDA(launch_append_rows(ap, stream), "append rows launch");
+        const NewRows rows{k_new, v_new, at<int32_t>(ws, w.slot), cache->vnorm};
         bool gsum = false;
         if ((e = run_attend(shape, cache, 0, shape->layers, cx.L1, q, out, ws, w.at, cx.scoring, nullptr, nullptr,
-                            stream, nullptr, true, 0, 0, nullptr, &gsum)))
+                            stream, nullptr, true, 0, 0, &rows, &gsum)))
             return e;
         return layer_evict(shape, p, cache, ema, ws, cx, stream, gsum);
     }
@@ -952,40 +942,42 @@ ikv_status ikv_step(const ikv_shape *shape, const ikv_params *p, ikv_cache *cach
     // kernel that counts leaves its counters zero again
     if ((e = zero_control_words(p, ws, w, stream))) return e;
     if (tm && (e = record(tm->begin, stream))) return e;
-    // With the tensor-core attention the append is bookkeeping only (the new token's slot,
-    // position and utility; len += 1, one CTA per sequence): the attention CTA whose chunk
-    // holds the new slot stores that layer and KV head's rows itself and uses them in place
-    // of the slot's old contents.  The CUDA-core path appends the rows first.
-    const bool tc_rows = use_tc(shape, cache, shape->layers, cx.L1);
-    int32_t *slot = at<int32_t>(ws, w.slot);
-    if ((e = append_impl(shape, cache, tc_rows ? nullptr : k_new, tc_rows ? nullptr : v_new, ema, cx.init_mean,
-                         at<int32_t>(ws, w.done), stream, true, tc_rows ? slot : nullptr)))
-        return e;
+    // The attention launch appends the new token: a CTA per sequence does the bookkeeping (its
+    // position and utility; the length with it goes to len1, for the step's later kernels), and
+    // the CTA whose chunk holds the new slot stores that layer and KV head's rows and uses them
+    // in place of the slot's old contents.  The compaction writes the step's final lengths.
     if (tm && (e = record(tm->append_end, stream))) return e;
-    // the rest of the chain may overlap each kernel's ramp-up with its predecessor's tail
-    // (not when per-kernel events are recorded: those time each kernel alone)
+    // the chain may overlap each kernel's ramp-up with its predecessor's tail (not when
+    // per-kernel events are recorded: those time each kernel alone)
     std::optional<PdlScope> pdl;
-    if (!tm) pdl.emplace();
-    AppendArgs rows{};
-    rows.k_new = k_new;
-    rows.v_new = v_new;
-    rows.slot = slot;
-    rows.vnorm = cache->vnorm;
+    if (!tm && p->ws_zeroed) pdl.emplace();  // (behind memsets, from the second kernel on)
+    int32_t *len1 = at<int32_t>(ws, w.len1);
+    NewRows rows{k_new, v_new, nullptr, cache->vnorm, {}};
+    rows.book.on = 1;
+    rows.book.len1 = len1;
+    rows.book.pos = cache->pos;
+    rows.book.next_pos = cache->next_pos;
+    rows.book.ema = ema;
+    rows.book.init_mean = cx.init_mean;
+    rows.book.dead_slots = cache->dead_slots;
     bool gsum = false;  // the attention may hand over normalised group sums instead of logits
     if ((e = run_attend(shape, cache, 0, shape->layers, cx.L1, q, out, ws, w.at, cx.scoring, nullptr, nullptr, stream,
-                        tm, true, 0, 0, tc_rows ? &rows : nullptr, &gsum)))
+                        tm, true, 0, 0, &rows, &gsum)))
         return e;
     if (tm && (e = record(tm->combine_end, stream))) return e;
+    if (!tm && !pdl) pdl.emplace();
+    ikv_cache appended = *cache;  // as the kernels between the attention and the compaction see it
+    appended.len = len1;
     float *raw = p->trace ? at<float>(ws, w.raw) : nullptr;
     const SelectFuse fs = select_fuse(p, cache, ws, cx);
     bool selected = false;
-    if (cx.scoring && (e = run_score(shape, cache, shape->layers, cx.elig, cx.n_elig, cx.L1, ws, w.at, p->alpha, ema,
+    if (cx.scoring && (e = run_score(shape, &appended, shape->layers, cx.elig, cx.n_elig, cx.L1, ws, w.at, p->alpha, ema,
                                      raw, stream, p->agg_mode, p->scorer, cx.sw, 0, false,
                                      p->trace ? nullptr : &fs, &selected, gsum)))
         return e;
     if (tm && (e = record(tm->score_end, stream))) return e;
-    if ((e = trace_before(shape, p, cache, ws, cx, stream))) return e;
-    if ((e = evict_impl(shape, p, cache, ema, ws, w, stream, tm, selected))) return e;
+    if ((e = trace_before(shape, p, &appended, ws, cx, stream))) return e;
+    if ((e = evict_impl(shape, p, &appended, ema, ws, w, stream, tm, selected, cache->len))) return e;
     if (tm && (e = record(tm->end, stream))) return e;
     return trace_after(shape, p, cache, ws, cx, stream);
 }
@@ -1022,20 +1014,7 @@ ikv_status ikv_step_layer(const ikv_shape *shape, const ikv_params *p, ikv_cache
         return fail(IKV_ERR_ALIGN, "q/out/k_new/v_new must be 16-byte aligned");
     cache = &cx.cv;
     PdlScope pdl;
-    AppendArgs a{};
-    a.k = cache->k;
-    a.v = cache->v;
-    a.pv = view_of(shape, cache);
-    a.batch = shape->batch;
-    a.layers = 1;
-    a.rows_per_seq = rows_per_seq(shape);
-    a.cap = cx.cap;
-    a.elem_bytes = elem_bytes(shape);
-    a.k_new = k_new;
-    a.v_new = v_new;
-    a.vnorm = cache->vnorm;
-    a.layer0 = layer;
-    a.slot = at<int32_t>(ws, cx.w.slot);
+    const NewRows rows{k_new, v_new, at<int32_t>(ws, cx.w.slot), cache->vnorm};
     bool eligible = false;
     for (int k = 0; k < cx.n_elig; ++k) eligible |= cx.elig[k] == layer;
     // the new token's rows and one layer's attention; on refresh steps its logits and
@@ -1043,7 +1022,7 @@ ikv_status ikv_step_layer(const ikv_shape *shape, const ikv_params *p, ikv_cache
     // ikv_step_end's score pass
     bool gsum = false;  // the same for every layer call of the step (attend_gsum)
     return run_attend(shape, cache, layer, 1, cx.L1, q, out, ws, cx.w.at, cx.scoring && eligible, nullptr, nullptr,
-                      stream, nullptr, true, shape->layers, layer, &a, &gsum);
+                      stream, nullptr, true, shape->layers, layer, &rows, &gsum);
 }
 
 ikv_status ikv_step_end(const ikv_shape *shape, const ikv_params *p, ikv_cache *cache, float *ema, int32_t t,

@@ -8,9 +8,12 @@
 // in the log2 domain; the logits are written out for the Eq. 1 score pass.  The warps'
 // results meet in shared memory once, at the end; a unit of several splits is merged by its
 // last CTA to arrive.
-#include "merge.cuh"
+#include "book.cuh"
 
 namespace ikv {
+
+__device__ unsigned int g_attend_error = 0;  // bit 2: an append found no free slot (start + len = cap)
+
 namespace {
 
 // 16 bytes to shared memory, the first n of them (0 or 16) from gmem and the rest zeros
@@ -77,6 +80,28 @@ __device__ __forceinline__ void finish_split(const AttendArgs &a, float *obuf, f
                            static_cast<T *>(a.out) + (hrow + h) * D, a.lse2 + lrow + h);
 }
 
+// The new token's K and V rows of (layer, KV head) from k_new / v_new into pool row `row`, and the
+// V row's norm into *vnorm (or null), by one warp.
+template <typename T, int D>
+__device__ __forceinline__ void store_new_rows(const AttendArgs &a, int64_t unit, int64_t row, float *vnorm) {
+    constexpr int kChunks = D * (int)sizeof(T) / 16, E = 16 / (int)sizeof(T);
+    const int lane = threadIdx.x & 31;
+    float sq = 0.f;
+    for (int c = lane; c < kChunks; c += 32) {
+        const uint4 k = reinterpret_cast<const uint4 *>(a.k_new)[unit * kChunks + c];
+        const uint4 v = reinterpret_cast<const uint4 *>(a.v_new)[unit * kChunks + c];
+        reinterpret_cast<uint4 *>(const_cast<void *>(a.k))[row * kChunks + c] = k;
+        reinterpret_cast<uint4 *>(const_cast<void *>(a.v))[row * kChunks + c] = v;
+        const T *x = reinterpret_cast<const T *>(&v);
+#pragma unroll
+        for (int e = 0; e < E; ++e) sq += static_cast<float>(x[e]) * static_cast<float>(x[e]);
+    }
+    if (vnorm) {
+        sq = warp_sum(sq);
+        if (lane == 0) *vnorm = sqrtf(sq);
+    }
+}
+
 // A sequence without slots: output 0, log-sum-exp -inf (written by its first split's CTA).
 template <typename T>
 __device__ __forceinline__ void store_empty(const AttendArgs &a, int G, int D, int b, int li, int g) {
@@ -125,11 +150,25 @@ __global__ void __launch_bounds__(kAttendThreads, 2) attend_f32_kernel(const Att
     pdl_wait();
     extern __shared__ __align__(128) unsigned char smem[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int s = blockIdx.x, g = blockIdx.y;
-    const int b = blockIdx.z % a.batch, li = blockIdx.z / a.batch;
+    // 1-D grid: the bookkeeping CTAs, if any, then splits, kv heads, sequences, layers
+    int bid = blockIdx.x;
+    if (a.book.on) {
+        if (bid < a.batch) {
+            book_sequence<kAttendThreads>(a.book, a.len, a.pv.start, a.cap, a.rows_per_seq, bid, &g_attend_error);
+            return;
+        }
+        bid -= a.batch;
+    }
+    const int s = bid % a.n_splits;
+    bid /= a.n_splits;
+    const int g = bid % a.pv.kv_heads;
+    bid /= a.pv.kv_heads;
+    const int b = bid % a.batch, li = bid / a.batch;
     const int l = a.layer0 + li;
-    const int L = a.len[b];
+    const int L0 = a.len[b];
     const int S0 = a.pv.start_of(b);
+    const bool grown = a.book.on && S0 + L0 < a.cap;
+    const int L = L0 + (grown ? 1 : 0);
     const int t0 = s * a.split_tokens;
     if (t0 >= L) {
         if (s == 0) store_empty<float>(a, G, D, b, li, g);
@@ -148,11 +187,16 @@ __global__ void __launch_bounds__(kAttendThreads, 2) attend_f32_kernel(const Att
 
     const unsigned char *kb = reinterpret_cast<const unsigned char *>(a.k) + lr * 16;
     const unsigned char *vb = reinterpret_cast<const unsigned char *>(a.v) + lr * 16;
-    // pool row of token lane % TW of the warp's group j (-1 past the split), one per lane;
-    // looked up one group ahead of its use, so the block table's latency is off the path
+    // the new token's slot (-1: none): its rows come from k_new / v_new, not from the pool
+    const int t_new = a.book.on ? (grown ? L0 : -1) : a.k_new ? a.slot[b] : -1;
+    const int64_t unit = ((int64_t)li * a.batch + b) * a.pv.kv_heads + g;
+    const unsigned char *kn = reinterpret_cast<const unsigned char *>(a.k_new) + unit * C::kRowB + lr * 16;
+    const unsigned char *vn = reinterpret_cast<const unsigned char *>(a.v_new) + unit * C::kRowB + lr * 16;
+    // pool row of token lane % TW of the warp's group j (-1 past the split, -2 the new token), one
+    // per lane; looked up one group ahead of its use, so the block table's latency is off the path
     auto lookup = [&](int j) -> int64_t {
         const int tok = t0 + (warp + C::kWarps * j) * TW + lane % TW;
-        return j < mine && tok < t1 ? a.pv.row_phys(b, l, g, S0 + tok) : -1;
+        return j < mine && tok < t1 ? tok == t_new ? -2 : a.pv.row_phys(b, l, g, S0 + tok) : -1;
     };
     auto issue = [&](int j, int64_t row) {
         unsigned char *st = ring + (j % NST) * C::kStageB + half * T * C::kRowB + lr * 16;
@@ -160,8 +204,8 @@ __global__ void __launch_bounds__(kAttendThreads, 2) attend_f32_kernel(const Att
         for (int t = 0; t < T; ++t) {
             const int64_t r = __shfl_sync(0xffffffffu, row, half * T + t);
             const int64_t at = (r < 0 ? 0 : r) * C::kRowB;
-            cp_async16_zfill(st + t * C::kRowB, kb + at, r >= 0);
-            cp_async16_zfill(st + (TW + t) * C::kRowB, vb + at, r >= 0);
+            cp_async16_zfill(st + t * C::kRowB, r == -2 ? kn : kb + at, r != -1);
+            cp_async16_zfill(st + (TW + t) * C::kRowB, r == -2 ? vn : vb + at, r != -1);
         }
     };
 #pragma unroll
@@ -170,6 +214,9 @@ __global__ void __launch_bounds__(kAttendThreads, 2) attend_f32_kernel(const Att
         cp_async_commit();
     }
     int64_t row_next = lookup(NST - 1);
+    if (warp == 0 && t_new >= t0 && t_new < t1)  // into the cache, for later steps
+        store_new_rows<float, D>(a, unit, a.pv.row_phys(b, l, g, S0 + t_new),
+                                 a.vnorm ? a.vnorm + (((int64_t)l * a.batch + b) * a.pv.kv_heads + g) * a.cap + t_new : nullptr);
 
     float q[G][4];  // the lane's four dims of each head, pre-scaled into the log2 domain
     const float *qg = reinterpret_cast<const float *>(a.q) + (((int64_t)li * a.batch + b) * a.q_heads + (int64_t)g * G) * D;
@@ -201,7 +248,7 @@ __global__ void __launch_bounds__(kAttendThreads, 2) attend_f32_kernel(const Att
         const int tok = t0 + (warp + C::kWarps * i) * TW + half * T + tx;
 #pragma unroll
         for (int j = 0; j < VPL; ++j)
-            if (i < mine && hx < G && tok + j < t1 && (!prow || __ldg(prow + tok + j) >= 0)) bits |= 1u << j;
+            if (i < mine && hx < G && tok + j < t1 && (!prow || tok + j == t_new || __ldg(prow + tok + j) >= 0)) bits |= 1u << j;
         return bits;
     };
     uint32_t live_next = live_of(0);
@@ -371,12 +418,26 @@ __global__ void __launch_bounds__(kAttendThreads, Bf16Cfg<D>::kCtasPerSm) attend
     pdl_wait();
     extern __shared__ __align__(128) unsigned char smem[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int s = blockIdx.x, g = blockIdx.y;
-    const int b = blockIdx.z % a.batch, li = blockIdx.z / a.batch;
+    // 1-D grid: the bookkeeping CTAs, if any, then splits, kv heads, sequences, layers
+    int bid = blockIdx.x;
+    if (a.book.on) {
+        if (bid < a.batch) {
+            book_sequence<kAttendThreads>(a.book, a.len, a.pv.start, a.cap, a.rows_per_seq, bid, &g_attend_error);
+            return;
+        }
+        bid -= a.batch;
+    }
+    const int s = bid % a.n_splits;
+    bid /= a.n_splits;
+    const int g = bid % a.pv.kv_heads;
+    bid /= a.pv.kv_heads;
+    const int b = bid % a.batch, li = bid / a.batch;
     const int l = a.layer0 + li;
     const int G = a.q_heads / a.pv.kv_heads;
-    const int L = a.len[b];
+    const int L0 = a.len[b];
     const int S0 = a.pv.start_of(b);
+    const bool grown = a.book.on && S0 + L0 < a.cap;
+    const int L = L0 + (grown ? 1 : 0);
     const int t0 = s * a.split_tokens;
     if (t0 >= L) {
         if (s == 0) store_empty<__nv_bfloat16>(a, G, D, b, li, g);
@@ -395,29 +456,39 @@ __global__ void __launch_bounds__(kAttendThreads, Bf16Cfg<D>::kCtasPerSm) attend
     constexpr int kStride = C::kWarps * 32;
     const int64_t page0 = (int64_t)l * a.pv.num_pages;
     const int32_t *table = a.pv.block_table + (int64_t)b * a.pv.max_pages;
+    // the new token's slot (-1: none): its rows come from k_new / v_new, not from the pool
+    const int t_new = a.book.on ? (grown ? L0 : -1) : a.k_new ? a.slot[b] : -1;
+    constexpr uint32_t kNewRow = ~0u - 1u;
     auto lookup = [&](int base) -> uint32_t {
         const int tok = base + lane;
         if (tok >= t1) return ~0u;
+        if (tok == t_new) return kNewRow;
         const int phys = S0 + tok;
         const int lp = a.pv.page_shift >= 0 ? phys >> a.pv.page_shift : phys / a.pv.page_size;
         return (uint32_t)(((page0 + table[lp]) * a.pv.kv_heads + g) * a.pv.page_size + (phys - lp * a.pv.page_size));
     };
-    auto alive = [&](int base) -> bool { return base + lane < t1 && (!prow || __ldg(prow + base + lane) >= 0); };
+    auto alive = [&](int base) -> bool {
+        const int tok = base + lane;
+        return tok < t1 && (!prow || tok == t_new || __ldg(prow + tok) >= 0);
+    };
     // 16-byte chunk c of a row lies at c ^ (row % 8): the eight rows an ldmatrix reads at one
     // chunk fall into different banks
     const int cr = lane / C::RL, cc = lane % C::RL;
     const unsigned char *kb = reinterpret_cast<const unsigned char *>(a.k) + cc * 16;
     const unsigned char *vb = reinterpret_cast<const unsigned char *>(a.v) + cc * 16;
+    const int64_t unit = ((int64_t)li * a.batch + b) * a.pv.kv_heads + g;
+    const unsigned char *kn = reinterpret_cast<const unsigned char *>(a.k_new) + unit * C::kRowB + cc * 16;
+    const unsigned char *vn = reinterpret_cast<const unsigned char *>(a.v_new) + unit * C::kRowB + cc * 16;
     auto issue = [&](int stage, int half, uint32_t rows) {
         const uint32_t st = ring + stage * C::kStageB + cr * C::kRowB;
 #pragma unroll
         for (int t = 0; t < TW; t += C::RPI) {
             const uint32_t r = __shfl_sync(0xffffffffu, rows, half * TW + t + cr);
             const uint32_t n = r == ~0u ? 0u : 16u;
-            const uint64_t at = (uint64_t)(r == ~0u ? 0u : r) * C::kRowB;
+            const uint64_t at = (uint64_t)(r >= kNewRow ? 0u : r) * C::kRowB;
             const uint32_t dst = st + t * C::kRowB + ((cc ^ ((t + cr) & 7)) << 4);
-            cp_async16_n(dst, kb + at, n);
-            cp_async16_n(dst + TW * C::kRowB, vb + at, n);
+            cp_async16_n(dst, r == kNewRow ? kn : kb + at, n);
+            cp_async16_n(dst + TW * C::kRowB, r == kNewRow ? vn : vb + at, n);
         }
         cp_async_commit();
     };
@@ -428,6 +499,10 @@ __global__ void __launch_bounds__(kAttendThreads, Bf16Cfg<D>::kCtasPerSm) attend
     }
     uint32_t rows_next = lookup(tok0 + kStride);
     uint32_t live = __ballot_sync(0xffffffffu, alive(tok0));
+    if (warp == 0 && t_new >= t0 && t_new < t1)  // into the cache, for later steps
+        store_new_rows<__nv_bfloat16, D>(a, unit, a.pv.row_phys(b, l, g, S0 + t_new),
+                                         a.vnorm ? a.vnorm + (((int64_t)l * a.batch + b) * a.pv.kv_heads + g) * a.cap + t_new
+                                                 : nullptr);
 
     // the lane's head (M row) and its tokens tq, tq + 1, tq + 8, tq + 9 of a stage
     const int h = lane >> 2, tq = (lane & 3) * 2;
@@ -552,13 +627,17 @@ __global__ void __launch_bounds__(kAttendThreads, Bf16Cfg<D>::kCtasPerSm) attend
     finish_split<__nv_bfloat16, D, C::GP, C::kWarps>(a, obuf, mlbuf, G, s, ns_active, b, li, g);
 }
 
+dim3 attend_grid(const AttendArgs &a) {
+    return dim3((unsigned)a.n_splits * a.pv.kv_heads * a.batch * a.n_layers + (a.book.on ? a.batch : 0));
+}
+
 template <int D, int G>
 cudaError_t launch_attend_f32_g(const AttendArgs &a, cudaStream_t st) {
     constexpr int smem = F32Cfg<D, G>::kSmemBytes;
     auto k = attend_f32_kernel<D, G>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    e = launch_k(k, dim3(a.n_splits, a.pv.kv_heads, a.batch * a.n_layers), dim3(kAttendThreads), smem, st, a);
+    e = launch_k(k, attend_grid(a), dim3(kAttendThreads), smem, st, a);
     note_launch();
     return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -579,7 +658,7 @@ cudaError_t launch_attend_bf16(const AttendArgs &a, cudaStream_t st) {
     constexpr int smem = Bf16Cfg<D>::kSmemBytes;
     cudaError_t e = cudaFuncSetAttribute(attend_bf16_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    e = launch_k(attend_bf16_kernel<D>, dim3(a.n_splits, a.pv.kv_heads, a.batch * a.n_layers), dim3(kAttendThreads), smem,
+    e = launch_k(attend_bf16_kernel<D>, attend_grid(a), dim3(kAttendThreads), smem,
                  st, a);
     note_launch();
     return e != cudaSuccess ? e : cudaGetLastError();
@@ -596,6 +675,13 @@ cudaError_t launch_attend(const AttendArgs &a, int dtype, int head_dim, int grou
         if (head_dim == 64) return launch_attend_f32<64>(a, group, st);
     }
     return cudaErrorInvalidValue;
+}
+
+cudaError_t read_clear_attend_error(unsigned int *v) {
+    unsigned int z = 0;
+    cudaError_t e = cudaMemcpyFromSymbol(v, g_attend_error, sizeof(*v));
+    if (e == cudaSuccess) e = cudaMemcpyToSymbol(g_attend_error, &z, sizeof(z));
+    return e;
 }
 
 }  // namespace ikv

@@ -30,7 +30,7 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
-#include "ikv_internal.cuh"
+#include "book.cuh"
 
 namespace ikv {
 
@@ -89,6 +89,7 @@ struct TcArgs {
     // the slot's old contents; vnorm (or null) gets their V norms
     const __nv_bfloat16 *k_new, *v_new;
     const int32_t *slot;
+    BookArgs book;              // on: the first a.batch CTAs append, the new slot is len[b]
     __nv_bfloat16 *k_pool, *v_pool;
     float *vnorm;
     // every unit is a single chunk: instead of per-head logits, write per token the KV
@@ -259,16 +260,26 @@ __global__ void __launch_bounds__(kThreads, 2)
     // dispatched last and fills the final wave.  The chunks of one CTA run as passes over
     // the same TMEM columns; their (max, sum, output) are merged in registers.
     const int n_units = a.batch * a.n_layers * a.kv_heads;
-    const int cta = blockIdx.x / n_units;  // CTA index within the unit
-    const int unit_id = blockIdx.x % n_units;
+    int bid = blockIdx.x;
+    if (a.book.on) {
+        if (bid < a.batch) {
+            book_sequence<kThreads>(a.book, a.len, a.start, a.cap, a.rows_per_seq, bid, &g_tc_error);
+            return;
+        }
+        bid -= a.batch;
+    }
+    const int cta = bid / n_units;  // CTA index within the unit
+    const int unit_id = bid % n_units;
     const int g = unit_id % a.kv_heads;
     const int b = (unit_id / a.kv_heads) % a.batch, li = (unit_id / a.kv_heads) / a.batch;
     const int l = a.layer0 + li;
     // The unit's valid rows are physical slots [S0, S0 + L).  Chunks cut the 128-aligned
     // physical tiles covering them (TMA boxes stay page aligned); rows outside are masked.
     // (L2 loads: an early CTA reads these before the dependency wait)
-    const int L = __ldcg(a.len + b);
+    const int L0 = __ldcg(a.len + b);
     const int S0 = a.start ? __ldcg(a.start + b) : 0;
+    const bool grown = a.book.on && S0 + L0 < a.cap;
+    const int L = L0 + (grown ? 1 : 0);
     const int ft = S0 / kTile;
     const int nt_unit = L > 0 ? (S0 + L + kTile - 1) / kTile - ft : 0;
     const int item = a.split_tokens / kTile;  // tiles per chunk
@@ -331,7 +342,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     // writes the new rows into the loaded K and V tiles before their products read them.
     int p_new = -1;
     if (a.k_new) {
-        const int j = __ldcg(a.slot + b);
+        const int j = a.book.on ? (grown ? L0 : -1) : __ldcg(a.slot + b);
         const int pn = S0 + j;
         if (j >= 0 && pn >= chunk_t0(0) && pn < chunk_t0(np - 1) + chunk_n(np - 1) * kTile) p_new = pn;
     }
@@ -555,7 +566,7 @@ __global__ void __launch_bounds__(kThreads, 2)
             uint32_t live_bits = 0u;
             for (int i = 0; i < n; ++i) {
                 const int tok = t0 + i * kTile + tid;  // physical slot; logical slot tok - S0
-                if (tok >= lo && tok < t1 && (!prow || __ldg(prow + (tok - S0)) >= 0)) live_bits |= 1u << i;
+                if (tok >= lo && tok < t1 && (!prow || tok == p_new || __ldg(prow + (tok - S0)) >= 0)) live_bits |= 1u << i;
             }
             if (ok) ok = mbar_wait(s_full, p & 1, abort_flag);
             ok = __all_sync(0xffffffffu, ok);
@@ -970,12 +981,13 @@ cudaError_t launch_attend_tc(const AttendArgs &a, const TcOutputs &o, int group,
     t.k_pool = reinterpret_cast<__nv_bfloat16 *>(const_cast<void *>(a.k));
     t.v_pool = reinterpret_cast<__nv_bfloat16 *>(const_cast<void *>(a.v));
     t.vnorm = a.vnorm;
+    t.book = a.book;
     t.gsum = a.gsum;
     t.early = a.early;
     t.stall = g_stall_next.exchange(0);
     const int64_t units = (int64_t)a.pv.kv_heads * a.batch * a.n_layers;
     t.passes = tc_passes(units, a.n_splits, sms, a.gsum != 0);
-    dim3 grid((unsigned)(((a.n_splits + t.passes - 1) / t.passes) * units));
+    dim3 grid((unsigned)(((a.n_splits + t.passes - 1) / t.passes) * units + (a.book.on ? a.batch : 0)));
     cudaError_t e;
     switch (group) {
         case 1: e = launch_tc_g<1>(mk, mv, t, grid, st); break;
@@ -1001,11 +1013,12 @@ extern "C" ikv_status ikv_device_status(uint32_t *flags) {
     unsigned int v = 0, z = 0;
     cudaError_t e = cudaMemcpyFromSymbol(&v, ikv::g_tc_error, sizeof(v));
     if (e == cudaSuccess) e = cudaMemcpyToSymbol(ikv::g_tc_error, &z, sizeof(z));
-    unsigned int ap = 0, lw = 0, tr = 0;
+    unsigned int ap = 0, at = 0, lw = 0, tr = 0;
+    if (e == cudaSuccess) e = ikv::read_clear_attend_error(&at);
     if (e == cudaSuccess) e = ikv::read_clear_append_error(&ap);
     if (e == cudaSuccess) e = ikv::read_clear_layer_error(&lw);
     if (e == cudaSuccess) e = ikv::read_clear_trace_error(&tr);
     if (e != cudaSuccess) return ikv::report(IKV_ERR_CUDA, "ikv_device_status: %s", cudaGetErrorString(e));
-    *flags = v | (ap ? 4u : 0u) | lw | tr;
+    *flags = v | at | (ap ? 4u : 0u) | lw | tr;
     return IKV_OK;
 }

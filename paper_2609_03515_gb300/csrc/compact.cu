@@ -88,6 +88,11 @@ __device__ __forceinline__ void gather_row(T *row, const int32_t *kp, int n) {
     }
 }
 
+// A sequence whose slots all stay: its length as it is.
+__device__ __forceinline__ void keep_length(const CompactArgs &a, int b) {
+    if (a.len_out != a.len) a.len_out[b] = a.len[b];
+}
+
 // Deferred compaction: sequence b only marks its evicted slots dead while its dead
 // slots (the ones already dead plus this step's evictions: len - kept) stay within
 // max_holes.  Every row of b keeps the same number of slots, so row b * rps decides.
@@ -120,10 +125,14 @@ __device__ __forceinline__ void compact_stable_item(const CompactArgs &a, const 
     const int tid = threadIdx.x;
     const int kvh = a.pv.kv_heads;
     const int nkv = a.layers * kvh;
-    if (a.keep_len[b * a.rows_per_seq] < 0) return;  // selection marked the victim dead: nothing to do
+    if (a.keep_len[b * a.rows_per_seq] < 0) {  // selection marked the victim dead: nothing to do
+        if (x == 0 && tid == 0) keep_length(a, b);
+        return;
+    }
     const int L = a.len[b];
     const int S = a.start ? a.start[b] : 0;
     if (defer_of(a, b, L, S)) {  // nothing moves; len, start and the arrival counter stay as they are
+        if (x == 0 && tid == 0) keep_length(a, b);
         if (x >= nkv) mark_dead_row(a, b * a.rows_per_seq + (x - nkv), L);
         return;
     }
@@ -292,7 +301,7 @@ __device__ __forceinline__ void compact_stable_item(const CompactArgs &a, const 
     __syncthreads();
     if (tid == 0) {
         if (arrive_acq_rel(&a.done[b]) == nkv + a.rows_per_seq - 1) {
-            a.len[b] = n0;
+            a.len_out[b] = n0;
             if (a.start) a.start[b] = new_start;
             a.done[b] = 0;
         }
@@ -324,7 +333,9 @@ __global__ void __launch_bounds__(kCompThreads, 3) compact_stable_strided_kernel
     for (int k0 = 0; blockIdx.x + (int64_t)k0 * gridDim.x < n_items; k0 += 32) {
         if (threadIdx.x < 32) {
             const int64_t item = blockIdx.x + (int64_t)(k0 + threadIdx.x) * gridDim.x;
-            flagged[threadIdx.x] = item < n_items ? a.keep_len[(int)(item / nx) * a.rows_per_seq] < 0 : 1;
+            const int b = (int)(item / nx);
+            flagged[threadIdx.x] = item < n_items ? a.keep_len[b * a.rows_per_seq] < 0 : 1;
+            if (item < n_items && flagged[threadIdx.x] && item % nx == 0) keep_length(a, b);
         }
         __syncthreads();
 #pragma unroll 1
@@ -390,7 +401,10 @@ __global__ void __launch_bounds__(kCompThreads) holefill_move_kernel(const Compa
     const int b = blockIdx.y, x = blockIdx.x;
     const int kvh = a.pv.kv_heads;
     const int nkv = a.layers * kvh;
-    if (a.keep_len[b * a.rows_per_seq] < 0) return;  // selection marked the victim dead: nothing to do
+    if (a.keep_len[b * a.rows_per_seq] < 0) {  // selection marked the victim dead: nothing to do
+        if (x == 0 && tid == 0) keep_length(a, b);
+        return;
+    }
     if (x < nkv) {
         const int l = x / kvh, g = x % kvh;
         const int r = b * a.rows_per_seq + (a.row_by_layer ? l : a.rows_per_seq == 1 ? 0 : g);
@@ -419,6 +433,7 @@ __global__ void __launch_bounds__(kCompThreads) holefill_move_kernel(const Compa
     const int nm = a.n_moves[r];
     if (nm < 0) {  // deferred: mark this step's evictions dead; len stays
         mark_dead_row(a, r, a.len[b]);
+        if (rr == 0 && tid == 0) keep_length(a, b);
         return;
     }
     const int32_t *mv = a.moves + (int64_t)r * a.cap * 2;
@@ -429,7 +444,7 @@ __global__ void __launch_bounds__(kCompThreads) holefill_move_kernel(const Compa
         pos[d] = pos[s];
         if (ema) ema[d] = ema[s];
     }
-    if (rr == 0 && tid == 0) a.len[b] = a.keep_len[r];
+    if (rr == 0 && tid == 0) a.len_out[b] = a.keep_len[r];
 }
 
 // New token of every sequence into slot len[b] of every layer and kv head.
@@ -540,53 +555,6 @@ __global__ void __launch_bounds__(kCompThreads) append_kernel(const AppendArgs a
     }
 }
 
-// Split step: the new token's rows of layers layer0 .. layer0 + layers - 1 into the
-// slot the begin call reserved.  CTA (x, b) copies (layer, kv head) rows 8x .. 8x+7 of
-// sequence b and stores their value-row norms.
-__global__ void __launch_bounds__(kCompThreads) append_rows_kernel(const AppendArgs a) {
-    pdl_wait();
-    const int tid = threadIdx.x;
-    const int b = blockIdx.y;
-    const int kvh = a.pv.kv_heads;
-    const int nkv = a.layers * kvh;
-    const int j = a.slot[b];
-    if (j < 0) return;  // no room: the begin call flagged the error and kept len
-    const int S = a.pv.start_of(b);
-    const int rowB = a.pv.head_dim * a.elem_bytes;
-    const int CPR = rowB >> 4;
-    unsigned char *kb = reinterpret_cast<unsigned char *>(a.k);
-    unsigned char *vb = reinterpret_cast<unsigned char *>(a.v);
-    const unsigned char *kn = reinterpret_cast<const unsigned char *>(a.k_new);
-    const unsigned char *vn = reinterpret_cast<const unsigned char *>(a.v_new);
-    for (int idx = tid; idx < kAppendRows * CPR; idx += kCompThreads) {
-        const int x = blockIdx.x * kAppendRows + idx / CPR, c = idx % CPR;
-        if (x < nkv) {
-            const int li = x / kvh, g = x % kvh;
-            const int64_t src = (((int64_t)li * a.batch + b) * kvh + g) * rowB + c * 16;
-            const int64_t dst = a.pv.row_phys(b, a.layer0 + li, g, S + j) * rowB + c * 16;
-            *reinterpret_cast<uint4 *>(kb + dst) = *reinterpret_cast<const uint4 *>(kn + src);
-            *reinterpret_cast<uint4 *>(vb + dst) = *reinterpret_cast<const uint4 *>(vn + src);
-        }
-    }
-    if (a.vnorm) {
-        const int x = blockIdx.x * kAppendRows + (tid >> 5), lane = tid & 31;
-        if ((tid >> 5) < kAppendRows && x < nkv) {
-            const int li = x / kvh, g = x % kvh;
-            const int64_t e0 = (((int64_t)li * a.batch + b) * kvh + g) * a.pv.head_dim;
-            float sq = 0.f;
-            for (int e = lane; e < a.pv.head_dim; e += 32) {
-                const float xv = a.elem_bytes == 2
-                                     ? __bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(a.v_new)[e0 + e])
-                                     : reinterpret_cast<const float *>(a.v_new)[e0 + e];
-                sq += xv * xv;
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-            if (lane == 0) a.vnorm[(((int64_t)(a.layer0 + li) * a.batch + b) * kvh + g) * a.cap + j] = sqrtf(sq);
-        }
-    }
-}
-
 }  // namespace
 
 cudaError_t launch_compact(const CompactArgs &a, int mode, int sms, cudaStream_t st) {
@@ -636,13 +604,6 @@ cudaError_t launch_append(const AppendArgs &a, cudaStream_t st) {
     const int nkv = a.layers * a.pv.kv_heads;
     dim3 grid(a.k_new ? (nkv + kAppendRows - 1) / kAppendRows : 1, a.batch);
     cudaError_t e = launch_k(append_kernel, grid, dim3(kCompThreads), 0, st, a);
-    note_launch();
-    return e != cudaSuccess ? e : cudaGetLastError();
-}
-
-cudaError_t launch_append_rows(const AppendArgs &a, cudaStream_t st) {
-    dim3 grid((a.layers * a.pv.kv_heads + kAppendRows - 1) / kAppendRows, a.batch);
-    cudaError_t e = launch_k(append_rows_kernel, grid, dim3(kCompThreads), 0, st, a);
     note_launch();
     return e != cudaSuccess ? e : cudaGetLastError();
 }

@@ -85,6 +85,15 @@ struct PagedView {
     }
 };
 
+// A step's append, by extra CTAs of its attention launch (book.cuh)
+struct BookArgs {
+    int32_t on;                 // nonzero: they run, and len is the length before the append
+    int32_t *len1;              // [batch] the length after it
+    int32_t *pos, *next_pos;
+    float *ema;
+    int32_t init_mean, dead_slots;
+};
+
 struct AttendArgs {
     const void *k, *v;          // pools
     PagedView pv;
@@ -103,12 +112,13 @@ struct AttendArgs {
     // logits and lse2 hold sc_layers layers per sequence; local layer li is their layer
     // sc_layer0 + li (a per-layer launch writes into a whole step's arrays)
     int32_t sc_layers, sc_layer0;
-    // tensor-core kernel, split step: the new token's rows of this (single) layer,
-    // [batch][kv_heads][D], stored into logical slot slot[b] (-1: none) before they are
-    // read; their V norms into vnorm (or null).  k_new null: no append.
+    // the new token's rows of the launch's layers, [n_layers][batch][kv_heads][D], stored into
+    // logical slot slot[b] (-1: none) and used in place of what that slot held; their V norms
+    // into vnorm (or null).  k_new null: no append.
     const void *k_new, *v_new;
-    const int32_t *slot;
+    const int32_t *slot;        // unused when book.on: the new token's slot is len[b]
     float *vnorm;
+    BookArgs book;
     // tensor-core kernel, every unit one chunk: logits holds, per token, each KV head's sum
     // of its query group's normalised probabilities ([batch][sc_layers][kv_heads][lstride])
     // instead of per-head logits
@@ -191,6 +201,14 @@ struct ScoreOneArgs {
 };
 cudaError_t launch_score_one(const ScoreOneArgs &a, int32_t max_len, int sms, cudaStream_t st);
 
+// a step's new rows, and its append if the attention does that too, as AttendArgs takes them
+struct NewRows {
+    const void *k, *v;
+    const int32_t *slot;
+    float *vnorm;
+    BookArgs book;
+};
+
 // tensor-core attention (bf16, head_dim 128): attend_tc.cu
 constexpr int kTcTile = 128;
 bool tc_supported(int dtype, int head_dim, int group, int page_size);
@@ -231,6 +249,8 @@ struct CompactArgs {
     int32_t batch, layers, rows_per_seq, cap, elem_bytes;
     int32_t mode;               // IKV_COMPACT_*
     int32_t *len, *pos;
+    int32_t *len_out;           // [batch] receives the lengths: len itself, or, when len holds a step's
+                                // lengths with the new token, the cache's (then written in every case)
     int32_t *start;             // [batch] or null; advanced by the shorter-side mode
     int32_t *done;              // [batch] arrival counters, zero on entry; reset by the last CTA
     float *ema;
@@ -256,15 +276,11 @@ struct AppendArgs {
     int32_t dead_slots;         // the mean initialisation skips slots with pos < 0
     int32_t *done;              // [batch] arrival counters, zero on entry; reset by the last CTA
     float *vnorm;               // [layers][batch][kv_heads][cap]: the new row's norm is stored, or null
-    // split step: k_new == null makes launch_append do the bookkeeping only and record
-    // each sequence's reserved logical slot (-1: no room) in slot[b]; launch_append_rows
-    // then writes layer layer0's rows (k_new: [batch][kv_heads][D]) into that slot
-    int32_t layer0;
+    // k_new == null makes launch_append do the bookkeeping only and record each sequence's
+    // reserved logical slot (-1: no room) in slot[b]; the attention stores the rows
     int32_t *slot;
 };
 cudaError_t launch_append(const AppendArgs &a, cudaStream_t st);
-// rows of layers layer0 .. layer0 + layers - 1 (k_new: [layers][batch][kv_heads][D]) into slot[b]
-cudaError_t launch_append_rows(const AppendArgs &a, cudaStream_t st);
 
 // Per-layer eviction (IKV_EVICT_LAYER): a position-indexed state m [batch][pos_cap]
 // shared by all layers; layer l's positions in pos row b * layers + l.  Within a step no
@@ -312,5 +328,7 @@ cudaError_t launch_trace(const TraceArgs &a, cudaStream_t st);
 cudaError_t read_clear_trace_error(unsigned int *v);
 // reads and clears the append kernel's device error word (bit 0: no free slot)
 cudaError_t read_clear_append_error(unsigned int *v);
+// the same of the kernels of attend.cu (bit 2)
+cudaError_t read_clear_attend_error(unsigned int *v);
 
 }  // namespace ikv

@@ -1,0 +1,121 @@
+"""The append inside a step's attention launch, at the edges of the kernels' tiles: the new
+token's rows, position, utility and length, and a sequence without room."""
+import math
+
+import pytest
+import torch
+
+from paper_2609_03515_gb300 import DecodeCache, ikv
+
+pytestmark = pytest.mark.gpu
+
+LENS = [0, 1, 7, 8, 15, 16, 31, 127, 128, 129, 255, 300]
+
+
+@pytest.mark.parametrize("gran", [ikv.IKV_GRAN_SEQ, ikv.IKV_GRAN_KVHEAD])
+@pytest.mark.parametrize("dtype,d,ps", [(ikv.IKV_BF16, 128, 64), (ikv.IKV_BF16, 128, 24), (ikv.IKV_BF16, 64, 16),
+                                        (ikv.IKV_F32, 64, 16), (ikv.IKV_F32, 128, 48)])
+def test_step_appends(dtype, d, ps, gran):
+    dt = torch.bfloat16 if dtype == ikv.IKV_BF16 else torch.float32
+    kvh, G, layers, nb = 2, 4, 3, len(LENS)
+    gen = torch.Generator(device="cuda").manual_seed(d + ps)
+    c = DecodeCache(nb, layers, G * kvh, kvh, d, max(LENS) + 8, dtype=dtype, page_size=ps, page_perm_seed=2,
+                    granularity=gran, value_norms=True)
+    c.k.copy_(torch.randn(c.k.shape, generator=gen, device="cuda"))
+    c.v.copy_(torch.randn(c.v.shape, generator=gen, device="cuda"))
+    c.set_prefill(LENS, [10000] * nb)  # nothing to evict
+    c.start.copy_(torch.tensor([(3 * b) % 7 for b in range(nb)], dtype=torch.int32))
+    full = nb - 1
+    c.start[full] = c.cap - LENS[full]  # no room for its new token
+    c.ema.copy_(torch.rand(c.ema.shape, generator=gen, device="cuda"))
+    c.pos[torch.rand(c.pos.shape, generator=gen, device="cuda") < 0.15] = -1
+    for b, L in enumerate(LENS):  # a stale mark in the slot that the new token gets
+        if L < c.cap:
+            c.pos.view(nb, -1, c.cap)[b, :, L] = -1
+    q = torch.randn(layers, nb, G * kvh, d, generator=gen, device="cuda").to(dt)
+    kn = torch.randn(layers, nb, kvh, d, generator=gen, device="cuda").to(dt)
+    vn = torch.randn(layers, nb, kvh, d, generator=gen, device="cuda").to(dt)
+    out = torch.full((layers, nb, G * kvh, d), 9.0, device="cuda").to(dt)
+    ema0, pos0 = c.ema.clone(), c.pos.clone()
+    p = c.params(0.5, refresh_period=2, max_holes=8)
+    cch = c.cache(max(LENS), dead_slots=True)
+    n = ikv.ikv_step_workspace_size(c.shape(), cch)
+    ws = torch.full((n,), 0xAB, dtype=torch.uint8, device="cuda")
+    ikv.ikv_step(c.shape(), p, cch, c.ema, 2, q, kn, vn, out, ws, n)  # t = 2: the mean initialisation
+    torch.cuda.synchronize()
+    assert ikv.ikv_device_status() == 4
+    R = c.rows_per_seq
+    for b, L in enumerate(LENS):
+        new = b != full
+        assert int(c.next_pos[b]) == L + new
+        # lengths: a sequence compacts only past max_holes dead slots, its order kept
+        dead = [int((pos0[b * R + r, :L] < 0).sum()) for r in range(R)]
+        if R > 1:  # rows of one sequence with different numbers of dead slots are no state of the library
+            live = [pos0[b * R + r, :L] >= 0 for r in range(R)]
+        else:
+            live = [pos0[b, :L] >= 0]
+        for l in range(layers):
+            for g in range(kvh):
+                rr = 0 if R == 1 else g
+                lv = torch.cat([live[rr], torch.ones(int(new), dtype=torch.bool, device="cuda")])
+                if not bool(lv.any()):
+                    continue
+                if dead[0] <= 8 or not new:
+                    K, V = c.gather(c.k, b, l, g, L).double(), c.gather(c.v, b, l, g, L).double()
+                    if new:
+                        if int(c.len[b]) == L + 1:
+                            got_k, got_v = c.gather(c.k, b, l, g, L + 1)[L], c.gather(c.v, b, l, g, L + 1)[L]
+                            assert torch.equal(got_k, kn[l, b, g]) and torch.equal(got_v, vn[l, b, g])
+                            vnorm = float(vn[l, b, g].double().norm())
+                            assert abs(float(c.vnorm[l, b, g, L]) - vnorm) < 1e-5 * max(1.0, vnorm)
+                        else:
+                            continue
+                        K = torch.cat([K, kn[l, b, g].double()[None]])
+                        V = torch.cat([V, vn[l, b, g].double()[None]])
+                    elif int(c.len[b]) != L:
+                        continue
+                    z = q[l, b, g * G:(g + 1) * G].double() @ K.T / math.sqrt(d)
+                    z[:, ~lv] = -math.inf
+                    want = torch.softmax(z, -1) @ V
+                    err = (out[l, b, g * G:(g + 1) * G].double() - want).abs().max()
+                    assert err < (2e-2 if dtype == ikv.IKV_BF16 else 1e-4), (L, l, g, float(err))
+        if new and int(c.len[b]) == L + 1:
+            for r in range(R):
+                row = b * R + r
+                assert int(c.pos[row, L]) == L
+                mean = ema0[row, :L][live[r]].double().mean() if bool(live[r].any()) else torch.tensor(0.0)
+                assert abs(float(c.ema[row, L]) - float(mean)) < 1e-5
+
+
+@pytest.mark.parametrize("dtype,d", [(ikv.IKV_BF16, 128), (ikv.IKV_F32, 64)])
+def test_step_lengths_without_eviction(dtype, d):
+    """Lengths and positions over steps that evict nothing, then defer, then compact."""
+    dt = torch.bfloat16 if dtype == ikv.IKV_BF16 else torch.float32
+    for mode in (ikv.IKV_COMPACT_STABLE, ikv.IKV_COMPACT_STABLE_SHORT, ikv.IKV_COMPACT_HOLEFILL):
+        lens, budget, holes = [5, 40, 130], [9, 38, 130], 3
+        c = DecodeCache(3, 2, 4, 2, d, 400, dtype=dtype, page_size=16, page_perm_seed=2)
+        c.k.normal_()
+        c.v.normal_()
+        c.set_prefill(lens, budget)
+        ws = c.step_workspace()
+        L, live = list(lens), list(lens)
+        z = torch.randn(2, 3, 2, d, device="cuda").to(dt)
+        q = torch.randn(2, 3, 4, d, device="cuda").to(dt)
+        out = torch.empty_like(q)
+        for t in range(1, 12):
+            p = c.params(0.9, refresh_period=2, max_holes=holes, compact_mode=mode, ws_zeroed=t > 1)
+            ikv.ikv_step(c.shape(), p, c.cache(max(L)), c.ema, t, q, z, z, out, ws, ws.numel())
+            L = [x + 1 for x in L]
+            live = [x + 1 for x in live]
+            for b in range(3):
+                kept = min(live[b], budget[b])
+                if not L[b] - kept <= holes:
+                    L[b] = kept
+                live[b] = kept
+            assert c.len.cpu().tolist() == L, (mode, t)
+            assert c.next_pos.cpu().tolist() == [x + t for x in lens]
+            for b in range(3):
+                pos = c.pos[b, :L[b]].cpu()
+                assert int((pos >= 0).sum()) == live[b]
+                assert pos[pos >= 0].unique().numel() == live[b]
+        assert ikv.ikv_device_status() == 0
