@@ -11,7 +11,7 @@ namespace {
 // beside this one work from it (slot len[b] is the new token's, live whatever pos still says
 // there).  No room: len1[b] = len[b] and bit 2 of *err.
 template <int NT>
-__device__ __forceinline__ void book_sequence(const BookArgs &k, const int32_t *len, const int32_t *start, int32_t cap,
+__device__ __noinline__ void book_sequence(const BookArgs &k, const int32_t *len, const int32_t *start, int32_t cap,
                                               int32_t rows_per_seq, int b, unsigned int *err) {
     constexpr int NW = NT / 32, U = 8;
     __shared__ float scratch[2][NW];

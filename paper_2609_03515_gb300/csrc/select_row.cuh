@@ -48,7 +48,7 @@ constexpr int kSelMaxCtas = 8;  // CTAs that share a row (portable cluster size)
 // The selection of utility row r by C CTAs of NT threads (C > 1: the cluster they form; this
 // one is its `rank`-th), entered by all of their threads.  CTA `rank` owns a contiguous C-th of
 // the row's slots and keeps their keys in keys[0, keys_cap) (shared memory) when they fit;
-// otherwise every sweep reads the row again, eight loads in flight a thread.
+// otherwise every sweep reads the row again, a few loads in flight a thread.
 template <int NT>
 __device__ __forceinline__ void select_row(int rank, int C, int r, int32_t cap, const float *__restrict__ util,
                                            const int32_t *__restrict__ len, int32_t rps,
@@ -56,11 +56,12 @@ __device__ __forceinline__ void select_row(int rank, int C, int r, int32_t cap, 
                                            int32_t *keep_len, DeferArgs df, uint32_t *keys, int keys_cap) {
     static_assert(NT >= 256 && NT % 32 == 0, "the digit scan needs 256 threads at least, whole warps");
     constexpr int NW = NT / 32;
-    constexpr int U = 8;  // keys a thread has in flight
+    constexpr int U = NT == 256 ? 4 : 8;  // keys a thread has in flight
     __shared__ uint32_t hist[2][256];
     __shared__ uint32_t warp_a[NW], warp_b[NW];
     __shared__ unsigned long long warp_min[NW], s_min;
     __shared__ uint32_t s_digit, s_above, s_live, s_gt, s_eq;
+    __shared__ bool s_whole;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b = r / rps;
@@ -219,12 +220,19 @@ __device__ __forceinline__ void select_row(int rank, int C, int r, int32_t cap, 
                     if (incl - v < k && incl >= k) {  // exactly one digit satisfies this
                         s_digit = 255u - (uint32_t)tid;
                         s_above = incl - v;
+                        s_whole = incl == k;
                     }
                 }
                 __syncthreads();
                 k -= s_above;
                 prefix |= s_digit << shift;
                 mask |= 0xFFu << shift;
+                // every key of the digit's bin is kept (short rows: after two digits, as a rule):
+                // the cut runs just below the bin, the remaining digits do not matter
+                if (s_whole && prefix != 0u) {
+                    prefix -= 1u;
+                    break;
+                }
             }
             theta = prefix;
         }
@@ -257,17 +265,25 @@ __device__ __forceinline__ void select_row(int rank, int C, int r, int32_t cap, 
             warp_b[warp] = eq;
         }
         __syncthreads();
-        if (tid == 0) {
-            uint32_t g = 0u, e = 0u;
-            for (int w = 0; w < NW; ++w) {
-                const uint32_t wg = warp_a[w], we = warp_b[w];
-                warp_a[w] = g;
-                warp_b[w] = e;
-                g += wg;
-                e += we;
+        if (warp == 0) {  // exclusive over the warps
+            uint32_t g = lane < NW ? warp_a[lane] : 0u, e = lane < NW ? warp_b[lane] : 0u;
+            const uint32_t g0 = g, e0 = e;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t yg = __shfl_up_sync(0xffffffffu, g, o), ye = __shfl_up_sync(0xffffffffu, e, o);
+                if (lane >= o) {
+                    g += yg;
+                    e += ye;
+                }
             }
-            s_gt = g;
-            s_eq = e;
+            if (lane < NW) {
+                warp_a[lane] = g - g0;
+                warp_b[lane] = e - e0;
+            }
+            if (lane == NW - 1) {
+                s_gt = g;
+                s_eq = e;
+            }
         }
         sync_all();
         uint32_t gt_all = 0u, gt_run = warp_a[warp], eq_run = warp_b[warp];
