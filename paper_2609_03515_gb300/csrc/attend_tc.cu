@@ -128,26 +128,34 @@ __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
         : "memory");
     return ok != 0;
 }
+// The same, suspended in hardware until the phase completes or about `ns` have passed.
+__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity, uint32_t ns) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\tselp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity), "r"(ns)
+        : "memory");
+    return ok != 0;
+}
 __device__ __forceinline__ uint64_t global_ns() {
     uint64_t t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
 }
-// Bounded wait on an mbarrier phase (non-blocking polls, at most kWaitNs of wall
-// time).  Returns false -- raising the CTA's abort flag and the global error
+constexpr uint32_t kTryNs = 2000;  // a suspended wait's length; the waits below loop over it
+// Bounded wait on an mbarrier phase (suspended waits, at most kWaitNs of wall
+// time in all).  Returns false -- raising the CTA's abort flag and the global error
 // word -- if the phase does not complete in time, or returns false at once if
 // another role of the CTA has already aborted.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort,
                                           uint64_t limit_ns = kWaitNs) {
     if (mbar_test(bar, parity)) return true;
     const uint64_t start = global_ns();
-    for (uint32_t i = 1;; ++i) {
-        if (mbar_test(bar, parity)) return true;
-        if (i > 64) __nanosleep(32);
-        if ((i & 63u) == 0) {
-            if (*abort) return false;
-            if (global_ns() - start > limit_ns) break;
-        }
+    for (;;) {
+        if (mbar_try(bar, parity, kTryNs)) return true;
+        if (*abort) return false;
+        if (global_ns() - start > limit_ns) break;
     }
     *abort = 1;
     atomicOr(&g_tc_error, kErrTimeout);
@@ -157,14 +165,13 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 // Wait for the MMAs this thread has issued, whatever the abort flag says (at most kWaitNs):
 // TMEM is freed only after every tcgen05 operation writing it has completed.
 __device__ __forceinline__ void mbar_drain(uint32_t bar, uint32_t parity) {
+    if (mbar_test(bar, parity)) return;
     const uint64_t start = global_ns();
-    for (uint32_t i = 0; !mbar_test(bar, parity); ++i) {
-        if (i > 64) __nanosleep(32);
-        if ((i & 63u) == 63u && global_ns() - start > kWaitNs) {
+    while (!mbar_try(bar, parity, kTryNs))
+        if (global_ns() - start > kWaitNs) {
             atomicOr(&g_tc_error, kErrTimeout);
             return;
         }
-    }
 }
 
 // L2 policy for data read once and never again in the step (the K/V stream): its lines are
