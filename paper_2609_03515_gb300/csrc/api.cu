@@ -570,7 +570,7 @@ ikv_status ikv_select_budget(int32_t rows, int32_t cap, const float *util, const
         return fail(IKV_ERR_ARG, "util/len/budget/keep/keep_len is NULL");
     // max_holes 0: the kernel never writes pos here
     IKV_TRY_CUDA(launch_select(rows, cap, util, len, rows_per_seq_, budget, const_cast<int32_t *>(pos), keep,
-                               keep_len, DeferArgs{0, cap, nullptr}, sm_count(), stream),
+                               keep_len, DeferArgs{0, cap, nullptr, 0}, sm_count(), stream),
                  "select launch");
     return IKV_OK;
 }
@@ -593,8 +593,9 @@ ikv_status ikv_compact_workspace_size(const ikv_shape *shape, const ikv_cache *c
 static ikv_status compact_impl(const ikv_shape *shape, ikv_cache *cache, const int32_t *keep, const int32_t *keep_len,
                                float *ema, int32_t mode, int32_t *moves, int32_t *n_moves, int32_t *done,
                                cudaStream_t stream, int32_t max_holes = 0, bool by_layer = false,
-                               int32_t *len_out = nullptr) {
+                               int32_t *len_out = nullptr, bool mark = false) {
     CompactArgs a{};
+    a.mark = mark ? 1 : 0;
     a.k = cache->k;
     a.v = cache->v;
     a.pv = view_of(shape, cache);
@@ -777,19 +778,19 @@ static ikv_status zero_control_words(const ikv_params *p, void *ws, const StepWs
 // Step 5: selection, then deferred or immediate compaction.
 static ikv_status evict_impl(const ikv_shape *shape, const ikv_params *p, ikv_cache *cache, float *ema, void *ws,
                              const StepWs &w, cudaStream_t stream, const ikv_timing *tm, bool selected = false,
-                             int32_t *len_out = nullptr) {
+                             int32_t *len_out = nullptr, bool mark = false) {
     const int32_t cap = cap_of(cache);
     const int32_t R = shape->batch * rows_per_seq(shape);
     if (!selected)
         IKV_TRY_CUDA(launch_select(R, cap, ema, cache->len, rows_per_seq(shape), p->budget,
                                    cache->dead_slots ? cache->pos : nullptr, at<int32_t>(ws, w.keep),
-                                   at<int32_t>(ws, w.keep_len), DeferArgs{p->max_holes, cap, cache->start}, sm_count(), stream),
+                                   at<int32_t>(ws, w.keep_len), DeferArgs{p->max_holes, cap, cache->start, 0}, sm_count(), stream),
                      "select launch");
     ikv_status e;
     if (tm && (e = record(tm->select_end, stream))) return e;
     return compact_impl(shape, cache, at<int32_t>(ws, w.keep), at<int32_t>(ws, w.keep_len), ema, p->compact_mode,
                         at<int32_t>(ws, w.moves), at<int32_t>(ws, w.n_moves), at<int32_t>(ws, w.cdone), stream,
-                        p->max_holes, false, len_out);
+                        p->max_holes, false, len_out, mark);
 }
 
 // The selection the score pass may run itself (not under the rank trace, whose raw
@@ -803,7 +804,7 @@ static SelectFuse select_fuse(const ikv_params *p, const ikv_cache *cache, void 
     f.pos = cache->dead_slots ? cache->pos : nullptr;
     f.keep = at<int32_t>(ws, cx.w.keep);
     f.keep_len = at<int32_t>(ws, cx.w.keep_len);
-    f.df = DeferArgs{p->max_holes, cx.cap, cache->start};
+    f.df = DeferArgs{p->max_holes, cx.cap, cache->start, 0};
     return f;
 }
 
@@ -835,7 +836,7 @@ static ikv_status trace_before(const ikv_shape *shape, const ikv_params *p, cons
     const int32_t R = shape->batch * rows_per_seq(shape);
     IKV_TRY_CUDA(launch_select(R, cx.cap, at<float>(ws, cx.w.raw), cache->len, rows_per_seq(shape), p->budget,
                                cache->dead_slots ? cache->pos : nullptr, at<int32_t>(ws, cx.w.keep_raw),
-                               at<int32_t>(ws, cx.w.n_raw), DeferArgs{0, cx.cap, nullptr}, sm_count(), stream),
+                               at<int32_t>(ws, cx.w.n_raw), DeferArgs{0, cx.cap, nullptr, 0}, sm_count(), stream),
                  "trace select launch");
     IKV_TRY_CUDA(launch_trace_gather(trace_args(shape, p, cache, ws, cx), cx.L1, stream), "trace gather launch");
     return IKV_OK;
@@ -890,7 +891,7 @@ static ikv_status layer_evict(const ikv_shape *shape, const ikv_params *p, ikv_c
                  "layer fold launch");
     const int32_t K = shape->layers;
     IKV_TRY_CUDA(launch_select(shape->batch * K, cx.cap, at<float>(ws, cx.w.util), cache->len, K, p->budget, nullptr,
-                               at<int32_t>(ws, cx.w.keep), at<int32_t>(ws, cx.w.keep_len), DeferArgs{0, cx.cap, nullptr},
+                               at<int32_t>(ws, cx.w.keep), at<int32_t>(ws, cx.w.keep_len), DeferArgs{0, cx.cap, nullptr, 0},
                                sm_count(), stream),
                  "select launch");
     return compact_impl(shape, cache, at<int32_t>(ws, cx.w.keep), at<int32_t>(ws, cx.w.keep_len), nullptr,
@@ -960,6 +961,15 @@ ikv_status ikv_step(const ikv_shape *shape, const ikv_params *p, ikv_cache *cach
     rows.book.ema = ema;
     rows.book.init_mean = cx.init_mean;
     rows.book.dead_slots = cache->dead_slots;
+    // utilities untouched by this step's attention: the bookkeeping CTAs select, too
+    const bool ahead = !cx.scoring;
+    if (ahead) {
+        rows.book.select = 1;
+        rows.book.budget = p->budget;
+        rows.book.keep = at<int32_t>(ws, w.keep);
+        rows.book.keep_len = at<int32_t>(ws, w.keep_len);
+        rows.book.df = DeferArgs{p->max_holes, cx.cap, cache->start, 1};
+    }
     bool gsum = false;  // the attention may hand over normalised group sums instead of logits
     if ((e = run_attend(shape, cache, 0, shape->layers, cx.L1, q, out, ws, w.at, cx.scoring, nullptr, nullptr, stream,
                         tm, true, 0, 0, &rows, &gsum)))
@@ -970,14 +980,14 @@ ikv_status ikv_step(const ikv_shape *shape, const ikv_params *p, ikv_cache *cach
     appended.len = len1;
     float *raw = p->trace ? at<float>(ws, w.raw) : nullptr;
     const SelectFuse fs = select_fuse(p, cache, ws, cx);
-    bool selected = false;
+    bool selected = ahead;
     if (cx.scoring && (e = run_score(shape, &appended, shape->layers, cx.elig, cx.n_elig, cx.L1, ws, w.at, p->alpha, ema,
                                      raw, stream, p->agg_mode, p->scorer, cx.sw, 0, false,
                                      p->trace ? nullptr : &fs, &selected, gsum)))
         return e;
     if (tm && (e = record(tm->score_end, stream))) return e;
     if ((e = trace_before(shape, p, &appended, ws, cx, stream))) return e;
-    if ((e = evict_impl(shape, p, &appended, ema, ws, w, stream, tm, selected, cache->len))) return e;
+    if ((e = evict_impl(shape, p, &appended, ema, ws, w, stream, tm, selected, cache->len, ahead))) return e;
     if (tm && (e = record(tm->end, stream))) return e;
     return trace_after(shape, p, cache, ws, cx, stream);
 }

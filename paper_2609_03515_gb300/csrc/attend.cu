@@ -154,7 +154,8 @@ __global__ void __launch_bounds__(kAttendThreads, 2) attend_f32_kernel(const Att
     int bid = blockIdx.x;
     if (a.book.on) {
         if (bid < a.batch) {
-            book_sequence<kAttendThreads>(a.book, a.len, a.pv.start, a.cap, a.rows_per_seq, bid, &g_attend_error);
+            book_sequence<kAttendThreads>(a.book, a.len, a.pv.start, a.cap, a.rows_per_seq, bid, &g_attend_error,
+                                          reinterpret_cast<uint32_t *>(smem), C::kRing / 4);
             return;
         }
         bid -= a.batch;
@@ -422,7 +423,8 @@ __global__ void __launch_bounds__(kAttendThreads, Bf16Cfg<D>::kCtasPerSm) attend
     int bid = blockIdx.x;
     if (a.book.on) {
         if (bid < a.batch) {
-            book_sequence<kAttendThreads>(a.book, a.len, a.pv.start, a.cap, a.rows_per_seq, bid, &g_attend_error);
+            book_sequence<kAttendThreads>(a.book, a.len, a.pv.start, a.cap, a.rows_per_seq, bid, &g_attend_error,
+                                          reinterpret_cast<uint32_t *>(smem), C::kRing / 4);
             return;
         }
         bid -= a.batch;

@@ -270,7 +270,8 @@ __global__ void __launch_bounds__(kThreads, 2)
     int bid = blockIdx.x;
     if (a.book.on) {
         if (bid < a.batch) {
-            book_sequence<kThreads>(a.book, a.len, a.start, a.cap, a.rows_per_seq, bid, &g_tc_error);
+            book_sequence<kThreads>(a.book, a.len, a.start, a.cap, a.rows_per_seq, bid, &g_tc_error,
+                                    reinterpret_cast<uint32_t *>(sm), kNst * kStage / 4);
             return;
         }
         bid -= a.batch;

@@ -1,6 +1,7 @@
 // The bookkeeping of a step's append, done by extra CTAs of its attention launch.
 #pragma once
 #include "merge.cuh"
+#include "select_row.cuh"
 
 namespace ikv {
 namespace {
@@ -9,10 +10,12 @@ namespace {
 // over the live slots of its row), next_pos, and len1[b] = the length with it, which the step's later
 // kernels read; len[b] itself is left to the compaction, because the attention CTAs that run
 // beside this one work from it (slot len[b] is the new token's, live whatever pos still says
-// there).  No room: len1[b] = len[b] and bit 2 of *err.
+// there).  No room: len1[b] = len[b] and bit 2 of *err.  With k.select it then selects the
+// sequence's rows, hidden behind the attention (a kernel of its own after it cost 5 us a step);
+// keys, keys_cap: the CTA's shared memory for their keys.
 template <int NT>
 __device__ __noinline__ void book_sequence(const BookArgs &k, const int32_t *len, const int32_t *start, int32_t cap,
-                                              int32_t rows_per_seq, int b, unsigned int *err) {
+                                           int32_t rows_per_seq, int b, unsigned int *err, uint32_t *keys, int keys_cap) {
     constexpr int NW = NT / 32, U = 8;
     __shared__ float scratch[2][NW];
     const int tid = threadIdx.x;
@@ -65,6 +68,13 @@ __device__ __noinline__ void book_sequence(const BookArgs &k, const int32_t *len
         if (room) k.next_pos[b] += 1;
         else atomicOr(err, 4u);  // the token was not stored; ikv_device_status reports it
         k.len1[b] = L + (room ? 1 : 0);
+    }
+    if (!k.select) return;
+    __syncthreads();  // the new token's utility and position
+    for (int rr = 0; rr < rows_per_seq; ++rr) {
+        select_row<NT>(0, 1, b * rows_per_seq + rr, L + (room ? 1 : 0), cap, k.ema, rows_per_seq, k.budget,
+                       k.dead_slots ? k.pos : nullptr, k.keep, k.keep_len, k.df, keys, keys_cap);
+        __syncthreads();  // its shared memory is reused
     }
 }
 

@@ -93,6 +93,12 @@ __device__ __forceinline__ void keep_length(const CompactArgs &a, int b) {
     if (a.len_out != a.len) a.len_out[b] = a.len[b];
 }
 
+// Utility row rr of sequence b, whose victim the selection only named: marked dead.
+__device__ __forceinline__ void mark_victim(const CompactArgs &a, int b, int rr) {
+    const int64_t row = ((int64_t)b * a.rows_per_seq + rr) * a.cap;
+    if (a.mark) a.pos[row + a.keep[row]] = -1;
+}
+
 // Deferred compaction: sequence b only marks its evicted slots dead while its dead
 // slots (the ones already dead plus this step's evictions: len - kept) stay within
 // max_holes.  Every row of b keeps the same number of slots, so row b * rps decides.
@@ -125,8 +131,9 @@ __device__ __forceinline__ void compact_stable_item(const CompactArgs &a, const 
     const int tid = threadIdx.x;
     const int kvh = a.pv.kv_heads;
     const int nkv = a.layers * kvh;
-    if (a.keep_len[b * a.rows_per_seq] < 0) {  // selection marked the victim dead: nothing to do
+    if (a.keep_len[b * a.rows_per_seq] < 0) {  // the victim is only marked dead: nothing moves
         if (x == 0 && tid == 0) keep_length(a, b);
+        if (x >= nkv && tid == 0) mark_victim(a, b, x - nkv);
         return;
     }
     const int L = a.len[b];
@@ -335,7 +342,11 @@ __global__ void __launch_bounds__(kCompThreads, 3) compact_stable_strided_kernel
             const int64_t item = blockIdx.x + (int64_t)(k0 + threadIdx.x) * gridDim.x;
             const int b = (int)(item / nx);
             flagged[threadIdx.x] = item < n_items ? a.keep_len[b * a.rows_per_seq] < 0 : 1;
-            if (item < n_items && flagged[threadIdx.x] && item % nx == 0) keep_length(a, b);
+            if (item < n_items && flagged[threadIdx.x]) {
+                const int x = (int)(item % nx), nkv = a.layers * a.pv.kv_heads;
+                if (x == 0) keep_length(a, b);
+                if (x >= nkv) mark_victim(a, b, x - nkv);
+            }
         }
         __syncthreads();
 #pragma unroll 1
@@ -401,8 +412,9 @@ __global__ void __launch_bounds__(kCompThreads) holefill_move_kernel(const Compa
     const int b = blockIdx.y, x = blockIdx.x;
     const int kvh = a.pv.kv_heads;
     const int nkv = a.layers * kvh;
-    if (a.keep_len[b * a.rows_per_seq] < 0) {  // selection marked the victim dead: nothing to do
+    if (a.keep_len[b * a.rows_per_seq] < 0) {  // the victim is only marked dead: nothing moves
         if (x == 0 && tid == 0) keep_length(a, b);
+        if (x >= nkv && tid == 0) mark_victim(a, b, x - nkv);
         return;
     }
     if (x < nkv) {

@@ -85,6 +85,17 @@ struct PagedView {
     }
 };
 
+// Deferred compaction inside selection: when a row has exactly one slot too many and
+// the sequence may defer (len - budget <= max_holes and start + len < cap), select
+// marks the victim dead itself and writes keep_len = -1 - budget, which tells the
+// compaction kernels that nothing moves.  max_holes = 0 disables it.
+struct DeferArgs {
+    int32_t max_holes;
+    int32_t cap;
+    const int32_t *start;       // [batch] or null
+    int32_t later;              // nonzero: only name the victim, in keep[r][0]; the compaction marks it
+};
+
 // A step's append, by extra CTAs of its attention launch (book.cuh)
 struct BookArgs {
     int32_t on;                 // nonzero: they run, and len is the length before the append
@@ -92,6 +103,12 @@ struct BookArgs {
     int32_t *pos, *next_pos;
     float *ema;
     int32_t init_mean, dead_slots;
+    // nonzero: they also select each row's survivors -- on steps that leave the utilities as
+    // they are, the selection does not depend on the attention
+    int32_t select;
+    const int32_t *budget;      // [batch]
+    int32_t *keep, *keep_len;   // [rows][cap], [rows]
+    DeferArgs df;               // later: the attention beside them still reads the positions
 };
 
 struct AttendArgs {
@@ -131,16 +148,6 @@ struct AttendArgs {
     // tensor-core kernel: the launch may set up and start its K/V stream before the
     // programmatic-dependency wait (see TcArgs::early)
     int32_t early;
-};
-
-// Deferred compaction inside selection: when a row has exactly one slot too many and
-// the sequence may defer (len - budget <= max_holes and start + len < cap), select
-// marks the victim dead itself and writes keep_len = -1 - budget, which tells the
-// compaction kernels that nothing moves.  max_holes = 0 disables it.
-struct DeferArgs {
-    int32_t max_holes;
-    int32_t cap;
-    const int32_t *start;       // [batch] or null
 };
 
 struct ScoreArgs {
@@ -257,6 +264,7 @@ struct CompactArgs {
     const int32_t *keep, *keep_len;
     int32_t *moves;             // hole-fill: [rows][cap][2] (src, dst), null for stable
     int32_t *n_moves;           // hole-fill: [rows]
+    int32_t mark;               // flagged rows (keep_len < 0): the victim keep[r][0] is still to be marked dead
     int32_t max_holes;          // > 0: while a sequence's dead slots stay <= max_holes, mark
                                 // the evicted slots dead (pos = -1) instead of compacting
     float *vnorm;               // [layers][batch][kv_heads][cap] value-row norms moved with the rows, or null

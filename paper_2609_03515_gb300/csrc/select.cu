@@ -30,13 +30,14 @@ constexpr int kSelKeysMax = 48 * 1024;  // keys a CTA keeps in shared memory
 
 template <int NT>
 __global__ void __launch_bounds__(NT, NT == 1024 ? 1 : 2)
-    select_kernel(int32_t cap, const float *__restrict__ util, const int32_t *__restrict__ len, int32_t rps,
+    select_kernel(int32_t cap, const float *util, const int32_t *__restrict__ len, int32_t rps,
                   const int32_t *__restrict__ budget, int32_t *pos, int32_t *keep, int32_t *keep_len, DeferArgs df,
                   int32_t ctas, int32_t keys_cap) {
     extern __shared__ uint32_t keys[];
     pdl_wait();
-    select_row<NT>(blockIdx.x % ctas, ctas, blockIdx.x / ctas, cap, util, len, rps, budget, pos, keep, keep_len, df,
-                   keys, keys_cap);
+    const int r = blockIdx.x / ctas;
+    select_row<NT>(blockIdx.x % ctas, ctas, r, len[r / rps], cap, util, rps, budget, pos, keep, keep_len, df, keys,
+                   keys_cap);
 }
 
 }  // namespace

@@ -49,14 +49,17 @@ constexpr int kSelMaxCtas = 8;  // CTAs that share a row (portable cluster size)
 // one is its `rank`-th), entered by all of their threads.  CTA `rank` owns a contiguous C-th of
 // the row's slots and keeps their keys in keys[0, keys_cap) (shared memory) when they fit;
 // otherwise every sweep reads the row again, a few loads in flight a thread.
+// L: the row's slots in use.
 template <int NT>
-__device__ __forceinline__ void select_row(int rank, int C, int r, int32_t cap, const float *__restrict__ util,
-                                           const int32_t *__restrict__ len, int32_t rps,
+__device__ __forceinline__ void select_row(int rank, int C, int r, int L, int32_t cap, const float *util, int32_t rps,
                                            const int32_t *__restrict__ budget, int32_t *pos, int32_t *keep,
                                            int32_t *keep_len, DeferArgs df, uint32_t *keys, int keys_cap) {
-    static_assert(NT >= 256 && NT % 32 == 0, "the digit scan needs 256 threads at least, whole warps");
+    static_assert(NT % 32 == 0 && NT <= 1024, "whole warps");
     constexpr int NW = NT / 32;
     constexpr int U = NT == 256 ? 4 : 8;  // keys a thread has in flight
+    constexpr int DT = NT < 256 ? NT : 256;                   // threads of the digit scan,
+    constexpr int DPT = (256 + DT - 1) / DT;                  // and the digits each of them holds
+    static_assert(DT % 32 == 0, "whole warps");
     __shared__ uint32_t hist[2][256];
     __shared__ uint32_t warp_a[NW], warp_b[NW];
     __shared__ unsigned long long warp_min[NW], s_min;
@@ -65,7 +68,6 @@ __device__ __forceinline__ void select_row(int rank, int C, int r, int32_t cap, 
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b = r / rps;
-    const int L = len[b];
     const int B = max(budget[b], 0);
     const int S = df.start ? df.start[b] : 0;
     const int seg = (L + C - 1) / C;
@@ -155,7 +157,9 @@ __device__ __forceinline__ void select_row(int rank, int C, int r, int32_t cap, 
         // deferred compaction (the rule the compaction kernels apply): the victim is
         // only marked dead, and keep_len < 0 tells compaction that nothing moves
         if (rank == 0 && tid == 0) {
-            pr[(int)(~(uint32_t)(best & 0xFFFFFFFFull))] = -1;
+            const int ev = (int)(~(uint32_t)(best & 0xFFFFFFFFull));
+            if (df.later) kp[0] = ev;
+            else pr[ev] = -1;
             keep_len[r] = -1 - B;
         }
         if (C > 1) cluster_sync();  // a CTA may not leave while another reads its shared memory
@@ -195,16 +199,22 @@ __device__ __forceinline__ void select_row(int rank, int C, int r, int32_t cap, 
                 }
                 sync_all();
                 // (every CTA is past its reads of the other buffer)
-                uint32_t v = 0u, x = 0u;
-                if (tid < 256) {
-                    hist[(pass & 1) ^ 1][tid] = 0u;
-                    // inclusive counts from the top digit down: thread t holds digit 255 - t
-                    uint32_t w[kSelMaxCtas];
+                // inclusive counts from the top digit down: thread t holds digits from 255 - t DPT down
+                uint32_t v[DPT], x = 0u;
+                if (tid < DT) {
 #pragma unroll
-                    for (int c = 0; c < kSelMaxCtas; ++c) w[c] = c < C ? peer(&h[255 - tid], c) : 0u;
+                    for (int q = 0; q < DPT; ++q) {
+                        const int d = 255 - (tid * DPT + q);
+                        v[q] = 0u;
+                        if (d < 0) continue;
+                        hist[(pass & 1) ^ 1][d] = 0u;
+                        uint32_t w[kSelMaxCtas];
 #pragma unroll
-                    for (int c = 0; c < kSelMaxCtas; ++c) v += w[c];
-                    x = v;
+                        for (int c = 0; c < kSelMaxCtas; ++c) w[c] = c < C ? peer(&h[d], c) : 0u;
+#pragma unroll
+                        for (int c = 0; c < kSelMaxCtas; ++c) v[q] += w[c];
+                        x += v[q];
+                    }
 #pragma unroll
                     for (int o = 1; o < 32; o <<= 1) {
                         const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
@@ -213,14 +223,17 @@ __device__ __forceinline__ void select_row(int rank, int C, int r, int32_t cap, 
                     if (lane == 31) warp_a[warp] = x;
                 }
                 __syncthreads();
-                if (tid < 256) {
-                    uint32_t before = 0u;
-                    for (int w = 0; w < warp; ++w) before += warp_a[w];
-                    const uint32_t incl = before + x;
-                    if (incl - v < k && incl >= k) {  // exactly one digit satisfies this
-                        s_digit = 255u - (uint32_t)tid;
-                        s_above = incl - v;
-                        s_whole = incl == k;
+                if (tid < DT) {
+                    uint32_t incl = x;
+                    for (int w = 0; w < warp; ++w) incl += warp_a[w];
+#pragma unroll
+                    for (int q = DPT - 1; q >= 0; --q) {  // incl: through digit q of the thread's
+                        if (incl - v[q] < k && incl >= k) {  // exactly one digit satisfies this
+                            s_digit = 255u - (uint32_t)(tid * DPT + q);
+                            s_above = incl - v[q];
+                            s_whole = incl == k;
+                        }
+                        incl -= v[q];
                     }
                 }
                 __syncthreads();
