@@ -20,9 +20,6 @@ namespace {
 __device__ __forceinline__ void cp_async16_n(uint32_t smem, const void *gmem, uint32_t n) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(smem), "l"(gmem), "r"(n) : "memory");
 }
-__device__ __forceinline__ void cp_async16_zfill(void *smem, const void *gmem, bool in) {
-    cp_async16_n(static_cast<uint32_t>(__cvta_generic_to_shared(smem)), gmem, in ? 16u : 0u);
-}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
@@ -111,40 +108,63 @@ __device__ __forceinline__ void store_empty(const AttendArgs &a, int G, int D, i
         a.lse2[((int64_t)b * a.sc_layers + a.sc_layer0 + li) * a.q_heads + (int64_t)g * G + threadIdx.x] = -INFINITY;
 }
 
+// N consecutive floats of shared memory, N * 4 bytes aligned (16 at most)
+template <int N>
+__device__ __forceinline__ void load_vec(const float *p, float (&x)[N]) {
+    if constexpr (N == 1) {
+        x[0] = *p;
+    } else if constexpr (N == 2) {
+        const float2 y = *reinterpret_cast<const float2 *>(p);
+        x[0] = y.x;
+        x[1] = y.y;
+    } else {
+#pragma unroll
+        for (int i = 0; i < N / 4; ++i) {
+            const float4 y = reinterpret_cast<const float4 *>(p)[i];
+            x[4 * i] = y.x;
+            x[4 * i + 1] = y.y;
+            x[4 * i + 2] = y.z;
+            x[4 * i + 3] = y.w;
+        }
+    }
+}
+
 // fp32 K/V.  HBM bound: a K and V byte costs G / 4 FMAs, half an SM's rate at G = 8.  Every
-// warp is on its own: it takes every fourth group of 8 (d = 128) or 16 (d = 64) tokens of
+// warp is on its own: it takes every fourth group of T (d = 128) or 2 T (d = 64) tokens of
 // the split through its own cp.async ring and keeps its own online softmax, so the loop has
 // no block barrier, and each lane reads back the 16 bytes of each row that it copied itself.
-// A lane's partial dot products of 8 tokens x G heads are summed over the row's lanes by a
+// A lane's partial dot products of T tokens x G heads are summed over the row's lanes by a
 // halving exchange (one shuffle a value instead of five), which leaves each lane with the
 // logits it exponentiates; the probabilities go through a few hundred bytes of shared memory
-// to the P.V products.  8 warps an SM (two CTAs) keep 128 KB in flight.  Measured, a whole
-// step of b = 4, 8 layers, 16 / 4 heads of 128, 2048 tokens (269 MB, 39.7 us at the copy
-// rate): 185.1 -> 76.9 us against attend_split_kernel, which ran one CTA of four warps an
-// SM with five block barriers per 64-token tile; tiny steps save the combine launch.
+// to the P.V products.  Measured, a whole step of b = 4, 8 layers, 16 / 4 heads of 128, 2048
+// tokens (269 MB, 39.7 us at the copy rate): 185.1 -> 76.9 us against a kernel of one CTA of
+// four warps an SM with five block barriers per 64-token tile.  Warps hide the rest, not deep
+// rings: two CTAs of three stages an SM 72.7 us, three of two stages 61.8 (G = 4; four of
+// T = 4 and three stages 65.4); at G = 8, whose logits of 8 tokens fill the registers, two
+// CTAs 89.8 us, three with T = 4 and four stages 81.4.
 template <int D, int G>
 struct F32Cfg {
     static constexpr int GP = G == 7 ? 8 : G;
     static constexpr int RL = D / 4;              // lanes of a row (16 bytes each)
     static constexpr int RPI = 32 / RL;           // rows a warp reads at once
-    static constexpr int T = 8;                   // tokens per group and row slot
+    static constexpr int T = G <= 4 ? 8 : 4;      // tokens per group and row slot
     static constexpr int TW = T * RPI;            // tokens per warp and group
     static constexpr int kRowB = D * 4;
     static constexpr int kStageB = 2 * TW * kRowB;
-    static constexpr int NST = 3;
+    static constexpr int NST = G <= 4 ? 2 : 4;
     static constexpr int kWarps = kAttendThreads / 32;
     static constexpr int kRing = kWarps * NST * kStageB;
     static constexpr int P = kWarps * RPI;        // independent softmaxes of a CTA
     static constexpr int N = T * GP;              // logits of a group per row slot
     static constexpr int VPL = N > RL ? N / RL : 1;   // logits a lane ends up with
     static constexpr int DUP = N < RL ? RL / N : 1;   // lanes holding the same logit
-    static constexpr int kPw = RPI * (T + 1) * GP;    // floats per warp: probabilities, rescales
+    static constexpr int kPw = (RPI * (T + 1) * GP + 3) / 4 * 4;  // floats per warp: probabilities, rescales
     static constexpr int kSmemBytes = kRing + (kWarps * kPw + 2 * P * GP) * 4;
     static_assert(P * G * D * 4 <= kRing && kWarps * kMaxSplits * 4 <= kRing, "the merge reuses the ring");
 };
 
 template <int D, int G>
-__global__ void __launch_bounds__(kAttendThreads, 2) attend_f32_kernel(const AttendArgs a) {
+__global__ void __launch_bounds__(kAttendThreads, kF32CtasPerSm) attend_f32_kernel(const AttendArgs a) {
     using C = F32Cfg<D, G>;
     constexpr int GP = C::GP, T = C::T, TW = C::TW, NST = C::NST, VPL = C::VPL, DUP = C::DUP;
     pdl_wait();
@@ -193,20 +213,24 @@ __global__ void __launch_bounds__(kAttendThreads, 2) attend_f32_kernel(const Att
     const int64_t unit = ((int64_t)li * a.batch + b) * a.pv.kv_heads + g;
     const unsigned char *kn = reinterpret_cast<const unsigned char *>(a.k_new) + unit * C::kRowB + lr * 16;
     const unsigned char *vn = reinterpret_cast<const unsigned char *>(a.v_new) + unit * C::kRowB + lr * 16;
-    // pool row of token lane % TW of the warp's group j (-1 past the split, -2 the new token), one
-    // per lane; looked up one group ahead of its use, so the block table's latency is off the path
-    auto lookup = [&](int j) -> int64_t {
+    // pool row of token lane % TW of the warp's group j (kNoRow past the split, kNewRow the new
+    // token; a row index fits 32 bits: rows are 256 bytes at least), one per lane; looked up one
+    // group ahead of its use, so the block table's latency is off the path
+    constexpr uint32_t kNoRow = ~0u, kNewRow = ~0u - 1u;
+    auto lookup = [&](int j) -> uint32_t {
         const int tok = t0 + (warp + C::kWarps * j) * TW + lane % TW;
-        return j < mine && tok < t1 ? tok == t_new ? -2 : a.pv.row_phys(b, l, g, S0 + tok) : -1;
+        return j < mine && tok < t1 ? tok == t_new ? kNewRow : (uint32_t)a.pv.row_phys(b, l, g, S0 + tok) : kNoRow;
     };
-    auto issue = [&](int j, int64_t row) {
-        unsigned char *st = ring + (j % NST) * C::kStageB + half * T * C::kRowB + lr * 16;
+    const uint32_t ring_u = static_cast<uint32_t>(__cvta_generic_to_shared(ring)) + half * T * C::kRowB + lr * 16;
+    auto issue = [&](int stage, uint32_t row) {
+        const uint32_t st = ring_u + stage * C::kStageB;
 #pragma unroll
         for (int t = 0; t < T; ++t) {
-            const int64_t r = __shfl_sync(0xffffffffu, row, half * T + t);
-            const int64_t at = (r < 0 ? 0 : r) * C::kRowB;
-            cp_async16_zfill(st + t * C::kRowB, r == -2 ? kn : kb + at, r != -1);
-            cp_async16_zfill(st + (TW + t) * C::kRowB, r == -2 ? vn : vb + at, r != -1);
+            const uint32_t r = __shfl_sync(0xffffffffu, row, half * T + t);
+            const uint32_t n = r == kNoRow ? 0u : 16u;
+            const uint64_t at = (uint64_t)(r >= kNewRow ? 0u : r) * C::kRowB;
+            cp_async16_n(st + t * C::kRowB, r == kNewRow ? kn : kb + at, n);
+            cp_async16_n(st + (TW + t) * C::kRowB, r == kNewRow ? vn : vb + at, n);
         }
     };
 #pragma unroll
@@ -214,7 +238,7 @@ __global__ void __launch_bounds__(kAttendThreads, 2) attend_f32_kernel(const Att
         issue(i, lookup(i));
         cp_async_commit();
     }
-    int64_t row_next = lookup(NST - 1);
+    uint32_t row_next = lookup(NST - 1);
     if (warp == 0 && t_new >= t0 && t_new < t1)  // into the cache, for later steps
         store_new_rows<float, D>(a, unit, a.pv.row_phys(b, l, g, S0 + t_new),
                                  a.vnorm ? a.vnorm + (((int64_t)l * a.batch + b) * a.pv.kv_heads + g) * a.cap + t_new : nullptr);
@@ -254,14 +278,16 @@ __global__ void __launch_bounds__(kAttendThreads, 2) attend_f32_kernel(const Att
     };
     uint32_t live_next = live_of(0);
 
+    int stage = 0;
     for (int i = 0; i < mine; ++i) {
-        if (i + NST - 1 < mine) issue(i + NST - 1, row_next);
+        if (i + NST - 1 < mine) issue(stage == 0 ? NST - 1 : stage - 1, row_next);
         cp_async_commit();
         row_next = lookup(i + NST);
         const uint32_t live = live_next;
         live_next = live_of(i + 1);
         cp_async_wait<NST - 1>();
-        const unsigned char *st = ring + (i % NST) * C::kStageB + half * T * C::kRowB + lr * 16;
+        const unsigned char *st = ring + stage * C::kStageB + half * T * C::kRowB + lr * 16;
+        stage = stage == NST - 1 ? 0 : stage + 1;
         float z[C::N];
 #pragma unroll
         for (int t = 0; t < T; ++t) {
@@ -325,9 +351,11 @@ __global__ void __launch_bounds__(kAttendThreads, 2) attend_f32_kernel(const Att
 #pragma unroll
         for (int t = 0; t < T; ++t) {
             const float4 v = *reinterpret_cast<const float4 *>(st + (TW + t) * C::kRowB);
+            float pt[GP];
+            load_vec<GP>(p_s + (half * T + t) * GP, pt);
 #pragma unroll
             for (int h = 0; h < G; ++h) {
-                const float p = p_s[(half * T + t) * GP + h];
+                const float p = pt[h];
                 o[h][0] = fmaf(p, v.x, o[h][0]);
                 o[h][1] = fmaf(p, v.y, o[h][1]);
                 o[h][2] = fmaf(p, v.z, o[h][2]);

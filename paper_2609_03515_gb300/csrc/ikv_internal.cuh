@@ -233,7 +233,7 @@ cudaError_t launch_attend_tc(const AttendArgs &a, const TcOutputs &o, int group,
 
 // launchers (return cudaError_t of the launch)
 // CTAs of its kernels an SM holds (shared memory)
-constexpr int kF32CtasPerSm = 2, kBf16D64CtasPerSm = 4, kBf16D128CtasPerSm = 2;
+constexpr int kF32CtasPerSm = 3, kBf16D64CtasPerSm = 4, kBf16D128CtasPerSm = 2;
 cudaError_t launch_attend(const AttendArgs &a, int dtype, int head_dim, int group, cudaStream_t st);
 cudaError_t launch_score_ema(const ScoreArgs &a, int32_t max_len, int sms, cudaStream_t st);
 // token blocks (and tokens per lane V) the score pass uses for max_len
