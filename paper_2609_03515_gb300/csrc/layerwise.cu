@@ -93,64 +93,85 @@ __global__ void __launch_bounds__(kInvThreads) layer_inverse_kernel(const LayerA
     if (p >= 0 && p < a.pos_cap) a.inv[((int64_t)b * a.layers + l) * a.pos_cap + p] = j;
 }
 
-// One thread per live token position p (held by some layer): walks the layers in
-// order; at every eligible layer of a refresh step m <- alpha m + (1 - alpha) s, s the
+// LG lanes per live token position p (held by some layer), each for up to NB consecutive
+// layers: at every eligible layer of a refresh step m <- alpha m + (1 - alpha) s, s the
 // layer's pooled score of p if it holds p, else 0; each layer holding p gets m as its
 // utility of p's slot.  The final m is stored.  Dead positions are left as they are.
+// A lane folds its layers from zero; the lanes of a position compose those affine maps in
+// layer order (shuffles), which gives each the m that enters its layers.  Bound by the
+// instructions of a lane's chain: one lane walking 32 layers took 12 us at 32 layers x 3.3k
+// slots, its loads batched however (a step 116.8 us, 110.8 this way).
 constexpr int kFoldThreads = 256;
-// 8, 16 and 32 measured alike (~15 us per fold at 32 layers x 3.3k slots): past the first
-// batch the fold is bound by its scattered reads, not by their latency chain
-#ifndef IKV_FOLD_BATCH
-#define IKV_FOLD_BATCH 8
-#endif
-constexpr int kFoldBatch = IKV_FOLD_BATCH;  // layers whose lookups are in flight together
+template <int LG, int NB>
 __global__ void __launch_bounds__(kFoldThreads) layer_fold_kernel(const LayerArgs a) {
     pdl_wait();
+    constexpr int PP = 32 / LG;  // positions per warp
+    const int lane = threadIdx.x & 31;
+    const int grp = lane / PP, sub = lane % PP;
     const int b = blockIdx.y;
-    const int p = blockIdx.x * kFoldThreads + threadIdx.x;
-    if (p >= a.next_pos[b] || p >= a.pos_cap) return;
-    if (!((__ldg(a.live + (int64_t)b * a.live_words + (p >> 5)) >> (p & 31)) & 1u)) return;
+    const int p = (blockIdx.x * (kFoldThreads / 32) + (threadIdx.x >> 5)) * PP + sub;
+    const bool on = p < a.next_pos[b] && p < a.pos_cap &&
+                    ((__ldg(a.live + (int64_t)b * a.live_words + (p >> 5)) >> (p & 31)) & 1u);
+    if (!__any_sync(0xffffffffu, on)) return;
     const int L = a.len[b];
     float *mp = a.m + (int64_t)b * a.pos_cap + p;
-    float m = *mp;
-    int k = 0;  // eligible layers folded so far
-    for (int l0 = 0; l0 < a.layers; l0 += kFoldBatch) {
-        // the batch's slot lookups, then their checks and scores, all issued before use
-        int j[kFoldBatch];
-        bool held[kFoldBatch];
-        float sc[kFoldBatch];
+    float m = on ? *mp : 0.f;
+    const int per = (a.layers + LG - 1) / LG;
+    const int l0 = grp * per, l1 = min(l0 + per, a.layers);
+    const int64_t row0 = (int64_t)b * a.layers + l0;
+    // the lane's slot lookups, then their checks and scores, all issued before use
+    int j[NB];
+    const int32_t *ip = a.inv + row0 * a.pos_cap + p;
 #pragma unroll
-        for (int u = 0; u < kFoldBatch; ++u) {
-            const int l = l0 + u;
-            j[u] = l < a.layers ? __ldg(a.inv + ((int64_t)b * a.layers + l) * a.pos_cap + p) : -1;
-        }
+    for (int u = 0; u < NB; ++u, ip += a.pos_cap) j[u] = on && l0 + u < l1 ? __ldg(ip) : -1;
+    uint32_t held = 0u, elig = 0u;
+    const int32_t *pp = a.pos + row0 * a.cap;
 #pragma unroll
-        for (int u = 0; u < kFoldBatch; ++u) {
-            const int64_t row = (int64_t)b * a.layers + l0 + u;
-            held[u] = j[u] >= 0 && j[u] < L && __ldg(a.pos + row * a.cap + j[u]) == p;
-        }
-        int kk = k;
+    for (int u = 0; u < NB; ++u, pp += a.cap)
+        if (j[u] >= 0 && j[u] < L && __ldg(pp + j[u]) == p) held |= 1u << u;
+    float sc[NB];
+    if (a.scoring) {
+        int k = 0;  // eligible layers before the lane's
+        for (int l = 0; l < l0; l += 32)
+            k += __popc(a.elig_bits[l >> 5] & (l0 - l >= 32 ? ~0u : (1u << (l0 - l)) - 1u));
+        const float *sp = a.sbuf + ((int64_t)b * a.n_elig + k) * a.lstride;
 #pragma unroll
-        for (int u = 0; u < kFoldBatch; ++u) {
+        for (int u = 0; u < NB; ++u) {
             const int l = l0 + u;
             sc[u] = 0.f;
-            if (l < a.layers && a.scoring && ((a.elig_bits[l >> 5] >> (l & 31)) & 1u)) {
-                if (held[u]) sc[u] = __ldg(a.sbuf + ((int64_t)b * a.n_elig + kk) * a.lstride + j[u]);
-                ++kk;
+            if (l < l1 && ((a.elig_bits[l >> 5] >> (l & 31)) & 1u)) {
+                elig |= 1u << u;
+                if ((held >> u) & 1u) sc[u] = __ldg(sp + j[u]);
+                sp += a.lstride;
             }
-        }
-#pragma unroll
-        for (int u = 0; u < kFoldBatch; ++u) {
-            const int l = l0 + u;
-            if (l >= a.layers) break;
-            if (a.scoring && ((a.elig_bits[l >> 5] >> (l & 31)) & 1u)) {
-                m = a.alpha * m + (1.f - a.alpha) * sc[u];
-                ++k;
-            }
-            if (held[u]) a.util[((int64_t)b * a.layers + l) * a.cap + j[u]] = m;
         }
     }
-    *mp = m;
+    const float beta = 1.f - a.alpha;
+    float f = 1.f, c = 0.f;  // the lane's layers: m -> f m + c
+#pragma unroll
+    for (int u = 0; u < NB; ++u)
+        if ((elig >> u) & 1u) {
+            c = a.alpha * c + beta * sc[u];
+            f *= a.alpha;
+        }
+#pragma unroll
+    for (int g = 0; g < LG - 1; ++g) {
+        const float fg = __shfl_sync(0xffffffffu, f, g * PP + sub), cg = __shfl_sync(0xffffffffu, c, g * PP + sub);
+        if (g < grp) m = fg * m + cg;
+    }
+    float *up = a.util + row0 * a.cap;
+#pragma unroll
+    for (int u = 0; u < NB; ++u, up += a.cap) {
+        if ((elig >> u) & 1u) m = a.alpha * m + beta * sc[u];
+        if ((held >> u) & 1u) up[j[u]] = m;
+    }
+    if (on && grp == LG - 1) *mp = m;
+}
+
+template <int LG, int NB>
+cudaError_t launch_fold(const LayerArgs &a, int32_t max_pos, cudaStream_t st) {
+    constexpr int kPos = kFoldThreads / LG;  // positions of a CTA
+    return launch_k(layer_fold_kernel<LG, NB>, dim3((max_pos + kPos - 1) / kPos, a.batch), dim3(kFoldThreads), 0, st, a);
 }
 
 }  // namespace
@@ -173,8 +194,11 @@ cudaError_t launch_layer_fold(const LayerArgs &a, int32_t max_len, int32_t max_p
                              dim3(kInvThreads), 0, st, a);
     note_launch();
     if (e != cudaSuccess) return e;
-    e = launch_k(layer_fold_kernel, dim3((max_pos + kFoldThreads - 1) / kFoldThreads, a.batch), dim3(kFoldThreads), 0,
-                 st, a);
+    // lanes per position for at most eight layers each (16 beyond 256 layers)
+    e = a.layers <= 32 ? launch_fold<4, 8>(a, max_pos, st)
+        : a.layers <= 64 ? launch_fold<8, 8>(a, max_pos, st)
+        : a.layers <= 128 ? launch_fold<16, 8>(a, max_pos, st)
+                          : launch_fold<32, 16>(a, max_pos, st);
     note_launch();
     return e != cudaSuccess ? e : cudaGetLastError();
 }
