@@ -304,6 +304,14 @@ __global__ void __launch_bounds__(kScoreThreads, 4) score_kernel(const ScoreArgs
             a.sel_pos[(int64_t)r * a.cap + (int)(~(uint32_t)(s_best & 0xFFFFFFFFull))] = -1;
             a.keep_len[r] = -1 - B;
         }
+    } else if (n_live == L && n_live <= B + 1) {
+        // no dead slot and at most one to go: the partials name it, the row need not be read
+        const int kept = min(n_live, B), ev = kept == n_live ? L : (int)(~(uint32_t)(s_best & 0xFFFFFFFFull));
+        int32_t *kp = a.keep + (int64_t)r * a.cap;
+        if (kept > 0)
+            for (int i = threadIdx.x; i < L; i += kScoreThreads)
+                if (i != ev) kp[i < ev ? i : i - 1] = i;
+        if (threadIdx.x == 0) a.keep_len[r] = kept;
     } else {
         select_row<kScoreThreads>(0, 1, r, L, a.cap, a.ema, a.rows_per_seq, a.budget, a.sel_pos, a.keep, a.keep_len,
                                   a.df, reinterpret_cast<uint32_t *>(wsm), a.sel_keys);

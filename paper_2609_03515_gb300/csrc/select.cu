@@ -51,22 +51,19 @@ cudaError_t launch_select(int32_t rows, int32_t cap, const float *util, const in
     while (C > 1 && ((int64_t)rows * C > 2 * sms || (int64_t)C * kSelSlots > cap)) C >>= 1;
     const int seg = (cap + C - 1) / C;
     const int32_t keys_cap = seg < kSelKeysMax ? seg : kSelKeysMax;
-    static bool limit_set = false;
-    if (!limit_set) {
-        const int bytes = kSelKeysMax * (int)sizeof(uint32_t);
-        cudaError_t e = cudaFuncSetAttribute(select_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(select_kernel<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        if (e != cudaSuccess) return e;
-        limit_set = true;
-    }
     // threads for about one batch of eight keys each: more warps would issue the same predicated
     // batches for nothing (one row of 1096 slots: 14.3 us with 1024 threads, 10.2 with 256)
     const int nt = seg <= 2048 ? 256 : C > 1 || seg <= 4608 ? 512 : 1024;
+    auto kernel = nt == 256 ? select_kernel<256> : nt == 512 ? select_kernel<512> : select_kernel<1024>;
+    const size_t smem = (size_t)keys_cap * sizeof(uint32_t);
+    if (smem > 40 * 1024) {  // (with the kernel's own, past what a launch gets unasked)
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)C * (unsigned)rows);
     cfg.blockDim = dim3(nt);
-    cfg.dynamicSmemBytes = (size_t)keys_cap * sizeof(uint32_t);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
     int n = 0;
@@ -84,9 +81,8 @@ cudaError_t launch_select(int32_t rows, int32_t cap, const float *util, const in
     }
     cfg.attrs = attr;
     cfg.numAttrs = n;
-    cudaError_t e = cudaLaunchKernelEx(
-        &cfg, nt == 256 ? select_kernel<256> : nt == 512 ? select_kernel<512> : select_kernel<1024>, cap, util, len,
-        rows_per_seq, budget, pos, keep, keep_len, df, C, keys_cap);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, cap, util, len, rows_per_seq, budget, pos, keep, keep_len, df, C,
+                                       keys_cap);
     note_launch();
     return e != cudaSuccess ? e : cudaGetLastError();
 }
