@@ -393,8 +393,10 @@ __global__ void __launch_bounds__(kAttendThreads, kF32CtasPerSm) attend_f32_kern
 // b = 8, 16 layers, 32 / 8 heads of 64, 2048 tokens (539 MB, 79.5 us at the copy rate):
 // 222.4 -> 128.5 us against the CUDA-core kernel with its block barriers; 128 dims in
 // 48-token pages 271 -> 208 us when 32 tokens, not 16, came to share the row look-ups and
-// the registers left room for 16 warps an SM.  What is left: the ramp of each CTA (length,
-// table, rows: three dependent loads) and 1.7 waves of CTAs.
+// the registers left room for 16 warps an SM.  The two halves of a block are a rolled loop
+// at 64 dims (unrolled, 128 registers spill 48 bytes: 122.4 us a step against 118.8) and
+// unrolled at 128 (255 registers, no spill: 206.3 us against 207.4).  What is left: the
+// ramp of each CTA (length, table, rows: three dependent loads) and 1.7 waves of CTAs.
 __device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t (&r)[4]) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
@@ -567,7 +569,7 @@ __global__ void __launch_bounds__(kAttendThreads, Bf16Cfg<D>::kCtasPerSm) attend
         const uint32_t rows = rows_next;
         rows_next = lookup(tok0 + 2 * kStride);
         const bool alive_next = alive(tok0 + kStride);
-#pragma unroll
+#pragma unroll (D == 64 ? 1 : 2)
         for (int half = 0; half < 2; ++half) {
             __syncwarp();  // the stage about to be refilled was read in the previous round
             issue(stage == 0 ? NST - 1 : stage - 1, half, rows);
