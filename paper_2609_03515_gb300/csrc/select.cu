@@ -52,7 +52,7 @@ cudaError_t launch_select(int32_t rows, int32_t cap, const float *util, const in
     const int seg = (cap + C - 1) / C;
     const int32_t keys_cap = seg < kSelKeysMax ? seg : kSelKeysMax;
     // threads for about one batch of eight keys each: more warps would issue the same predicated
-    // batches for nothing (one row of 1096 slots: 14.3 us with 1024 threads, 10.2 with 256)
+    // batches for nothing (one row of 1096 slots: 14.3 us with 1024 threads, 8.2 with 256)
     const int nt = seg <= 2048 ? 256 : C > 1 || seg <= 4608 ? 512 : 1024;
     auto kernel = nt == 256 ? select_kernel<256> : nt == 512 ? select_kernel<512> : select_kernel<1024>;
     const size_t smem = (size_t)keys_cap * sizeof(uint32_t);
