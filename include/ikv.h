@@ -246,10 +246,7 @@ ikv_status ikv_attend_path(const ikv_shape *shape, const ikv_cache *cache, int32
  * (more than 1 when the units alone nearly fill that wave but their chunks do not);
  * *group_sums is 1 when every unit is one chunk, so the launch hands the score pass
  * per-KV-head sums of normalised probabilities instead of per-head logits (Eq. 1 needs
- * only those).  (Inside ikv_step, units of two to eight chunks may also run as
- * thread-block clusters that hand over group sums, their tiles cut evenly into the same
- * number of chunks; the query describes a launch without clusters.)  *path as
- * ikv_attend_path.  Host only; launches nothing.  Any output
+ * only those).  *path as ikv_attend_path.  Host only; launches nothing.  Any output
  * pointer may be NULL; fails with IKV_ERR_ARG if n_layers is outside [1, layers] or
  * sms < 0. */
 ikv_status ikv_attend_plan(const ikv_shape *shape, const ikv_cache *cache, int32_t n_layers, int32_t sms,

@@ -210,9 +210,9 @@ void choose_splits(const ikv_shape *s, int n_layers, int32_t max_len, int32_t *s
     // slots: waves x tokens of a split, plus what each CTA costs besides (its ramp, as tokens
     // of its stream: 112 KB of an SM's stream shared by the CTAs on it) and what a merge does.
     // Measured, us a step for 1 / 2 / 3 / 4 / 5 / 7 splits of 2049 tokens.  fp32, d = 128,
-    // G = 4: 128 units 115 / 75 / 64 / 71 / 69 / 62 (7 taken: 1.96 waves), 256 units
-    // 130 / 135 / 113 / 115 / 109 / 110 (7 taken).  bf16, d = 64: 256 units 51 / 43 / 50 / 47 /
-    // 51 / 49 (2 taken), 1024 units 119 / 131 / 128 / 129 / 136 / 149 (1 taken).
+    // G = 4: 128 units 108 / 83 / 85 / 80 / 83 / 77 (7 taken: 2.95 waves), 256 units
+    // 129 / 135 / 135 / 135 / - / 135 (1 taken).  bf16, d = 64: 256 units 58 / 52 / 57 / 53 /
+    // - / 54 (2 taken), 1024 units 130 / 139 / 135 / 138 / 142 / 152 (1 taken).
     const int ctas = s->dtype == IKV_F32 ? kF32CtasPerSm : s->head_dim == 64 ? kBf16D64CtasPerSm : kBf16D128CtasPerSm;
     const int64_t slots = (int64_t)sms * ctas;
     const int64_t cta_tokens = (112 << 10) / (ctas * 2 * s->head_dim * elem_bytes(s));
@@ -244,8 +244,8 @@ static bool use_tc(const ikv_shape *s, const ikv_cache *c, int32_t layers_touche
            (int64_t)max_len + 127 <= (int64_t)kMaxSplits * tc_max_split_tokens() && pool_rows < (1ull << 31);
 }
 
-// Whether a layer call of the split step over n_layers layers at max_len writes normalised group
-// sums (run_attend with a gsum request): the tensor-core kernel with one chunk per unit.
+// Whether an attention launch over n_layers layers at max_len writes normalised group sums
+// (run_attend with a gsum request): the tensor-core kernel with one chunk per unit.
 bool attend_gsum(const ikv_shape *s, const ikv_cache *c, int32_t n_layers, int32_t max_len) {
     if (!use_tc(s, c, s->layers, max_len)) return false;
     int32_t it = 0, nc = 0;
@@ -273,21 +273,11 @@ ikv_status run_attend(const ikv_shape *s, const ikv_cache *c, int32_t layer0, in
     if (tc) {
         int32_t it = 0, nc = 0;
         // a start offset may put the first valid row anywhere in its 128-slot tile
-        const int64_t units = (int64_t)s->batch * n_layers * s->kv_heads;
-        tc_plan(max_len + 127, units, sm_count(), &it, &nc);
-        // one chunk per unit, or a cluster of them: the kernel can hand the score pass normalised
-        // group sums.  No clusters for a caller that merges the partials itself (it normalises
-        // too), nor for a layer call of the split step, whose early CTAs run beside the previous
-        // call's, where a cluster finds no room: 16 sequences, 8 layers of 8 KV heads, G = 8, 100
-        // tiles 1177 us a step against 1259 with clusters.
-        const bool clusters = !unmerged && sc_layers == 0;
-        a.gsum = gsum && logits && use_tc(s, c, s->layers, max_len) &&
-                         (nc == 1 || (clusters && tc_cluster_plan(max_len + 127, units, group, c->page_size, sm_count(),
-                                                                  nc, &it)))
-                     ? 1
-                     : 0;
+        tc_plan(max_len + 127, (int64_t)s->batch * n_layers * s->kv_heads, sm_count(), &it, &nc);
         a.split_tokens = it * 128;
         a.n_splits = nc;
+        // one chunk per unit: the kernel can hand the score pass normalised group sums
+        a.gsum = gsum && logits && nc == 1 && use_tc(s, c, s->layers, max_len) ? 1 : 0;
     } else
         choose_splits(s, n_layers, max_len, &a.split_tokens, &a.n_splits, sm_count());
     a.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)s->head_dim));

@@ -18,11 +18,6 @@
 //   * the softmax runs as two sweeps over the S tiles kept in TMEM: the chunk
 //     maximum per head, then logits write-out, exp2, row sums and the bf16 P
 //     operand (double-buffered in shared memory) that feeds the PV MMA;
-//   * where the score pass wants only sums over a KV head's query group, a third sweep writes
-//     those, normalised, in place of the logits: the CTAs of a unit are then a thread-block
-//     cluster and send each other their chunk's (max, sum) through distributed shared memory
-//     (28 layers of 32 x 4 units of 33 tiles, G = 7: 424 MB of logits become 61 MB of sums, a
-//     step 1338 -> 1248 us), or the unit is one chunk and nothing has to be sent;
 //   * between passes the softmax frees the S tiles and O (s_free, o_free
 //     barriers) and folds the pass's (max, sum, O) into running registers, the
 //     online-softmax rescaling by exp2(m_old - m_new).
@@ -63,18 +58,11 @@ constexpr int kOffRed = kOffP + 2 * kOpBytes;
 constexpr int kOffNew = kOffRed + 4 * kN * 4;   // split step: the new token's K and V rows (2 x 256 B)
 constexpr int kOffBar = kOffNew + 2 * kD * 2;
 // barriers: full[kNst], empty[kNst], s_full, p_full[2], p_empty[2], o_full, s_free, o_free, mma_done,
-// stall (the bounded-wait test's barrier, which nothing arrives at),
-// xchg (a cluster's exchange of (max, sum))
-constexpr int kNumBar = 2 * kNst + 11;
+// stall (the bounded-wait test's barrier, which nothing arrives at)
+constexpr int kNumBar = 2 * kNst + 10;
 constexpr uint64_t kStallNs = 10000ull;       // the bounded-wait test's limit: 10 us
 constexpr int kOffMisc = kOffBar + kNumBar * 8;
-constexpr int kMaxCluster = 8;                // chunks of a unit that can run as a cluster (portable size)
-constexpr int kOffXchg = kOffMisc + 16;       // misc: tmem slot, abort flag, last-split flag
-constexpr int kMinClusterGroup = 7, kMinClusterTiles = 11;
-// a cluster's (max, sum) per chunk and head, the unit's (max, 1 / sum) per head
-constexpr int kXchgBytes = (kMaxCluster + 1) * 8 * 8;
-constexpr int kSmemBytes = kOffXchg + kXchgBytes + 1024;  // + slack for 1024-byte alignment
-static_assert(kOffXchg % 8 == 0 && 2 * (kSmemBytes + 2304 + 1024) <= 228 * 1024, "two CTAs (with the bookkeeping's static memory) an SM");
+constexpr int kSmemBytes = kOffMisc + 16 + 1024;  // misc: tmem slot, abort flag, last-split flag   // + slack for 1024-byte alignment
 
 enum : unsigned { kErrTimeout = 1u };
 
@@ -104,10 +92,9 @@ struct TcArgs {
     BookArgs book;              // on: the first a.batch CTAs append, the new slot is len[b]
     __nv_bfloat16 *k_pool, *v_pool;
     float *vnorm;
-    // every unit is a single chunk, or a cluster's: instead of per-head logits, write per token
-    // the KV head's group sum of normalised probabilities, [batch][sc_layers][kv_heads][lstride]
+    // every unit is a single chunk: instead of per-head logits, write per token the KV
+    // head's group sum of normalised probabilities, [batch][sc_layers][kv_heads][lstride]
     int32_t gsum;
-    int32_t cluster;  // nonzero: the n_splits CTAs of a unit are a thread-block cluster
     int32_t passes;  // consecutive chunks per CTA (>= 1)
     // nonzero: nothing the preceding kernels in the stream still write is read before the
     // programmatic-dependency wait except through this launch's own new-token rows, so the
@@ -174,34 +161,6 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     atomicOr(&g_tc_error, kErrTimeout);
     return false;
 }
-
-// The same for arrivals of other CTAs of the cluster, whose shared-memory stores it acquires.
-__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int *abort) {
-    const uint64_t start = global_ns();
-    for (;;) {
-        uint32_t ok;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\tselp.u32 "
-            "%0, 1, 0, p;\n}\n"
-            : "=r"(ok)
-            : "r"(bar), "r"(parity), "r"(kTryNs)
-            : "memory");
-        if (ok) return true;
-        if (*abort) return false;
-        if (global_ns() - start > kWaitNs) break;
-    }
-    *abort = 1;
-    atomicOr(&g_tc_error, kErrTimeout);
-    return false;
-}
-// address in the shared memory of the cluster's CTA `rank` of this CTA's address `saddr`
-__device__ __forceinline__ uint32_t map_rank(uint32_t saddr, int rank) {
-    uint32_t ra;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(saddr), "r"(rank));
-    return ra;
-}
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 
 // Wait for the MMAs this thread has issued, whatever the abort flag says (at most kWaitNs):
 // TMEM is freed only after every tcgen05 operation writing it has completed.
@@ -291,10 +250,7 @@ __device__ __forceinline__ uint32_t sw128(uint32_t row, uint32_t col) {
 
 // MP: the launch may give a CTA more than one pass (a.passes > 1); without it the pass
 // loop, the s_free / o_free handshakes and the register fold compile away.
-// CL: the CTAs of a unit are a cluster (a.cluster) that exchanges its chunks' (max, sum), so
-// every CTA can write its rows' group sums although no CTA saw the whole unit.  The grid is
-// unit-major then, and each unit's tiles are cut evenly.
-template <int G, bool MP, bool CL>
+template <int G, bool MP>
 __global__ void __launch_bounds__(kThreads, 2)
     attend_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const TcArgs a) {
     constexpr int NC = G <= 4 ? 4 : 8;  // TMEM columns read per S tile
@@ -318,16 +274,10 @@ __global__ void __launch_bounds__(kThreads, 2)
                                     reinterpret_cast<uint32_t *>(sm), kNst * kStage / 4);
             return;
         }
-        if (CL) {  // whole clusters of bookkeeping CTAs: the rest of the last one has nothing to do
-            const int nb = (a.batch + a.n_splits - 1) / a.n_splits * a.n_splits;
-            if (bid < nb) return;
-            bid -= nb;
-        } else {
-            bid -= a.batch;
-        }
+        bid -= a.batch;
     }
-    const int cta = CL ? bid % a.n_splits : bid / n_units;  // CTA index within the unit (CL: rank in the cluster)
-    const int unit_id = CL ? bid / a.n_splits : bid % n_units;
+    const int cta = bid / n_units;  // CTA index within the unit
+    const int unit_id = bid % n_units;
     const int g = unit_id % a.kv_heads;
     const int b = (unit_id / a.kv_heads) % a.batch, li = (unit_id / a.kv_heads) / a.batch;
     const int l = a.layer0 + li;
@@ -340,9 +290,8 @@ __global__ void __launch_bounds__(kThreads, 2)
     const int L = L0 + (grown ? 1 : 0);
     const int ft = S0 / kTile;
     const int nt_unit = L > 0 ? (S0 + L + kTile - 1) / kTile - ft : 0;
-    int item = a.split_tokens / kTile;  // tiles per chunk
+    const int item = a.split_tokens / kTile;  // tiles per chunk
     const int ns_active = (nt_unit + item - 1) / item;  // chunks of the unit
-    if (CL && ns_active > 1) item = (nt_unit + ns_active - 1) / ns_active;  // the same count of even chunks
     const int c0 = cta * a.passes;                      // this CTA's first chunk
     if (c0 >= ns_active) {
         if (early) pdl_wait();
@@ -379,7 +328,6 @@ __global__ void __launch_bounds__(kThreads, 2)
     const uint32_t o_free = bar0 + 8u * (2 * kNst + 7);  // the softmax has read a pass's O
     const uint32_t mma_done = bar0 + 8u * (2 * kNst + 8);  // every MMA of the CTA has completed
     const uint32_t stall_bar = bar0 + 8u * (2 * kNst + 9);  // nothing arrives here (a.stall)
-    const uint32_t xchg = bar0 + 8u * (2 * kNst + 10);      // CL: every chunk's (max, sum) has arrived
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(sm + kOffMisc);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(sm + kOffMisc + 4);
 
@@ -450,7 +398,6 @@ __global__ void __launch_bounds__(kThreads, 2)
             mbar_init(o_free, 128);
             mbar_init(mma_done, 1);
             mbar_init(stall_bar, 1);
-            if (CL) mbar_init(xchg, ns_active * G);
             *abort_flag = 0;
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         }
@@ -515,13 +462,6 @@ __global__ void __launch_bounds__(kThreads, 2)
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
-    if (CL) {  // every CTA of the cluster runs and its exchange barrier is ready
-        cluster_arrive();
-        cluster_wait();
-        // The cluster's other phase says that a thread sends nothing more, so that no CTA leaves
-        // while another may still write to it.  Only the softmax warps send (see below).
-        if (warp >= 4) cluster_arrive();
-    }
     const uint32_t tmem = *tmem_slot;
     const uint32_t tS = tmem, tO = tmem + kOcol;
 
@@ -627,7 +567,6 @@ __global__ void __launch_bounds__(kThreads, 2)
             a.pos ? a.pos + ((int64_t)b * a.rows_per_seq + (a.rows_per_seq == 1 ? 0 : g)) * a.cap : nullptr;
         const int64_t lbase = (((int64_t)b * a.sc_layers + a.sc_layer0 + li) * H + (int64_t)g * G) * a.lstride;
         bool ok = true;
-        uint32_t cl_live = 0u;  // CL: the chunk's live_bits
         int Q = 0;  // P tiles written so far
         // Every bar.sync below runs once per pass in every softmax warp, whatever ok says.
         for (int p = 0; p < np; ++p) {
@@ -646,7 +585,6 @@ __global__ void __launch_bounds__(kThreads, 2)
                 const int tok = t0 + i * kTile + tid;  // physical slot; logical slot tok - S0
                 if (tok >= lo && tok < t1 && (!prow || tok == p_new || __ldg(prow + (tok - S0)) >= 0)) live_bits |= 1u << i;
             }
-            if (CL) cl_live = live_bits;
             if (ok) ok = mbar_wait(s_full, p & 1, abort_flag);
             ok = __all_sync(0xffffffffu, ok);
             fence_after_sync();
@@ -716,32 +654,10 @@ __global__ void __launch_bounds__(kThreads, 2)
             for (int h = 0; h < G; ++h) sum[h] = red[h] + red[kN + h] + red[2 * kN + h] + red[3 * kN + h];
             if (p + 1 < np) softmax_bar();  // red is rewritten by the next pass
 
-            if (CL) {
-                // this chunk's (max, sum) to every CTA of the unit, one thread a CTA and head
-                static_assert(G <= 8 && kMaxCluster * 8 <= 128, "a softmax thread per CTA and head");
-                const int r = tid >> 3, hh = tid & 7;
-                if (ok && hh < G && r < ns_active) {
-                    float mm = 0.f, ss = 0.f;
-#pragma unroll
-                    for (int h = 0; h < G; ++h)
-                        if (h == hh) {
-                            mm = mx[h];
-                            ss = sum[h];
-                        }
-                    asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(
-                                     map_rank(base + kOffXchg + (cta * 8 + hh) * 8, r)),
-                                 "f"(mm), "f"(ss)
-                                 : "memory");
-                    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(map_rank(xchg, r))
-                                 : "memory");
-                }
-                cluster_arrive();  // nothing more is sent
-            }
-
             // sweep 3 (single-chunk units): the chunk's max and sum are the unit's, so each row's
             // normalised probabilities are final; their sum over the KV head's query group is
             // stored per token.  The S tiles are still in TMEM (the PV products go to O).
-            if (!CL && a.gsum && a.logits && ok) {
+            if (a.gsum && a.logits && ok) {
                 if (ns_active == 1) {
                     float inv[G];
 #pragma unroll
@@ -930,50 +846,7 @@ __global__ void __launch_bounds__(kThreads, 2)
                 if (tid == 0) a.arrivals[unit] = 0;
             }
         }
-        if (CL) {
-            // sweep 3 of a cluster: the unit's (max, sum) from its chunks', then this chunk's group
-            // sums (the S tiles are still in TMEM)
-            if (ok) ok = mbar_wait_cluster(xchg, 0, abort_flag);
-            ok = __all_sync(0xffffffffu, ok);
-            float *un = reinterpret_cast<float *>(sm + kOffXchg) + kMaxCluster * 16;
-            if (ok && tid < G) {
-                const float2 *xc = reinterpret_cast<const float2 *>(sm + kOffXchg) + tid;
-                float mm = -INFINITY, ss = 0.f;
-                for (int r = 0; r < ns_active; ++r) mm = fmaxf(mm, xc[r * 8].x);
-                const float ref = mm == -INFINITY ? 0.f : mm;  // every row of the unit dead
-                for (int r = 0; r < ns_active; ++r) ss += xc[r * 8].y * exp2f(xc[r * 8].x - ref);
-                un[tid * 2] = ref;
-                un[tid * 2 + 1] = ss > 0.f ? 1.f / ss : 0.f;
-            }
-            __syncwarp();
-            softmax_bar();
-            if (ok) {
-                const int n = chunk_n(0), t0 = chunk_t0(0);
-                const int lo = max(t0, S0), t1 = min(t0 + n * kTile, S0 + L);
-                float mu[G], inv[G];
-#pragma unroll
-                for (int h = 0; h < G; ++h) {
-                    mu[h] = un[h * 2];
-                    inv[h] = un[h * 2 + 1];
-                }
-                const int64_t gbase = (((int64_t)b * a.sc_layers + a.sc_layer0 + li) * a.kv_heads + g) * a.lstride;
-                for (int i = 0; i < n; ++i) {
-                    float v[NC];
-                    tmem_ld<NC>(tS + lane_off + kN * i, v);
-                    const int tok = t0 + i * kTile + tid;
-                    if (tok >= lo && tok < t1) {
-                        float gs = 0.f;
-                        if ((cl_live >> i) & 1u) {
-#pragma unroll
-                            for (int h = 0; h < G; ++h) gs += exp2f(v[h] * a.scale_log2 - mu[h]) * inv[h];
-                        }
-                        a.logits[gbase + (tok - S0)] = gs;
-                    }
-                }
-            }
-        }
     }
-    if (CL) cluster_wait();
     fence_before_sync();
     __syncthreads();
     if (warp == 0) {
@@ -1007,38 +880,19 @@ bool make_map(CUtensorMap *m, const void *pool, uint64_t rows, int rows_per_box)
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int G, bool MP, bool CL>
+template <int G, bool MP>
 cudaError_t launch_tc_gm(const CUtensorMap &mk, const CUtensorMap &mv, const TcArgs &t, dim3 grid, cudaStream_t st) {
-    auto kernel = attend_tc_kernel<G, MP, CL>;
     static bool attr = false;
     if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+        cudaError_t e = cudaFuncSetAttribute(attend_tc_kernel<G, MP>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
         if (e != cudaSuccess) return e;
         attr = true;
     }
-    if (!CL) return launch_k(kernel, grid, dim3(kThreads), kSmemBytes, st, mk, mv, t);
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = kSmemBytes;
-    cfg.stream = st;
-    cudaLaunchAttribute at[2];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)t.n_splits;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = pdl_enabled() ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, kernel, mk, mv, t);
+    return launch_k(attend_tc_kernel<G, MP>, grid, dim3(kThreads), kSmemBytes, st, mk, mv, t);
 }
 template <int G>
 cudaError_t launch_tc_g(const CUtensorMap &mk, const CUtensorMap &mv, const TcArgs &t, dim3 grid, cudaStream_t st) {
-    if constexpr (G >= kMinClusterGroup)
-        if (t.cluster) return launch_tc_gm<G, false, true>(mk, mv, t, grid, st);
-    return t.passes > 1 ? launch_tc_gm<G, true, false>(mk, mv, t, grid, st)
-                        : launch_tc_gm<G, false, false>(mk, mv, t, grid, st);
+    return t.passes > 1 ? launch_tc_gm<G, true>(mk, mv, t, grid, st) : launch_tc_gm<G, false>(mk, mv, t, grid, st);
 }
 
 }  // namespace
@@ -1101,34 +955,6 @@ int tc_passes(int64_t units, int n_chunks, int sms, bool gsum) {
     return n_chunks;
 }
 
-// Whether the chunks of a unit run as clusters that hand over group sums instead of logits;
-// *item_tiles becomes the even share of the chunk count.  Two sides are weighed, as tiles of a
-// slot's stream (64 KB each).  For: of the G logits that are written and read per token, one
-// float stays, (G - 1) / 64 of the token's 512 bytes of K and V.  Against: the chunks are even
-// and a unit's run together, so no short remainders fill the last wave, and its phases (load
-// K, softmax, load V) fall together on an SM.  Measured, us a step of 28 layers, without / with
-// clusters: G = 7, 32 x 4 units a layer of 33 tiles 1338 / 1248, 8 x 4 of 33 351 / 341, 16 x 4
-// of 97 1893 / 1804, of 22 449 / 443, 4 x 4 of 27 151 / 147; G = 8, 16 x 4 of 39 829 / 763.
-// Chunks of 9 or 10 tiles can lose (8 x 4 units of 19 tiles 197 / 201, 16 x 4 382 / 375), which
-// two chunks can be and three or more (31 tiles at least) are not.  G = 4 gains little (16 x 7
-// units of 33 tiles 1080 / 1058) and can lose (4 x 8 of 18 186 / 191, 8 x 7 of 17 311 / 318);
-// pages of 16 tokens lose (G = 7, 8 x 4 units of 18 tiles 233 / 245): a tile's sixteen copies
-// are slow to issue, and then both CTAs of an SM wait for them at once.  From two waves on:
-// below, the remainders matter most.
-bool tc_cluster_plan(int32_t max_len, int64_t units, int group, int page_size, int sms, int32_t n_chunks,
-                     int32_t *item_tiles) {
-    const int64_t slots = (int64_t)2 * sms, ctas = units * n_chunks;
-    if (group < kMinClusterGroup || page_size < 64 || n_chunks < 2 || n_chunks > kMaxCluster || ctas < 2 * slots ||
-        tc_passes(units, n_chunks, sms, false) > 1)
-        return false;
-    const int64_t tiles = (max_len + kTile - 1) / kTile, item = (tiles + n_chunks - 1) / n_chunks;
-    if (item < kMinClusterTiles) return false;
-    const int64_t idle = (ctas + slots - 1) / slots * slots - ctas;  // of the last wave
-    if (64 * idle * item >= units * tiles * (group - 1)) return false;
-    *item_tiles = (int32_t)item;
-    return true;
-}
-
 std::atomic<int> g_stall_next{0};
 
 cudaError_t launch_attend_tc(const AttendArgs &a, const TcOutputs &o, int group, int sms, cudaStream_t st) {
@@ -1174,13 +1000,11 @@ cudaError_t launch_attend_tc(const AttendArgs &a, const TcOutputs &o, int group,
     t.vnorm = a.vnorm;
     t.book = a.book;
     t.gsum = a.gsum;
-    t.cluster = a.gsum && a.n_splits > 1 ? 1 : 0;
     t.early = a.early;
     t.stall = g_stall_next.exchange(0);
     const int64_t units = (int64_t)a.pv.kv_heads * a.batch * a.n_layers;
     t.passes = tc_passes(units, a.n_splits, sms, a.gsum != 0);
-    const int64_t book = !a.book.on ? 0 : t.cluster ? (a.batch + a.n_splits - 1) / a.n_splits * a.n_splits : a.batch;
-    dim3 grid((unsigned)(((a.n_splits + t.passes - 1) / t.passes) * units + book));
+    dim3 grid((unsigned)(((a.n_splits + t.passes - 1) / t.passes) * units + (a.book.on ? a.batch : 0)));
     cudaError_t e;
     switch (group) {
         case 1: e = launch_tc_g<1>(mk, mv, t, grid, st); break;

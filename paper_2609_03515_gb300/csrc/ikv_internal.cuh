@@ -136,7 +136,7 @@ struct AttendArgs {
     const int32_t *slot;        // unused when book.on: the new token's slot is len[b]
     float *vnorm;
     BookArgs book;
-    // tensor-core kernel, every unit one chunk or a cluster of chunks: logits holds, per token, each KV head's sum
+    // tensor-core kernel, every unit one chunk: logits holds, per token, each KV head's sum
     // of its query group's normalised probabilities ([batch][sc_layers][kv_heads][lstride])
     // instead of per-head logits
     int32_t gsum;
@@ -229,9 +229,6 @@ struct TcOutputs {
 void tc_plan(int32_t max_len, int64_t units, int sms, int32_t *item_tiles, int32_t *n_chunks);
 // consecutive chunks one CTA of the tensor-core kernel takes, for that chunk plan
 int tc_passes(int64_t units, int n_chunks, int sms, bool gsum);
-// group sums of units of several chunks: run as clusters, with *item_tiles tiles a chunk
-bool tc_cluster_plan(int32_t max_len, int64_t units, int group, int page_size, int sms, int32_t n_chunks,
-                     int32_t *item_tiles);
 cudaError_t launch_attend_tc(const AttendArgs &a, const TcOutputs &o, int group, int sms, cudaStream_t st);
 
 // launchers (return cudaError_t of the launch)

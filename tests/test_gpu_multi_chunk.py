@@ -1,5 +1,6 @@
-"""Group sums of units whose chunks run as a cluster: a step's utilities and outputs against
-fp64 PyTorch, at chunk counts 2 to 8, ragged lengths, start offsets and dead slots."""
+"""Units of 2 to 8 chunks in launches of two waves or more: a step's utilities and outputs
+against fp64 PyTorch, with ragged lengths, start offsets and dead slots; and the outputs do
+not depend on whether the step scores."""
 import math
 
 import pytest
@@ -19,7 +20,7 @@ LAYERS = 19  # batch x kv heads x 19 layers x chunks fills whole waves of 2 x 15
     ([15000, 1700], 2, 7, 256, ikv.IKV_GRAN_KVHEAD),              # 8
     ([14000, 13441], 2, 8, 64, ikv.IKV_GRAN_SEQ),                 # 8
 ])
-def test_cluster_group_sums(lens, kvh, G, ps, gran):
+def test_multi_chunk_units(lens, kvh, G, ps, gran):
     d, nb, H = 128, len(lens), kvh * G
     gen = torch.Generator(device="cuda").manual_seed(sum(lens))
     c = DecodeCache(nb, LAYERS, H, kvh, d, max(lens) + 130, dtype=ikv.IKV_BF16, page_size=ps, page_perm_seed=2,
@@ -52,6 +53,18 @@ def test_cluster_group_sums(lens, kvh, G, ps, gran):
         ikv.ikv_step(c.shape(), p, cch, c.ema, 1, q, kn, vn, out, ws, n)
     torch.cuda.synchronize()
     assert ikv.ikv_device_status() == 0
+    # the same token in a step that does not score: the same attention, bit for bit
+    got_ema, got_len, out1 = c.ema.clone(), c.len.clone(), torch.zeros_like(out)
+    c.set_prefill(lens, [10 ** 6] * nb)
+    c.start.copy_(torch.tensor([(29 * b) % 97 for b in range(nb)], dtype=torch.int32))
+    c.pos.copy_(pos0)
+    c.ema.copy_(ema0)
+    ikv.ikv_step(c.shape(), c.params(alpha, refresh_period=2, max_holes=10 ** 6), cch, c.ema, 2, q, kn, vn, out1, ws, n)
+    torch.cuda.synchronize()
+    assert ikv.ikv_device_status() == 0
+    assert torch.equal(out, out1)
+    c.ema.copy_(got_ema)
+    assert torch.equal(c.len, got_len)
     for b, L in enumerate(lens):
         assert int(c.len[b]) == L + 1
         want = torch.cat([ema0.view(nb, R, -1)[b, :, :L].double(), torch.zeros(R, 1, device="cuda").double()], 1)
