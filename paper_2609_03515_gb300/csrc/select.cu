@@ -56,10 +56,11 @@ cudaError_t launch_select(int32_t rows, int32_t cap, const float *util, const in
     const int nt = seg <= 2048 ? 256 : C > 1 || seg <= 4608 ? 512 : 1024;
     auto kernel = nt == 256 ? select_kernel<256> : nt == 512 ? select_kernel<512> : select_kernel<1024>;
     const size_t smem = (size_t)keys_cap * sizeof(uint32_t);
-    if (smem > 40 * 1024) {  // (with the kernel's own, past what a launch gets unasked)
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    // the limit is the process's, so every call writes the same value: with a call's own size, a
+    // small selection on another thread could lower it between this and the launch
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         kSelKeysMax * (int)sizeof(uint32_t));
+    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)C * (unsigned)rows);
     cfg.blockDim = dim3(nt);
@@ -81,8 +82,7 @@ cudaError_t launch_select(int32_t rows, int32_t cap, const float *util, const in
     }
     cfg.attrs = attr;
     cfg.numAttrs = n;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, cap, util, len, rows_per_seq, budget, pos, keep, keep_len, df, C,
-                                       keys_cap);
+    e = cudaLaunchKernelEx(&cfg, kernel, cap, util, len, rows_per_seq, budget, pos, keep, keep_len, df, C, keys_cap);
     note_launch();
     return e != cudaSuccess ? e : cudaGetLastError();
 }

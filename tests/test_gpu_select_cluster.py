@@ -1,5 +1,7 @@
 """Budgeted selection by clusters of CTAs: bit-exact against a stable sort at the sizes where
 the row's parts, the warps' parts and the keys in shared memory begin and end."""
+import threading
+
 import pytest
 import torch
 
@@ -76,3 +78,32 @@ def test_select_cluster_bit_exact(rows, cap, lens, dead):
         assert int(keep_len[r]) == want.numel(), (r, int(ln[r]), int(budget[r]))
         assert torch.equal(keep[r, :want.numel()].long(), want), (r, int(ln[r]), int(budget[r]))
         assert torch.all(keep[r, want.numel():] == -9)
+
+
+def test_select_sizes_on_two_threads():
+    """Selections of different capacities at the same time: the larger is not refused for a
+    shared-memory limit that the smaller one set (400 rows: one CTA a row, of the same kernel)."""
+    errors = []
+
+    def loop(cap):
+        try:
+            rows, s = 400, torch.cuda.Stream()
+            with torch.cuda.stream(s):
+                util = torch.rand(rows, cap, device="cuda")
+                ln = torch.full((rows,), 100, dtype=torch.int32, device="cuda")
+                keep = torch.zeros(rows, cap, dtype=torch.int32, device="cuda")
+                keep_len = torch.zeros(rows, dtype=torch.int32, device="cuda")
+                budget = ln - 7
+                for _ in range(2000):
+                    ikv.ikv_select_budget(rows, cap, util, ln, 1, budget, None, keep, keep_len, s)
+            s.synchronize()
+            assert int(keep_len.min()) == int(keep_len.max()) == 93
+        except Exception as e:
+            errors.append(e)
+
+    threads = [threading.Thread(target=loop, args=(cap,)) for cap in (11000, 48000)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
