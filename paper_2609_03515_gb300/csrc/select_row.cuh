@@ -77,7 +77,32 @@ __device__ __forceinline__ void select_row(int rank, int C, int r, int L, int32_
     int32_t *pr = pos ? pos + (int64_t)r * cap : nullptr;
     int32_t *kp = keep + (int64_t)r * cap;
     // (through L2: in the score pass other CTAs of the same launch wrote the utilities)
-    auto load_key = [&](int i) { return !pr || __ldcg(pr + i) >= 0 ? ord_key(__ldcg(u + i)) : kDeadKey; };
+    // slots i0, i0 + step, ... : their keys from the row, kDeadKey from `end` on (those load the last
+    // slot: with a branch around each load they went out one by one, 2.2 us a batch of eight)
+    auto load_keys = [&](int i0, int step, int end, uint32_t (&key)[U]) {
+        float x[U];
+        int32_t p[U];
+#pragma unroll
+        for (int k = 0; k < U; ++k) x[k] = __ldcg(u + min(i0 + k * step, end - 1));
+        if (pr) {
+#pragma unroll
+            for (int k = 0; k < U; ++k) p[k] = __ldcg(pr + min(i0 + k * step, end - 1));
+        } else {
+#pragma unroll
+            for (int k = 0; k < U; ++k) p[k] = 0;
+        }
+#pragma unroll
+        for (int k = 0; k < U; ++k) key[k] = i0 + k * step < end && p[k] >= 0 ? ord_key(x[k]) : kDeadKey;
+    };
+    // the same, from shared memory when they are there
+    auto get_keys = [&](int i0, int step, int end, uint32_t (&key)[U]) {
+        if (cached) {
+#pragma unroll
+            for (int k = 0; k < U; ++k) key[k] = i0 + k * step < end ? keys[i0 + k * step - lo] : kDeadKey;
+        } else {
+            load_keys(i0, step, end, key);
+        }
+    };
     auto sync_all = [&]() {
         if (C > 1) cluster_sync();
         else __syncthreads();
@@ -89,22 +114,15 @@ __device__ __forceinline__ void select_row(int rank, int C, int r, int L, int32_
     uint32_t cnt = 0u;
     unsigned long long best = ~0ull;
     for (int i0 = lo + tid; i0 < hi; i0 += NT * U) {
-        float x[U];
-        int32_t p[U];
+        uint32_t key[U];
+        load_keys(i0, NT, hi, key);
 #pragma unroll
         for (int k = 0; k < U; ++k) {
             const int i = i0 + k * NT;
-            x[k] = i < hi ? __ldcg(u + i) : 0.f;
-            p[k] = i < hi ? (pr ? __ldcg(pr + i) : 0) : -1;
-        }
-#pragma unroll
-        for (int k = 0; k < U; ++k) {
-            const int i = i0 + k * NT;
-            const uint32_t key = p[k] >= 0 ? ord_key(x[k]) : kDeadKey;
-            if (cached && i < hi) keys[i - lo] = key;
-            if (key == kDeadKey) continue;
+            if (cached && i < hi) keys[i - lo] = key[k];
+            if (key[k] == kDeadKey) continue;
             ++cnt;
-            const unsigned long long v = ((unsigned long long)key << 32) | (uint32_t)(~(uint32_t)i);
+            const unsigned long long v = ((unsigned long long)key[k] << 32) | (uint32_t)(~(uint32_t)i);
             best = v < best ? v : best;
         }
     }
@@ -185,17 +203,12 @@ __device__ __forceinline__ void select_row(int rank, int C, int r, int L, int32_
             for (int pass = 0; pass < 4; ++pass) {
                 const int shift = 24 - 8 * pass;
                 uint32_t *h = hist[pass & 1];
-                for (int i0 = lo; i0 < hi; i0 += NT * U) {
-                    uint32_t d[U];
-#pragma unroll
-                    for (int q = 0; q < U; ++q) {
-                        const int i = i0 + q * NT + tid;
-                        const uint32_t key = i < hi ? (cached ? keys[i - lo] : load_key(i)) : 0u;
-                        d[q] = i < hi && (key & mask) == prefix ? (key >> shift) & 0xFFu : 0xFFFFu;
-                    }
+                for (int i0 = lo + tid; i0 < hi; i0 += NT * U) {
+                    uint32_t key[U];
+                    get_keys(i0, NT, hi, key);
 #pragma unroll
                     for (int q = 0; q < U; ++q)
-                        if (d[q] != 0xFFFFu) atomicAdd(&h[d[q]], 1u);
+                        if (i0 + q * NT < hi && (key[q] & mask) == prefix) atomicAdd(&h[(key[q] >> shift) & 0xFFu], 1u);
                 }
                 sync_all();
                 // (every CTA is past its reads of the other buffer)
@@ -256,11 +269,7 @@ __device__ __forceinline__ void select_row(int rank, int C, int r, int L, int32_
         uint32_t gt = 0u, eq = 0u;
         for (int i0 = wlo + lane; i0 < whi; i0 += 32 * U) {
             uint32_t key[U];
-#pragma unroll
-            for (int q = 0; q < U; ++q) {
-                const int i = i0 + 32 * q;
-                key[q] = i < whi ? (cached ? keys[i - lo] : load_key(i)) : kDeadKey;
-            }
+            get_keys(i0, 32, whi, key);
 #pragma unroll
             for (int q = 0; q < U; ++q) {
                 gt += key[q] > theta;
@@ -320,11 +329,7 @@ __device__ __forceinline__ void select_row(int rank, int C, int r, int L, int32_
         const uint32_t below = (1u << lane) - 1u;
         for (int i0 = wlo; i0 < whi; i0 += 32 * U) {
             uint32_t key[U];
-#pragma unroll
-            for (int q = 0; q < U; ++q) {
-                const int i = i0 + 32 * q + lane;
-                key[q] = i < whi ? (cached ? keys[i - lo] : load_key(i)) : kDeadKey;
-            }
+            get_keys(i0 + lane, 32, whi, key);
 #pragma unroll
             for (int q = 0; q < U; ++q) {
                 if (i0 + 32 * q >= whi) break;
