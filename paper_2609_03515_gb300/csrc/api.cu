@@ -909,6 +909,25 @@ ikv_status ikv_step_workspace_size(const ikv_shape *shape, const ikv_cache *cach
     return IKV_OK;
 }
 
+// Whether a step whose attention leaves the utilities as they are selects in its bookkeeping CTAs,
+// beside the attention, instead of in a kernel after it.  A row's CTA sweeps the row alone, so the
+// attention must last as long: short rows, or many bytes of K and V per slot.  And where nothing
+// can be deferred the keep list must still be in L2 when the compaction reads it, which a large
+// stream of K and V sees to that it is not.  Measured, us a step with the selection beside / after
+// (bf16, 8 KV heads of 128 unless stated).  Deferred: 3277 slots, 32 layers 68.0 / 70.7, 2 layers
+// 11.8 / 14.9; 8192, one layer of 2 heads 14.3 / 16.2; 16384, 32 layers 306 / 310, 2 layers (8 KB a
+// slot) 34.2 / 36.8, 64 dims and 2 layers (4 KB) 33.3 / 27.0, 64 dims and 16 layers (32 KB) 101 / 104,
+// fp32 and 2 layers (16 KB) 64.9 / 63.3; 32768, 2 layers 68.3 / 56.0; 65536, 32 layers 1190 / 1202, 2
+// layers 135 / 104.  Not deferred: 3277 slots, 32 layers (430 MB) 187 / 167, 2 layers (27 MB)
+// 42.0 / 45.4; 16 sequences of 800, 32 layers 780 / 706.
+static bool select_beside(const ikv_shape *shape, const ikv_params *p, int32_t max_len) {
+    constexpr int64_t kShortRow = 8192, kSlotBytes = 32 << 10, kInL2Bytes = 32 << 20;
+    const int64_t slot_bytes =
+        (int64_t)shape->batch * shape->layers * shape->kv_heads * 2 * shape->head_dim * elem_bytes(shape);
+    if (p->max_holes == 0 && slot_bytes * max_len > kInL2Bytes) return false;
+    return max_len <= kShortRow || slot_bytes >= kSlotBytes;
+}
+
 ikv_status ikv_step(const ikv_shape *shape, const ikv_params *p, ikv_cache *cache, float *ema, int32_t t,
                     const void *q, const void *k_new, const void *v_new, void *out, void *ws, size_t ws_bytes,
                     cudaStream_t stream) {
@@ -943,7 +962,7 @@ ikv_status ikv_step(const ikv_shape *shape, const ikv_params *p, ikv_cache *cach
     // kernel that counts leaves its counters zero again
     if ((e = zero_control_words(p, ws, w, stream))) return e;
     if (tm && (e = record(tm->begin, stream))) return e;
-    // The attention launch appends the new token: a CTA per sequence does the bookkeeping (its
+    // The attention launch appends the new token: a CTA per utility row does the bookkeeping (its
     // position and utility; the length with it goes to len1, for the step's later kernels), and
     // the CTA whose chunk holds the new slot stores that layer and KV head's rows and uses them
     // in place of the slot's old contents.  The compaction writes the step's final lengths.
@@ -955,14 +974,14 @@ ikv_status ikv_step(const ikv_shape *shape, const ikv_params *p, ikv_cache *cach
     int32_t *len1 = at<int32_t>(ws, w.len1);
     NewRows rows{k_new, v_new, nullptr, cache->vnorm, {}};
     rows.book.on = 1;
+    rows.book.done = at<int32_t>(ws, w.done);
     rows.book.len1 = len1;
     rows.book.pos = cache->pos;
     rows.book.next_pos = cache->next_pos;
     rows.book.ema = ema;
     rows.book.init_mean = cx.init_mean;
     rows.book.dead_slots = cache->dead_slots;
-    // utilities untouched by this step's attention: the bookkeeping CTAs select, too
-    const bool ahead = !cx.scoring;
+    const bool ahead = !cx.scoring && select_beside(shape, p, cx.L1);
     if (ahead) {
         rows.book.select = 1;
         rows.book.budget = p->budget;

@@ -173,12 +173,13 @@ __global__ void __launch_bounds__(kAttendThreads, kF32CtasPerSm) attend_f32_kern
     // 1-D grid: the bookkeeping CTAs, if any, then splits, kv heads, sequences, layers
     int bid = blockIdx.x;
     if (a.book.on) {
-        if (bid < a.batch) {
-            book_sequence<kAttendThreads>(a.book, a.len, a.pv.start, a.cap, a.rows_per_seq, bid, &g_attend_error,
-                                          reinterpret_cast<uint32_t *>(smem), C::kRing / 4);
+        const int books = a.batch * a.rows_per_seq;
+        if (bid < books) {
+            book_row<kAttendThreads>(a.book, a.len, a.pv.start, a.cap, a.rows_per_seq, bid, &g_attend_error,
+                                     reinterpret_cast<uint32_t *>(smem), C::kRing / 4);
             return;
         }
-        bid -= a.batch;
+        bid -= books;
     }
     const int s = bid % a.n_splits;
     bid /= a.n_splits;
@@ -452,12 +453,13 @@ __global__ void __launch_bounds__(kAttendThreads, Bf16Cfg<D>::kCtasPerSm) attend
     // 1-D grid: the bookkeeping CTAs, if any, then splits, kv heads, sequences, layers
     int bid = blockIdx.x;
     if (a.book.on) {
-        if (bid < a.batch) {
-            book_sequence<kAttendThreads>(a.book, a.len, a.pv.start, a.cap, a.rows_per_seq, bid, &g_attend_error,
-                                          reinterpret_cast<uint32_t *>(smem), C::kRing / 4);
+        const int books = a.batch * a.rows_per_seq;
+        if (bid < books) {
+            book_row<kAttendThreads>(a.book, a.len, a.pv.start, a.cap, a.rows_per_seq, bid, &g_attend_error,
+                                     reinterpret_cast<uint32_t *>(smem), C::kRing / 4);
             return;
         }
-        bid -= a.batch;
+        bid -= books;
     }
     const int s = bid % a.n_splits;
     bid /= a.n_splits;
@@ -660,7 +662,7 @@ __global__ void __launch_bounds__(kAttendThreads, Bf16Cfg<D>::kCtasPerSm) attend
 }
 
 dim3 attend_grid(const AttendArgs &a) {
-    return dim3((unsigned)a.n_splits * a.pv.kv_heads * a.batch * a.n_layers + (a.book.on ? a.batch : 0));
+    return dim3((unsigned)a.n_splits * a.pv.kv_heads * a.batch * a.n_layers + (a.book.on ? a.batch * a.rows_per_seq : 0));
 }
 
 template <int D, int G>

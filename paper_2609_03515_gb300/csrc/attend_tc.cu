@@ -89,7 +89,7 @@ struct TcArgs {
     // the slot's old contents; vnorm (or null) gets their V norms
     const __nv_bfloat16 *k_new, *v_new;
     const int32_t *slot;
-    BookArgs book;              // on: the first a.batch CTAs append, the new slot is len[b]
+    BookArgs book;              // on: the first CTAs, one per utility row, append; the new slot is len[b]
     __nv_bfloat16 *k_pool, *v_pool;
     float *vnorm;
     // every unit is a single chunk: instead of per-head logits, write per token the KV
@@ -269,12 +269,13 @@ __global__ void __launch_bounds__(kThreads, 2)
     const int n_units = a.batch * a.n_layers * a.kv_heads;
     int bid = blockIdx.x;
     if (a.book.on) {
-        if (bid < a.batch) {
-            book_sequence<kThreads>(a.book, a.len, a.start, a.cap, a.rows_per_seq, bid, &g_tc_error,
-                                    reinterpret_cast<uint32_t *>(sm), kNst * kStage / 4);
+        const int books = a.batch * a.rows_per_seq;
+        if (bid < books) {
+            book_row<kThreads>(a.book, a.len, a.start, a.cap, a.rows_per_seq, bid, &g_tc_error,
+                               reinterpret_cast<uint32_t *>(sm), kNst * kStage / 4);
             return;
         }
-        bid -= a.batch;
+        bid -= books;
     }
     const int cta = bid / n_units;  // CTA index within the unit
     const int unit_id = bid % n_units;
@@ -1004,7 +1005,7 @@ cudaError_t launch_attend_tc(const AttendArgs &a, const TcOutputs &o, int group,
     t.stall = g_stall_next.exchange(0);
     const int64_t units = (int64_t)a.pv.kv_heads * a.batch * a.n_layers;
     t.passes = tc_passes(units, a.n_splits, sms, a.gsum != 0);
-    dim3 grid((unsigned)(((a.n_splits + t.passes - 1) / t.passes) * units + (a.book.on ? a.batch : 0)));
+    dim3 grid((unsigned)(((a.n_splits + t.passes - 1) / t.passes) * units + (a.book.on ? a.batch * a.rows_per_seq : 0)));
     cudaError_t e;
     switch (group) {
         case 1: e = launch_tc_g<1>(mk, mv, t, grid, st); break;

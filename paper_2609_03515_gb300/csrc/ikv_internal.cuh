@@ -96,9 +96,10 @@ struct DeferArgs {
     int32_t later;              // nonzero: only name the victim, in keep[r][0]; the compaction marks it
 };
 
-// A step's append, by extra CTAs of its attention launch (book.cuh)
+// A step's append, by extra CTAs of its attention launch, one per utility row (book.cuh)
 struct BookArgs {
     int32_t on;                 // nonzero: they run, and len is the length before the append
+    int32_t *done;              // [batch] arrival counters of a sequence's rows, zero on entry, left zero
     int32_t *len1;              // [batch] the length after it
     int32_t *pos, *next_pos;
     float *ema;

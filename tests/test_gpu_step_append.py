@@ -87,6 +87,59 @@ def test_step_appends(dtype, d, ps, gran):
                 assert abs(float(c.ema[row, L]) - float(mean)) < 1e-5
 
 
+# launches: attention and compaction, and a selection of its own where the bookkeeping CTAs would
+# outlast the attention (long rows over few bytes of K and V a slot) or nothing can be deferred
+# and the keep list would have left L2
+@pytest.mark.parametrize("L,layers,kvh,gran,holes,launches", [
+    (300, 3, 2, ikv.IKV_GRAN_KVHEAD, 4, 2), (300, 3, 2, ikv.IKV_GRAN_SEQ, 0, 2),
+    (8191, 1, 2, ikv.IKV_GRAN_KVHEAD, 4, 2), (8192, 1, 2, ikv.IKV_GRAN_KVHEAD, 4, 3),
+    (8192, 1, 2, ikv.IKV_GRAN_SEQ, 0, 3), (9000, 16, 4, ikv.IKV_GRAN_KVHEAD, 4, 2),
+    (2100, 16, 4, ikv.IKV_GRAN_KVHEAD, 0, 3),
+])
+def test_off_refresh_selection(L, layers, kvh, gran, holes, launches):
+    d, G, nb = 128, 2, 2
+    gen = torch.Generator(device="cuda").manual_seed(L + layers)
+    c = DecodeCache(nb, layers, G * kvh, kvh, d, L + 200, dtype=ikv.IKV_BF16, page_size=64, page_perm_seed=4,
+                    granularity=gran)
+    c.k.copy_(torch.randn(c.k.shape, generator=gen, device="cuda"))
+    c.v.copy_(torch.randn(c.v.shape, generator=gen, device="cuda"))
+    c.set_prefill([L] * nb, [L] * nb)
+    c.ema.copy_(torch.rand(c.ema.shape, generator=gen, device="cuda"))
+    c.ema[:, 17] = c.ema[:, 5]
+    c.ema[0, 5] = c.ema[0, 17] = 0.0  # a tie: the higher slot goes
+    ema0, pos0 = c.ema.clone(), c.pos.clone()
+    k0 = c.gather(c.k, 0, layers - 1, kvh - 1, L)
+    q = torch.randn(layers, nb, G * kvh, d, generator=gen, device="cuda").bfloat16()
+    kn = torch.randn(layers, nb, kvh, d, generator=gen, device="cuda").bfloat16()
+    out = torch.zeros_like(q)
+    cch = c.cache(L)
+    ws = c.step_workspace()
+    before = ikv.ikv_launch_count()
+    p = c.params(0.9, refresh_period=4, max_holes=holes)
+    ikv.ikv_step(c.shape(), p, cch, c.ema, 2, q, kn, kn, out, ws, ws.numel())
+    torch.cuda.synchronize()
+    assert ikv.ikv_launch_count() - before == launches
+    assert ikv.ikv_device_status() == 0
+    assert c.next_pos.tolist() == [L + 1] * nb and c.len.tolist() == [L + (holes > 0)] * nb
+    for r in range(c.rows):
+        mean = float(ema0[r, :L].double().mean())
+        if holes:
+            assert abs(float(c.ema[r, L]) - mean) < 1e-5 and int(c.pos[r, L]) == L
+        util = torch.cat([ema0[r, :L], torch.tensor([mean], device="cuda")])
+        victim = int((util == util.min()).nonzero().max())
+        want = torch.cat([pos0[r, :L], torch.tensor([L], dtype=torch.int32, device="cuda")])
+        if holes:
+            want[victim] = -1
+        else:
+            want = want[want != victim]
+        assert torch.equal(c.pos[r, :want.numel()], want), r
+        if r == (kvh if gran == ikv.IKV_GRAN_KVHEAD else 1) - 1:  # the last KV head of sequence 0
+            rows = torch.cat([k0, kn[layers - 1, 0, kvh - 1][None]])
+            keep = torch.arange(L + 1, device="cuda")
+            keep = keep if holes else keep[keep != victim]
+            assert torch.equal(c.gather(c.k, 0, layers - 1, kvh - 1, keep.numel()), rows[keep])
+
+
 @pytest.mark.parametrize("dtype,d", [(ikv.IKV_BF16, 128), (ikv.IKV_F32, 64)])
 def test_step_lengths_without_eviction(dtype, d):
     """Lengths and positions over steps that evict nothing, then defer, then compact."""
