@@ -338,6 +338,12 @@ ikv_status ikv_select_budget(int32_t rows, int32_t cap, const float *util, const
                              int32_t rows_per_seq, const int32_t *budget, const int32_t *pos, int32_t *keep,
                              int32_t *keep_len, cudaStream_t stream);
 
+/* How a selection of `rows` rows of up to max_len slots (ikv_select_budget: cap) is launched on a
+ * GPU with sms SMs (0: the current device's): *ctas CTAs a row, a thread-block cluster beyond one,
+ * of *threads threads.  A row shorter than max_len may leave some of its CTAs idle.  Host only;
+ * launches nothing.  Either output pointer may be NULL. */
+ikv_status ikv_select_plan(int32_t rows, int32_t max_len, int32_t sms, int32_t *ctas, int32_t *threads);
+
 /* ---------------------------------------------------------------------------
  * ikv_compact_kv -- in-place gather compaction after eviction ("cache
  * remapping" of the Appendix "Hook-level profiling" paragraph).

@@ -569,9 +569,18 @@ ikv_status ikv_select_budget(int32_t rows, int32_t cap, const float *util, const
     if (rows > 0 && (!util || !len || !budget || !keep || !keep_len))
         return fail(IKV_ERR_ARG, "util/len/budget/keep/keep_len is NULL");
     // max_holes 0: the kernel never writes pos here
-    IKV_TRY_CUDA(launch_select(rows, cap, util, len, rows_per_seq_, budget, const_cast<int32_t *>(pos), keep,
+    IKV_TRY_CUDA(launch_select(rows, cap, cap, util, len, rows_per_seq_, budget, const_cast<int32_t *>(pos), keep,
                                keep_len, DeferArgs{0, cap, nullptr, 0}, sm_count(), stream),
                  "select launch");
+    return IKV_OK;
+}
+
+ikv_status ikv_select_plan(int32_t rows, int32_t max_len, int32_t sms, int32_t *ctas, int32_t *threads) {
+    g_err[0] = 0;
+    if (rows < 0 || max_len < 0 || sms < 0) return fail(IKV_ERR_SHAPE, "rows/max_len/sms out of range");
+    const SelectPlan p = select_plan(rows, max_len, sms > 0 ? sms : sm_count());
+    if (ctas) *ctas = p.ctas;
+    if (threads) *threads = p.threads;
     return IKV_OK;
 }
 
@@ -777,12 +786,12 @@ static ikv_status zero_control_words(const ikv_params *p, void *ws, const StepWs
 
 // Step 5: selection, then deferred or immediate compaction.
 static ikv_status evict_impl(const ikv_shape *shape, const ikv_params *p, ikv_cache *cache, float *ema, void *ws,
-                             const StepWs &w, cudaStream_t stream, const ikv_timing *tm, bool selected = false,
+                             const StepWs &w, int32_t max_len, cudaStream_t stream, const ikv_timing *tm, bool selected = false,
                              int32_t *len_out = nullptr, bool mark = false) {
     const int32_t cap = cap_of(cache);
     const int32_t R = shape->batch * rows_per_seq(shape);
     if (!selected)
-        IKV_TRY_CUDA(launch_select(R, cap, ema, cache->len, rows_per_seq(shape), p->budget,
+        IKV_TRY_CUDA(launch_select(R, cap, max_len, ema, cache->len, rows_per_seq(shape), p->budget,
                                    cache->dead_slots ? cache->pos : nullptr, at<int32_t>(ws, w.keep),
                                    at<int32_t>(ws, w.keep_len), DeferArgs{p->max_holes, cap, cache->start, 0}, sm_count(), stream),
                      "select launch");
@@ -834,7 +843,7 @@ static ikv_status trace_before(const ikv_shape *shape, const ikv_params *p, cons
                                const StepCtx &cx, cudaStream_t stream) {
     if (!p->trace || !cx.scoring) return IKV_OK;
     const int32_t R = shape->batch * rows_per_seq(shape);
-    IKV_TRY_CUDA(launch_select(R, cx.cap, at<float>(ws, cx.w.raw), cache->len, rows_per_seq(shape), p->budget,
+    IKV_TRY_CUDA(launch_select(R, cx.cap, cx.L1, at<float>(ws, cx.w.raw), cache->len, rows_per_seq(shape), p->budget,
                                cache->dead_slots ? cache->pos : nullptr, at<int32_t>(ws, cx.w.keep_raw),
                                at<int32_t>(ws, cx.w.n_raw), DeferArgs{0, cx.cap, nullptr, 0}, sm_count(), stream),
                  "trace select launch");
@@ -890,7 +899,7 @@ static ikv_status layer_evict(const ikv_shape *shape, const ikv_params *p, ikv_c
     IKV_TRY_CUDA(launch_layer_fold(layer_args(shape, p, cache, ema, ws, cx), cx.L1, cache->pos_cap, stream),
                  "layer fold launch");
     const int32_t K = shape->layers;
-    IKV_TRY_CUDA(launch_select(shape->batch * K, cx.cap, at<float>(ws, cx.w.util), cache->len, K, p->budget, nullptr,
+    IKV_TRY_CUDA(launch_select(shape->batch * K, cx.cap, cx.L1, at<float>(ws, cx.w.util), cache->len, K, p->budget, nullptr,
                                at<int32_t>(ws, cx.w.keep), at<int32_t>(ws, cx.w.keep_len), DeferArgs{0, cx.cap, nullptr, 0},
                                sm_count(), stream),
                  "select launch");
@@ -1006,7 +1015,7 @@ ikv_status ikv_step(const ikv_shape *shape, const ikv_params *p, ikv_cache *cach
         return e;
     if (tm && (e = record(tm->score_end, stream))) return e;
     if ((e = trace_before(shape, p, &appended, ws, cx, stream))) return e;
-    if ((e = evict_impl(shape, p, &appended, ema, ws, w, stream, tm, selected, cache->len, ahead))) return e;
+    if ((e = evict_impl(shape, p, &appended, ema, ws, w, cx.L1, stream, tm, selected, cache->len, ahead))) return e;
     if (tm && (e = record(tm->end, stream))) return e;
     return trace_after(shape, p, cache, ws, cx, stream);
 }
@@ -1072,7 +1081,7 @@ ikv_status ikv_step_end(const ikv_shape *shape, const ikv_params *p, ikv_cache *
                                      p->trace ? nullptr : &fs, &selected, gsum)))
         return e;
     if ((e = trace_before(shape, p, &cx.cv, ws, cx, stream))) return e;
-    if ((e = evict_impl(shape, p, &cx.cv, ema, ws, cx.w, stream, nullptr, selected))) return e;
+    if ((e = evict_impl(shape, p, &cx.cv, ema, ws, cx.w, cx.L1, stream, nullptr, selected))) return e;
     return trace_after(shape, p, &cx.cv, ws, cx, stream);
 }
 

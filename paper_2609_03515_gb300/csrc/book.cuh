@@ -80,7 +80,7 @@ __device__ __noinline__ void book_row(const BookArgs &k, const int32_t *len, con
     }
     if (!k.select) return;
     __syncthreads();  // the new token's utility and position
-    select_row<NT>(0, 1, r, L + (room ? 1 : 0), cap, k.ema, rows_per_seq, k.budget, k.dead_slots ? k.pos : nullptr,
+    select_row<NT, false>(0, 1, r, L + (room ? 1 : 0), cap, k.ema, rows_per_seq, k.budget, k.dead_slots ? k.pos : nullptr,
                    k.keep, k.keep_len, k.df, keys, keys_cap);
 }
 

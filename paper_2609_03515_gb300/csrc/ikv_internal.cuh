@@ -247,9 +247,16 @@ cudaError_t launch_value_norms(const void *v, const PagedView &pv, const int32_t
                                int32_t cap, int dtype, float *vnorm, cudaStream_t st);
 cudaError_t launch_ema_update(int32_t rows, int32_t cap, float *ema, const float *score, const int32_t *len,
                               int32_t rows_per_seq, float alpha, int32_t max_len, cudaStream_t st);
-cudaError_t launch_select(int32_t rows, int32_t cap, const float *util, const int32_t *len, int32_t rows_per_seq,
-                          const int32_t *budget, int32_t *pos, int32_t *keep, int32_t *keep_len, const DeferArgs &df,
-                          int sms, cudaStream_t st);
+// How a selection of `rows` rows of up to max_len slots is launched: CTAs a row (a cluster beyond
+// one), threads a CTA, keys a CTA keeps in shared memory
+struct SelectPlan {
+    int32_t ctas, threads, keys;
+};
+SelectPlan select_plan(int64_t rows, int32_t max_len, int sms);
+// max_len bounds the rows' lengths
+cudaError_t launch_select(int32_t rows, int32_t cap, int32_t max_len, const float *util, const int32_t *len,
+                          int32_t rows_per_seq, const int32_t *budget, int32_t *pos, int32_t *keep, int32_t *keep_len,
+                          const DeferArgs &df, int sms, cudaStream_t st);
 
 struct CompactArgs {
     void *k, *v;

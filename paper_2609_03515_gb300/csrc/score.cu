@@ -313,7 +313,7 @@ __global__ void __launch_bounds__(kScoreThreads, 4) score_kernel(const ScoreArgs
                 if (i != ev) kp[i < ev ? i : i - 1] = i;
         if (threadIdx.x == 0) a.keep_len[r] = kept;
     } else {
-        select_row<kScoreThreads>(0, 1, r, L, a.cap, a.ema, a.rows_per_seq, a.budget, a.sel_pos, a.keep, a.keep_len,
+        select_row<kScoreThreads, false>(0, 1, r, L, a.cap, a.ema, a.rows_per_seq, a.budget, a.sel_pos, a.keep, a.keep_len,
                                   a.df, reinterpret_cast<uint32_t *>(wsm), a.sel_keys);
     }
 }

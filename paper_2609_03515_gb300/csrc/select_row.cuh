@@ -45,13 +45,16 @@ __device__ __forceinline__ unsigned long long ld_cluster(const unsigned long lon
 
 constexpr int kSelMaxCtas = 8;  // CTAs that share a row (portable cluster size)
 
-// The selection of utility row r by C CTAs of NT threads (C > 1: the cluster they form; this
-// one is its `rank`-th), entered by all of their threads.  CTA `rank` owns a contiguous C-th of
-// the row's slots and keeps their keys in keys[0, keys_cap) (shared memory) when they fit;
-// otherwise every sweep reads the row again, a few loads in flight a thread.
-// L: the row's slots in use.
-template <int NT>
-__device__ __forceinline__ void select_row(int rank, int C, int r, int L, int32_t cap, const float *util, int32_t rps,
+constexpr int kSelSlots = 3072;  // slots a CTA should have to be worth a cluster's barriers
+
+// The selection of utility row r by a CTA of NT threads (CL false), or by up to `ctas` CTAs of a
+// cluster, of which this one is the `rank`-th (CL), entered by all of their threads.  CTA `rank`
+// owns a contiguous share of the row's slots and keeps their keys in keys[0, keys_cap) (shared
+// memory) when they fit; otherwise every sweep reads the row again, a few loads in flight a
+// thread.  L: the row's slots in use.  A row too short for the whole cluster is shared by fewer of
+// its CTAs, down to one, and the others leave (a cluster barrier waits for no thread that has).
+template <int NT, bool CL>
+__device__ __forceinline__ void select_row(int rank, int ctas, int r, int L, int32_t cap, const float *util, int32_t rps,
                                            const int32_t *__restrict__ budget, int32_t *pos, int32_t *keep,
                                            int32_t *keep_len, DeferArgs df, uint32_t *keys, int keys_cap) {
     static_assert(NT % 32 == 0 && NT <= 1024, "whole warps");
@@ -70,6 +73,8 @@ __device__ __forceinline__ void select_row(int rank, int C, int r, int L, int32_
     const int b = r / rps;
     const int B = max(budget[b], 0);
     const int S = df.start ? df.start[b] : 0;
+    const int C = CL ? max(1, min(ctas, L / kSelSlots)) : 1;
+    if (CL && rank >= C) return;
     const int seg = (L + C - 1) / C;
     const int lo = min(rank * seg, L), hi = min(lo + seg, L);
     const bool cached = hi - lo <= keys_cap;
@@ -104,10 +109,11 @@ __device__ __forceinline__ void select_row(int rank, int C, int r, int L, int32_
         }
     };
     auto sync_all = [&]() {
-        if (C > 1) cluster_sync();
+        if (CL && C > 1) cluster_sync();
         else __syncthreads();
     };
-    auto peer = [&](const auto *p, int c) { return C > 1 ? ld_cluster(p, c) : *p; };
+    auto peer = [&](const auto *p, int c) { return CL && C > 1 ? ld_cluster(p, c) : *p; };
+    constexpr int kPeers = CL ? kSelMaxCtas : 1;
 
     // one sweep: the live count and the lowest (key, highest slot) among the live slots,
     // which is the victim whenever exactly one slot must go
@@ -157,15 +163,15 @@ __device__ __forceinline__ void select_row(int rank, int C, int r, int L, int32_
     int n_live = 0;
     best = ~0ull;
     {
-        uint32_t live[kSelMaxCtas];
-        unsigned long long low[kSelMaxCtas];
+        uint32_t live[kPeers];
+        unsigned long long low[kPeers];
 #pragma unroll
-        for (int c = 0; c < kSelMaxCtas; ++c) {
+        for (int c = 0; c < kPeers; ++c) {
             live[c] = c < C ? peer(&s_live, c) : 0u;
             low[c] = c < C ? peer(&s_min, c) : ~0ull;
         }
 #pragma unroll
-        for (int c = 0; c < kSelMaxCtas; ++c) {
+        for (int c = 0; c < kPeers; ++c) {
             n_live += (int)live[c];
             best = low[c] < best ? low[c] : best;
         }
@@ -180,7 +186,7 @@ __device__ __forceinline__ void select_row(int rank, int C, int r, int L, int32_
             else pr[ev] = -1;
             keep_len[r] = -1 - B;
         }
-        if (C > 1) cluster_sync();  // a CTA may not leave while another reads its shared memory
+        if (CL && C > 1) cluster_sync();  // a CTA may not leave while another reads its shared memory
         return;
     }
     if (rank == 0 && tid == 0) keep_len[r] = kept;
@@ -221,11 +227,11 @@ __device__ __forceinline__ void select_row(int rank, int C, int r, int L, int32_
                         v[q] = 0u;
                         if (d < 0) continue;
                         hist[(pass & 1) ^ 1][d] = 0u;
-                        uint32_t w[kSelMaxCtas];
+                        uint32_t w[kPeers];
 #pragma unroll
-                        for (int c = 0; c < kSelMaxCtas; ++c) w[c] = c < C ? peer(&h[d], c) : 0u;
+                        for (int c = 0; c < kPeers; ++c) w[c] = c < C ? peer(&h[d], c) : 0u;
 #pragma unroll
-                        for (int c = 0; c < kSelMaxCtas; ++c) v[q] += w[c];
+                        for (int c = 0; c < kPeers; ++c) v[q] += w[c];
                         x += v[q];
                     }
 #pragma unroll
@@ -310,14 +316,14 @@ __device__ __forceinline__ void select_row(int rank, int C, int r, int L, int32_
         sync_all();
         uint32_t gt_all = 0u, gt_run = warp_a[warp], eq_run = warp_b[warp];
         {
-            uint32_t g[kSelMaxCtas], e[kSelMaxCtas];
+            uint32_t g[kPeers], e[kPeers];
 #pragma unroll
-            for (int c = 0; c < kSelMaxCtas; ++c) {
+            for (int c = 0; c < kPeers; ++c) {
                 g[c] = c < C ? peer(&s_gt, c) : 0u;
                 e[c] = c < C ? peer(&s_eq, c) : 0u;
             }
 #pragma unroll
-            for (int c = 0; c < kSelMaxCtas; ++c) {
+            for (int c = 0; c < kPeers; ++c) {
                 gt_all += g[c];
                 if (c < rank) {
                     gt_run += g[c];
@@ -343,7 +349,7 @@ __device__ __forceinline__ void select_row(int rank, int C, int r, int L, int32_
             }
         }
     }
-    if (C > 1) cluster_sync();  // a CTA may not leave while another reads its shared memory
+    if (CL && C > 1) cluster_sync();  // a CTA may not leave while another reads its shared memory
 }
 
 }  // namespace

@@ -82,6 +82,7 @@ def _load():
         "ikv_ema_update": ([I32, I32, P, P, P, I32, F32, P], I32),
         "ikv_value_norms": ([SP, CP, P], I32),
         "ikv_select_budget": ([I32, I32, P, P, I32, P, P, P, P, P], I32),
+        "ikv_select_plan": ([I32, I32, I32, ctypes.POINTER(I32), ctypes.POINTER(I32)], I32),
         "ikv_compact_workspace_size": ([SP, CP, I32, ctypes.POINTER(SZ)], I32),
         "ikv_compact_kv": ([SP, CP, P, P, P, I32, P, SZ, P], I32),
         "ikv_append_token": ([SP, CP, P, P, P, I32, P, SZ, P], I32),
@@ -189,6 +190,13 @@ def ikv_value_norms(shape, cache, stream=None) -> None:
 def ikv_select_budget(rows, cap, util, length, rows_per_seq, budget, pos, keep, keep_len, stream=None) -> None:
     _check(_lib.ikv_select_budget(rows, cap, _p(util), _p(length), rows_per_seq, _p(budget), _p(pos), _p(keep),
                                   _p(keep_len), _stream(stream)), "ikv_select_budget")
+
+
+def ikv_select_plan(rows: int, max_len: int, sms: int = 0) -> dict:
+    """The launch of a selection of rows of up to max_len slots (see include/ikv.h)."""
+    v = [I32(0), I32(0)]
+    _check(_lib.ikv_select_plan(rows, max_len, sms, *[ctypes.byref(x) for x in v]), "ikv_select_plan")
+    return {"ctas": int(v[0].value), "threads": int(v[1].value)}
 
 
 def ikv_compact_workspace_size(shape, cache, mode) -> int:

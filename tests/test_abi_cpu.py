@@ -320,6 +320,24 @@ def test_attend_plan_properties(lib):
             assert r["n_chunks"] == 1, r
 
 
+def test_select_plan_query(lib):
+    """How many CTAs share a row of a selection follows the rows' length bound (not the slot
+    space's capacity) and keeps the launch to one CTA an SM (152 SMs)."""
+    def plan(rows, max_len):
+        return tuple(lib.ikv_select_plan(rows, max_len, 152)[k] for k in ("ctas", "threads"))
+    # a step's rows at their evicted length: one CTA, threads for a batch of keys each
+    assert plan(1, 52) == (1, 256) and plan(1, 2048) == (1, 256)
+    assert plan(1, 3278) == (1, 512) and plan(32, 4608) == (1, 512) and plan(1, 6143) == (1, 1024)
+    # long rows: clusters of CTAs with 3072 slots at least
+    assert plan(1, 6144) == (2, 512) and plan(1, 12288) == (4, 512) and plan(1, 24576) == (8, 512)
+    assert plan(32, 16385) == (4, 512) and plan(19, 70000) == (8, 512)
+    # more rows: a CTA an SM
+    assert plan(20, 70000) == (4, 512) and plan(76, 70000) == (2, 512) and plan(77, 70000) == (1, 1024)
+    assert lib.ikv_select_plan(0, 0, 1) == {"ctas": 1, "threads": 256}
+    with pytest.raises(lib.IKVError):
+        lib.ikv_select_plan(-1, 10, 152)
+
+
 def test_product_package_does_not_reference_the_oracle():
     """The CUDA path and its binding never import or link the CPU oracle."""
     pkg = os.path.join(ROOT, "paper_2609_03515_gb300")

@@ -27,22 +27,35 @@ def _want(util, pos, L, B):
 LENS = [0, 1, 2, 31, 33, 511, 512, 513, 1024, 1025, 4095, 4096, 4097, 8191, 8192, 8193, 16385]
 
 
-@pytest.mark.parametrize("rows,cap,lens", [
-    (17, 16448, LENS),             # clusters of eight, lengths that leave parts empty
-    (60, 3000, LENS[:10] + [3000]),  # clusters of two
-    (400, 1500, LENS[:10]),        # one CTA a row
-    (1, 70000, [70000]),           # one long row
-    (400, 70000, [60000, 33]),     # more keys than a CTA keeps in shared memory
+LONG = [24576, 24575, 12288, 3071, 6143, 6144, 6145, 9216, 18431, 21504, 1, 0]  # eight CTAs down to one
+
+
+@pytest.mark.parametrize("rows,cap,lens,ctas", [
+    (17, 16448, LENS, 4),
+    (19, 24576, LONG, 8),
+    (70, 6144, LENS[:13] + [6143, 6144], 2),
+    (60, 3000, LENS[:10] + [3000], 1),
+    (400, 1500, LENS[:10], 1),
+    (1, 70000, [70000], 8),            # one long row
+    (400, 70000, [60000, 33], 1),      # more keys than a CTA keeps in shared memory
+    (3, 400000, [400000, 70000], 8),   # the same in a cluster
 ])
 @pytest.mark.parametrize("dead", [False, True])
-def test_select_cluster_bit_exact(rows, cap, lens, dead):
+def test_select_cluster_bit_exact(rows, cap, lens, ctas, dead):
+    assert ikv.ikv_select_plan(rows, cap)["ctas"] == ctas
+    # clusters: every row once with each budget and kind of utility
+    for shift in range(1 if ctas == 1 else 28 if cap < 100000 else 7):
+        _bit_exact(rows, cap, lens, dead, shift)
+
+
+def _bit_exact(rows, cap, lens, dead, shift):
     assert max(lens) <= cap
-    gen = torch.Generator().manual_seed(rows + cap)
+    gen = torch.Generator().manual_seed(rows + cap + shift)
     ln = torch.tensor([lens[r % len(lens)] for r in range(rows)], dtype=torch.int32)
     kinds = ["spread", "ties", "special", "low"]
     util = torch.empty(rows, cap)
     for r in range(min(rows, 40)):
-        kind = kinds[(r // len(lens) + r) % 4]
+        kind = kinds[(r // len(lens) + r + shift) % 4]
         x = torch.randn(cap, generator=gen)
         if kind == "spread":
             x = torch.exp(4 * x - 9)
@@ -66,7 +79,7 @@ def test_select_cluster_bit_exact(rows, cap, lens, dead):
     # none, one, a tenth, all but two, all but one, all, more than there are
     pick = [lambda n: 0, lambda n: 1, lambda n: n // 10, lambda n: max(0, n - 2), lambda n: max(0, n - 1), lambda n: n,
             lambda n: n + 5]
-    budget = torch.tensor([pick[(3 * r + r // len(lens)) % 7](live[r]) for r in range(rows)], dtype=torch.int32)
+    budget = torch.tensor([pick[(3 * r + r // len(lens) + shift) % 7](live[r]) for r in range(rows)], dtype=torch.int32)
     keep = torch.full((rows, cap), -9, dtype=torch.int32, device="cuda")
     keep_len = torch.full((rows,), -9, dtype=torch.int32, device="cuda")
     ikv.ikv_select_budget(rows, cap, util.cuda(), ln.cuda(), 1, budget.cuda(), pos.cuda() if dead else None, keep,
