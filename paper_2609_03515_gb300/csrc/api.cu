@@ -253,10 +253,10 @@ bool attend_gsum(const ikv_shape *s, const ikv_cache *c, int32_t n_layers, int32
     return nc == 1;
 }
 
+// (the arrival counters in ws are zero, or `unmerged` is given and they are not used)
 ikv_status run_attend(const ikv_shape *s, const ikv_cache *c, int32_t layer0, int32_t n_layers, int32_t max_len,
-                      const void *q, void *out, void *ws, const AttendWs &w, bool logits, int32_t *split_out,
-                      int32_t *nsplit_out, cudaStream_t st, const ikv_timing *tm = nullptr,
-                      bool counters_zeroed = false, int32_t sc_layers = 0, int32_t sc_layer0 = 0,
+                      const void *q, void *out, void *ws, const AttendWs &w, bool logits, cudaStream_t st,
+                      const ikv_timing *tm = nullptr, int32_t sc_layers = 0, int32_t sc_layer0 = 0,
                       const NewRows *rows = nullptr, bool *gsum = nullptr, AttendArgs *unmerged = nullptr) {
     AttendArgs a{};
     a.k = c->k;
@@ -306,9 +306,6 @@ ikv_status run_attend(const ikv_shape *s, const ikv_cache *c, int32_t layer0, in
     // the last CTA of each unit of several splits merges them into out and lse2
     // (`unmerged`: the caller's next kernel does, from the arguments handed back in it)
     int32_t *arr = unmerged ? nullptr : at<int32_t>(ws, w.arrivals);
-    if (arr && a.n_splits > 1 && !counters_zeroed)
-        IKV_TRY_CUDA(cudaMemsetAsync(arr, 0, sizeof(int32_t) * (size_t)s->batch * n_layers * s->kv_heads, st),
-                     "cudaMemsetAsync");
     a.out = out;
     a.lse2 = at<float>(ws, w.lse2);
     a.arrivals = arr;
@@ -321,8 +318,6 @@ ikv_status run_attend(const ikv_shape *s, const ikv_cache *c, int32_t layer0, in
         IKV_TRY_CUDA(launch_attend(a, s->dtype, s->head_dim, group, st), "attend launch");
         if (tm && tm->attend_end) IKV_TRY_CUDA(cudaEventRecord(tm->attend_end, st), "cudaEventRecord");
     }
-    if (split_out) *split_out = a.split_tokens;
-    if (nsplit_out) *nsplit_out = a.n_splits;
     if (gsum) *gsum = a.gsum != 0;
     return IKV_OK;
 }
@@ -505,8 +500,8 @@ ikv_status ikv_decode_attend_score(const ikv_shape *shape, const ikv_cache *cach
     PdlScope pdl;
     AttendArgs at_args{};
     bool gsum = false;
-    if ((e = run_attend(shape, cache, layer, 1, cache->max_len, q, out, ws, w, want_score, nullptr, nullptr, stream,
-                        nullptr, false, 0, 0, nullptr, &gsum, &at_args)))
+    if ((e = run_attend(shape, cache, layer, 1, cache->max_len, q, out, ws, w, want_score, stream, nullptr, 0, 0,
+                        nullptr, &gsum, &at_args)))
         return e;
     const bool tc = use_tc(shape, cache, layer + 1, cache->max_len);
     ScoreOneArgs sa{};
@@ -961,8 +956,8 @@ ikv_status ikv_step(const ikv_shape *shape, const ikv_params *p, ikv_cache *cach
         PdlScope pdl;
         const NewRows rows{k_new, v_new, at<int32_t>(ws, w.slot), cache->vnorm};
         bool gsum = false;
-        if ((e = run_attend(shape, cache, 0, shape->layers, cx.L1, q, out, ws, w.at, cx.scoring, nullptr, nullptr,
-                            stream, nullptr, true, 0, 0, &rows, &gsum)))
+        if ((e = run_attend(shape, cache, 0, shape->layers, cx.L1, q, out, ws, w.at, cx.scoring, stream, nullptr, 0,
+                            0, &rows, &gsum)))
             return e;
         return layer_evict(shape, p, cache, ema, ws, cx, stream, gsum);
     }
@@ -999,8 +994,8 @@ ikv_status ikv_step(const ikv_shape *shape, const ikv_params *p, ikv_cache *cach
         rows.book.df = DeferArgs{p->max_holes, cx.cap, cache->start, 1};
     }
     bool gsum = false;  // the attention may hand over normalised group sums instead of logits
-    if ((e = run_attend(shape, cache, 0, shape->layers, cx.L1, q, out, ws, w.at, cx.scoring, nullptr, nullptr, stream,
-                        tm, true, 0, 0, &rows, &gsum)))
+    if ((e = run_attend(shape, cache, 0, shape->layers, cx.L1, q, out, ws, w.at, cx.scoring, stream, tm, 0, 0, &rows,
+                        &gsum)))
         return e;
     if (tm && (e = record(tm->combine_end, stream))) return e;
     if (!tm && !pdl) pdl.emplace();
@@ -1059,8 +1054,8 @@ ikv_status ikv_step_layer(const ikv_shape *shape, const ikv_params *p, ikv_cache
     // log-sum-exp land where the whole step's attention would put them, for
     // ikv_step_end's score pass
     bool gsum = false;  // the same for every layer call of the step (attend_gsum)
-    return run_attend(shape, cache, layer, 1, cx.L1, q, out, ws, cx.w.at, cx.scoring && eligible, nullptr, nullptr,
-                      stream, nullptr, true, shape->layers, layer, &rows, &gsum);
+    return run_attend(shape, cache, layer, 1, cx.L1, q, out, ws, cx.w.at, cx.scoring && eligible, stream, nullptr,
+                      shape->layers, layer, &rows, &gsum);
 }
 
 ikv_status ikv_step_end(const ikv_shape *shape, const ikv_params *p, ikv_cache *cache, float *ema, int32_t t,
