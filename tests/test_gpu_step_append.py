@@ -28,63 +28,60 @@ def test_step_appends(dtype, d, ps, gran):
     full = nb - 1
     c.start[full] = c.cap - LENS[full]  # no room for its new token
     c.ema.copy_(torch.rand(c.ema.shape, generator=gen, device="cuda"))
-    c.pos[torch.rand(c.pos.shape, generator=gen, device="cuda") < 0.15] = -1
-    for b, L in enumerate(LENS):  # a stale mark in the slot that the new token gets
-        if L < c.cap:
+    R = c.rows_per_seq
+    for b, L in enumerate(LENS):
+        for r in range(R):  # every row of a sequence has as many dead slots
+            c.pos[b * R + r, torch.randperm(L, generator=gen, device="cuda")[:round(0.15 * L)]] = -1
+        if L < c.cap:  # a stale mark in the slot that the new token gets
             c.pos.view(nb, -1, c.cap)[b, :, L] = -1
     q = torch.randn(layers, nb, G * kvh, d, generator=gen, device="cuda").to(dt)
     kn = torch.randn(layers, nb, kvh, d, generator=gen, device="cuda").to(dt)
     vn = torch.randn(layers, nb, kvh, d, generator=gen, device="cuda").to(dt)
     out = torch.full((layers, nb, G * kvh, d), 9.0, device="cuda").to(dt)
     ema0, pos0 = c.ema.clone(), c.pos.clone()
-    p = c.params(0.5, refresh_period=2, max_holes=8)
+    kv0 = [[[[c.gather(x, b, l, g, L) for g in range(kvh)] for l in range(layers)] for b, L in enumerate(LENS)]
+           for x in (c.k, c.v)]
+    c.vnorm.copy_(torch.rand(c.vnorm.shape, generator=gen, device="cuda"))
+    vnorm0 = c.vnorm.clone()
+    holes = 8
+    p = c.params(0.5, refresh_period=2, max_holes=holes)
     cch = c.cache(max(LENS), dead_slots=True)
     n = ikv.ikv_step_workspace_size(c.shape(), cch)
     ws = torch.full((n,), 0xAB, dtype=torch.uint8, device="cuda")
     ikv.ikv_step(c.shape(), p, cch, c.ema, 2, q, kn, vn, out, ws, n)  # t = 2: the mean initialisation
     torch.cuda.synchronize()
     assert ikv.ikv_device_status() == 4
-    R = c.rows_per_seq
     for b, L in enumerate(LENS):
-        new = b != full
+        new = int(b != full)
+        dead = round(0.15 * L)
         assert int(c.next_pos[b]) == L + new
-        # lengths: a sequence compacts only past max_holes dead slots, its order kept
-        dead = [int((pos0[b * R + r, :L] < 0).sum()) for r in range(R)]
-        if R > 1:  # rows of one sequence with different numbers of dead slots are no state of the library
-            live = [pos0[b * R + r, :L] >= 0 for r in range(R)]
-        else:
-            live = [pos0[b, :L] >= 0]
-        for l in range(layers):
-            for g in range(kvh):
-                rr = 0 if R == 1 else g
-                lv = torch.cat([live[rr], torch.ones(int(new), dtype=torch.bool, device="cuda")])
-                if not bool(lv.any()):
-                    continue
-                if dead[0] <= 8 or not new:
-                    K, V = c.gather(c.k, b, l, g, L).double(), c.gather(c.v, b, l, g, L).double()
-                    if new:
-                        if int(c.len[b]) == L + 1:
-                            got_k, got_v = c.gather(c.k, b, l, g, L + 1)[L], c.gather(c.v, b, l, g, L + 1)[L]
-                            assert torch.equal(got_k, kn[l, b, g]) and torch.equal(got_v, vn[l, b, g])
-                            vnorm = float(vn[l, b, g].double().norm())
-                            assert abs(float(c.vnorm[l, b, g, L]) - vnorm) < 1e-5 * max(1.0, vnorm)
-                        else:
-                            continue
-                        K = torch.cat([K, kn[l, b, g].double()[None]])
-                        V = torch.cat([V, vn[l, b, g].double()[None]])
-                    elif int(c.len[b]) != L:
-                        continue
-                    z = q[l, b, g * G:(g + 1) * G].double() @ K.T / math.sqrt(d)
+        # a sequence compacts only past max_holes dead slots, its order kept
+        compacted = dead > holes
+        n1 = L + new - (dead if compacted else 0)
+        assert int(c.len[b]) == n1, L
+        for r in range(R):
+            row = b * R + r
+            live = pos0[row, :L] >= 0
+            mean = float(ema0[row, :L][live].double().mean()) if bool(live.any()) else 0.0
+            pos = torch.cat([pos0[row, :L], torch.full((new,), L, dtype=torch.int32, device="cuda")])
+            ema = torch.cat([ema0[row, :L], torch.full((new,), mean, device="cuda")])
+            lv = pos >= 0
+            stay = lv if compacted else torch.ones_like(lv)
+            assert torch.equal(c.pos[row, :n1], pos[stay]), (L, r)
+            err = (c.ema[row, :n1] - ema[stay]).abs()
+            assert float(err.max()) < 1e-5 if n1 else True
+            for l in range(layers):
+                for g in range(kvh) if R == 1 else [r]:
+                    K, V = [torch.cat([x[b][l][g], y[l, b, g][None]][:1 + new]) for x, y in ((kv0[0], kn), (kv0[1], vn))]
+                    assert torch.equal(c.gather(c.k, b, l, g, n1), K[stay]), (L, l, g)
+                    assert torch.equal(c.gather(c.v, b, l, g, n1), V[stay]), (L, l, g)
+                    norm = torch.cat([vnorm0[l, b, g, :L], vn[l, b, g].double().norm().float()[None]][:1 + new])
+                    assert torch.allclose(c.vnorm[l, b, g, :n1], norm[stay], rtol=1e-5, atol=0), (L, l, g)
+                    z = q[l, b, g * G:(g + 1) * G].double() @ K.double().T / math.sqrt(d)
                     z[:, ~lv] = -math.inf
-                    want = torch.softmax(z, -1) @ V
+                    want = torch.softmax(z, -1) @ V.double() if bool(lv.any()) else torch.zeros(G, d, device="cuda")
                     err = (out[l, b, g * G:(g + 1) * G].double() - want).abs().max()
                     assert err < (2e-2 if dtype == ikv.IKV_BF16 else 1e-4), (L, l, g, float(err))
-        if new and int(c.len[b]) == L + 1:
-            for r in range(R):
-                row = b * R + r
-                assert int(c.pos[row, L]) == L
-                mean = ema0[row, :L][live[r]].double().mean() if bool(live[r].any()) else torch.tensor(0.0)
-                assert abs(float(c.ema[row, L]) - float(mean)) < 1e-5
 
 
 # launches: attention and compaction, and a selection of its own where the bookkeeping CTAs would
