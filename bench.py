@@ -86,7 +86,7 @@ def rank_seed(base_seed: int, rank: int) -> int:
 
 
 # revision of each attention kernel; a committed ncu summary counts only for its own revision
-ATTEND_KERNEL_REV = {"attend_tc_kernel": "attend_tc_v14", "attend_bf16_kernel": "attend_bf16_v1", "attend_f32_kernel": "attend_f32_v1"}
+ATTEND_KERNEL_REV = {"attend_tc_kernel": "attend_tc_v15", "attend_bf16_kernel": "attend_bf16_v1", "attend_f32_kernel": "attend_f32_v1"}
 
 
 def schedule_name(w) -> str:

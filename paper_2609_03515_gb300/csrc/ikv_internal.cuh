@@ -14,7 +14,12 @@ constexpr int kAttendThreads = 128;
 constexpr int kMaxSplits = 128;    // split-K partitions per (seq, layer, kv head)
 constexpr int kSplitMergeTokens = 64;  // cost of merging a unit's splits, as tokens of its stream
 constexpr int kMaxLayersPerScorePass = 32;
-constexpr int kFusedSelectMaxLen = 12288;  // longest row bound for which the score pass also selects
+// Longest row bound for which the score pass also selects, its keys (48 KB) within what four CTAs
+// an SM leave.  At 16384 a steady step gains little of the launch it saves and a first step, which
+// selects in earnest, loses: us with a kernel of its own / in the pass, one sequence, 32 layers:
+// 12.4k slots 275.5 / 274.5, 16k 348.0 / 347.6 (4 layers 55.0 / 53.7), first steps of 13k
+// 314 / 369, of 16k 401 / 470, eight of 14k 2700 / 2778.
+constexpr int kFusedSelectMaxLen = 12288;
 constexpr int kScoreLayersPerGroup = 8;   // eligible layers one score CTA folds (one warp each)
 constexpr int kMaxLayers = 512;
 
