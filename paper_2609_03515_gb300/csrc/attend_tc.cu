@@ -190,6 +190,10 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
         : "memory");
 }
 
+__device__ __forceinline__ void bulk_prefetch_l2(const void *p, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+
 // smem matrix descriptor, 128-byte swizzle (sm_100 family, version 1)
 __device__ __forceinline__ uint64_t sdesc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
     uint64_t d = (uint64_t)((saddr >> 4) & 0x3FFFu);
@@ -379,10 +383,13 @@ __global__ void __launch_bounds__(kThreads, 2)
     // Prologue.  The producer lane initialises the barriers and starts the K/V stream at
     // once (every load up to the ring's depth); the TMEM allocation and P zeroing below
     // overlap the loads' latency.  An early CTA does all of this before the dependency
-    // wait, so it overlaps the previous kernel's tail.  (It asks for no more than the ring
-    // holds: L2 prefetches of its other tiles cost more than they saved.  Steps of 32 layers
-    // driven one by one, us with / without them: 8 units of 27 tiles a layer 265 / 249, 8 of
-    // 103 456 / 426, 16 of 103 in 16-token pages 966 / 800; 16 layers, 128 of 27 771 / 645.)
+    // wait, so it overlaps the previous kernel's tail, and pulls its q rows into L2 (that cannot
+    // return stale data: L2 is where writes land).  32 layers driven one by one, us a step without
+    // / with the q rows: 8 units of 27 tiles a layer 245 / 245, of 104 430 / 418, of 128 490 / 479; 16
+    // layers of 32 units of 27 224 / 218.  (It asks for no more K and V than the ring holds: L2
+    // prefetches of its other tiles cost more than they saved, us with / without them: 8 units of
+    // 27 tiles 265 / 249, 8 of 103 456 / 426, 16 of 103 in 16-token pages 966 / 800; 16 layers, 128
+    // of 27 771 / 645, but 32 of 27 214 / 218 and 28 of 33 212 / 220.)
     if (warp == 4) {
         if (lane == 0) {
             for (int i = 0; i < kNst; ++i) {
@@ -404,6 +411,8 @@ __global__ void __launch_bounds__(kThreads, 2)
         }
         __syncwarp();
         while (ld_J < kNst && ld_p < np) issue_next();
+        if (early && lane == 0)
+            bulk_prefetch_l2(a.q + (((int64_t)li * a.batch + b) * a.q_heads + (int64_t)g * G) * kD, G * kD * 2);
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
