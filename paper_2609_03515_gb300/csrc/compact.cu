@@ -200,13 +200,17 @@ __device__ __forceinline__ void compact_stable_item(const CompactArgs &a, const 
             // for.  (Every thread finding its own rows, keep list then table then copy in turn:
             // 237 us for the first compaction of 32 layers x 8 KV heads to 3277 of 32769 slots,
             // 860 MB of reads and writes; this way 168 us, 0.75 of the copy rate.)
-            auto kept_slot = [&](int tile) {
-                const int j = tile_base(tile) + tid;
-                return tid < kCompRows && tile < n_tiles && j >= j0 && j < j1 ? kp[j] : -1;
-            };
+            // (rows outside the range look up its first or last row: with a branch around each load
+            // the five tiles of the start went out one load after the other)
+            auto row_of = [&](int tile) { return min(max(tile_base(tile) + tid, j0), j1 - 1); };
+            auto kept_slot = [&](int tile) { return kp[row_of(tile)]; };
             auto find = [&](int tile, int slot, uint32_t &src, uint32_t &dst) {
-                src = slot < 0 ? ~0u : (uint32_t)a.pv.row_phys(b, l, g, S + slot);
-                dst = slot < 0 ? ~0u : (uint32_t)a.pv.row_phys(b, l, g, new_start + tile_base(tile) + tid);
+                const int j = tile_base(tile) + tid;
+                const bool in = tile < n_tiles && j >= j0 && j < j1;
+                const uint32_t s = (uint32_t)a.pv.row_phys(b, l, g, S + slot);
+                const uint32_t d = (uint32_t)a.pv.row_phys(b, l, g, new_start + row_of(tile));
+                src = in ? s : ~0u;
+                dst = in ? d : ~0u;
             };
             auto put_rows = [&](int tile, uint32_t src, uint32_t dst) {
                 rows_s[tile % kCompRowSets][0][tid] = src;
@@ -214,17 +218,19 @@ __device__ __forceinline__ void compact_stable_item(const CompactArgs &a, const 
             };
             constexpr int kAhead = kCompStages - 1;  // tiles whose copies are in flight
             uint32_t src_next = ~0u, dst_next = ~0u;  // rows of tile `tile` + kAhead
-            int slot_next = -1;                       // kept slots of the one after it
+            int slot_next = 0;                        // kept slots of the one after it
             if (tid < kCompRows) {
                 int slot[kAhead + 1];
+                uint32_t src[kAhead + 1], dst[kAhead + 1];
 #pragma unroll
                 for (int i = 0; i <= kAhead; ++i) slot[i] = kept_slot(i);
                 slot_next = kept_slot(kAhead + 1);
 #pragma unroll
-                for (int i = 0; i <= kAhead; ++i) {
-                    find(i, slot[i], src_next, dst_next);
-                    if (i < kAhead) put_rows(i, src_next, dst_next);
-                }
+                for (int i = 0; i <= kAhead; ++i) find(i, slot[i], src[i], dst[i]);
+#pragma unroll
+                for (int i = 0; i < kAhead; ++i) put_rows(i, src[i], dst[i]);
+                src_next = src[kAhead];
+                dst_next = dst[kAhead];
             }
             __syncthreads();
             auto issue = [&](int tile) {
@@ -245,11 +251,11 @@ __device__ __forceinline__ void compact_stable_item(const CompactArgs &a, const 
                 cp_async_commit();
             }
             for (int tile = 0; tile < n_tiles; ++tile) {
-                if (tid < kCompRows) put_rows(tile + kAhead, src_next, dst_next);
+                if (tid < kCompRows && tile + kAhead < n_tiles) put_rows(tile + kAhead, src_next, dst_next);
                 __syncthreads();  // the stage about to be refilled was written out last iteration
                 if (tile + kAhead < n_tiles) issue(tile + kAhead);
                 cp_async_commit();
-                if (tid < kCompRows) {
+                if (tid < kCompRows && tile + kAhead + 1 < n_tiles) {  // (past the end nothing is waited for)
                     find(tile + kAhead + 1, slot_next, src_next, dst_next);
                     slot_next = kept_slot(tile + kAhead + 2);
                 }
