@@ -22,6 +22,8 @@
 // Hole-fill mode: survivors at slots >= n move into the evicted slots below n
 // (k-th hole <- k-th such survivor).  Sources and destinations are disjoint,
 // so every move is independent; the move list is built per row first.
+#include <atomic>
+
 #include "ikv_internal.cuh"
 
 namespace ikv {
@@ -573,33 +575,39 @@ __global__ void __launch_bounds__(kCompThreads) append_kernel(const AppendArgs a
     }
 }
 
+constexpr int kCompSmemMax = kCompStages * 2 * kCompRows * 128 * 4;  // rows of 128 fp32
+// (the limit is the process's: every call writes the same value)
+cudaError_t comp_smem_limit(void (*kernel)(CompactArgs)) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kCompSmemMax);
+}
+
 }  // namespace
 
 cudaError_t launch_compact(const CompactArgs &a, int mode, int sms, cudaStream_t st) {
     dim3 grid(a.layers * a.pv.kv_heads + a.rows_per_seq, a.batch);
     if (mode == IKV_COMPACT_STABLE || mode == IKV_COMPACT_STABLE_SHORT) {
         const int smem = kCompStages * 2 * kCompRows * a.pv.head_dim * a.elem_bytes;
-        static int attr_smem = 0;  // raise the dynamic shared-memory limits once per size
-        static int per_sm = 0;     // resident CTAs per SM of the strided kernel at attr_smem
-        if (smem > attr_smem || per_sm == 0) {
-            cudaError_t e =
-                cudaFuncSetAttribute(compact_stable_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(compact_stable_strided_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         smem);
+        // resident CTAs per SM of the strided kernel at this row size (32, 64 or 128 KB a CTA)
+        static std::atomic<int> resident[3];
+        static_assert((kCompSmemMax >> 16) == 2, "three sizes");
+        int per_sm = resident[smem >> 16].load(std::memory_order_relaxed);
+        cudaError_t e = cudaSuccess;
+        if (per_sm == 0) {
+            e = comp_smem_limit(compact_stable_strided_kernel);
             if (e == cudaSuccess)
                 e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, compact_stable_strided_kernel,
                                                                   kCompThreads, smem);
             if (e != cudaSuccess) return e;
             if (per_sm < 1) per_sm = 1;
-            attr_smem = smem;
+            resident[smem >> 16].store(per_sm, std::memory_order_relaxed);
         }
         const int64_t items = (int64_t)grid.x * grid.y;
         const int64_t wave = (int64_t)per_sm * (sms > 0 ? sms : 1);
-        cudaError_t e = items <= wave
-                            ? launch_k(compact_stable_kernel, grid, dim3(kCompThreads), smem, st, a)
-                            : launch_k(compact_stable_strided_kernel, dim3((unsigned)wave), dim3(kCompThreads), smem,
-                                       st, a);
+        auto kernel = items <= wave ? compact_stable_kernel : compact_stable_strided_kernel;
+        if (items > wave) grid = dim3((unsigned)wave);
+        e = comp_smem_limit(kernel);
+        if (e != cudaSuccess) return e;
+        e = launch_k(kernel, grid, dim3(kCompThreads), smem, st, a);
         note_launch();
         return e != cudaSuccess ? e : cudaGetLastError();
     }
